@@ -984,20 +984,22 @@ __global__ void __launch_bounds__(256) k_pair_geo(DevPot P, DevGrid g0, PassArgs
   const R s_i = sqrt6<R>() * si.sig, s_j = sqrt6<R>() * sj.sig;
   const R D2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
   int bad = D2 < (R)(kRMin * kRMin);
-  // component c of the record, at both entries of the pair (plane A below
-  // L.ca, plane B above)
+  // component c of the record, at both entries of the pair: the densities (c
+  // below 2 n_f) in plane A, the pair terms in plane B when the record is
+  // split, else after the densities
   typename GeoRec<R>::T* oa = buf + pr_.tp * (int64_t)L.ca;
   typename GeoRec<R>::T* oa2 = buf + pr_.tr * (int64_t)L.ca;
-  typename GeoRec<R>::T* ob = buf + L.b_off + pr_.tp * (int64_t)L.cb;
-  typename GeoRec<R>::T* ob2 = buf + L.b_off + pr_.tr * (int64_t)L.cb;
+  const int c_b = 2 * P.n_f;
+  typename GeoRec<R>::T* ob = L.cb ? buf + L.b_off + pr_.tp * (int64_t)L.cb : oa + c_b;
+  typename GeoRec<R>::T* ob2 = L.cb ? buf + L.b_off + pr_.tr * (int64_t)L.cb : oa2 + c_b;
   auto put = [&](int c, R v) {
     const typename GeoRec<R>::T w = GeoRec<R>::put(v);
-    if (c < L.ca) {
+    if (c < c_b) {
       oa[c] = w;
       oa2[c] = w;
     } else {
-      ob[c - L.ca] = w;
-      ob2[c - L.ca] = w;
+      ob[c - c_b] = w;
+      ob2[c - c_b] = w;
     }
   };
   if constexpr (PW != 0) {
