@@ -324,8 +324,10 @@ MXE_API mxe_status mxe_set_pass_shape(mxe_ctx *ctx, int32_t lanes, int32_t threa
 MXE_API mxe_status mxe_set_pair_block(mxe_ctx *ctx, int32_t pair_threads);
 MXE_API mxe_status mxe_get_pass_shape(mxe_ctx *ctx, int32_t *lanes, int32_t *threads, int32_t *pair_threads);
 
-/* Forms of the pair kernels this context's potential takes (host values,
- * either pointer may be NULL):
+/* Forms of the direct pair kernels for this context's potential (host values,
+ * either pointer may be NULL); exponential potentials with moderate decay
+ * rates and cut-offs are tabulated in r^2 instead in the accurate pass and in
+ * the FP64 relaxation passes, whatever their form:
  *  table_pattern 1: two species, two like pair terms and a cross term, a
  *    density that depends on the neighbour's species only (the species tables
  *    are compile-time constants in the pair kernels); 0: general tables.

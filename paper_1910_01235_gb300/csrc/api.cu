@@ -46,6 +46,10 @@ struct mxe_ctx {
   mxe_potential pot{};
   DevPot dp{};
   DevPot dp_pair{};  // the potential with every embedding switched off (pair terms alone)
+  // tabulated radial terms (radial_table.cuh; rows null: direct kernels): the
+  // accurate pass, and in FP64 contexts the relaxation's densities and forces
+  uint4* tab_rows = nullptr;
+  RadialTab tab_geo{}, tab_dens{}, tab_force{};
   // embedding average: 0 the Taylor form (Eq. F_taylor_mxe), 1 the exact rule
   int embedding = 0;
   double* emb_buf = nullptr;  // rule data of the exact average: (9 S) [n] doubles
@@ -749,6 +753,15 @@ mxe_status enqueue_emb_exact(mxe_ctx* c, const PassArgs& A, bool fp64) {
   return MXE_OK;
 }
 
+// One relaxation pass over the unordered pairs: tabulated in FP64 contexts
+// whose potential has tables, else direct.
+cudaError_t relax_pair_pass(mxe_ctx* c, bool force, const DevPot& PP, const PassArgs& A, void* dens, void* frc) {
+  if (c->precision == MXE_FP64 && c->tab_rows)
+    return launch_relax_tab(force, PP, c->grid, A, force ? c->tab_force : c->tab_dens, c->pair_rec, c->n_upairs,
+                            force ? frc : dens, c->stream);
+  return launch_relax_pair(c->precision, force, PP, c->grid, A, c->pair_rec, c->n_upairs, dens, frc, c->stream);
+}
+
 // Class names of the half-list kernels in the event timing.
 const char* relax_pair_name(bool force, int prec) {
   if (prec == MXE_FP64) return force ? "pair64_force" : "pair64_density";
@@ -811,7 +824,10 @@ mxe_status enqueue_passes(mxe_ctx* c, const mxe_state* s, PassArgs& A, bool want
       G.ab32lo = nullptr;
     }
     CK(TIMED(prec == MXE_FP64 ? "pair_geo64" : "pair_ff",
-             launch_pair_geo(prec, PP, c->grid, G, c->pair_rec, c->n_upairs, c->pair_buf, c->pair_cap, st)));
+             c->tab_rows ? launch_geo_tab(prec, PP, c->grid, G, c->tab_geo, c->pair_rec, c->n_upairs, c->pair_buf,
+                                          c->pair_cap, st)
+                         : launch_pair_geo(prec, PP, c->grid, G, c->pair_rec, c->n_upairs, c->pair_buf, c->pair_cap,
+                                           st)));
     CK(TIMED(accurate_gather_name(false, prec),
              launch_pair_gather(prec, false, c->nl, PP, G, c->pair_buf, c->pair_cap, st)));
     CK(TIMED(accurate_gather_name(true, prec),
@@ -822,8 +838,7 @@ mxe_status enqueue_passes(mxe_ctx* c, const mxe_state* s, PassArgs& A, bool want
     F.site_E = nullptr;  // energies already come from the accurate pass
     if (half_list_forces(c)) {
       // the relaxation's force pass: each unordered pair once, then the gather
-      CK(TIMED(relax_pair_name(true, prec), launch_relax_pair(prec, true, PP, c->grid, F, c->pair_rec,
-                                                               c->n_upairs, c->ent_dens, c->ent_frc, st)));
+      CK(TIMED(relax_pair_name(true, prec), relax_pair_pass(c, true, PP, F, c->ent_dens, c->ent_frc)));
       CK(TIMED(relax_gather_name(true, prec),
                launch_relax_gather(prec, true, c->nl, PP, F, c->ent_dens, c->ent_frc, st)));
     } else {
@@ -833,6 +848,30 @@ mxe_status enqueue_passes(mxe_ctx* c, const mxe_state* s, PassArgs& A, bool want
   }
   // the accurate pass: the exact average in FP64
   return c->embedding ? enqueue_emb_exact(c, A, true) : MXE_OK;
+}
+
+// The radial tables of a context with a pair index: planned on the host and
+// filled on the stream.  Potentials outside the plan's limits keep the direct
+// kernels (tab_rows stays null).
+cudaError_t build_radial_tabs(mxe_ctx* c) {
+  if (!has_pair_index(c)) return cudaSuccess;
+  const bool fp64 = c->precision == MXE_FP64;
+  const int kinds[3] = {fp64 ? kTabValue64 : kTabValueFF, kTabValue64, kTabDeriv64};
+  RadialTab* tabs[3] = {&c->tab_geo, &c->tab_dens, &c->tab_force};
+  const int m = fp64 ? 3 : 1;
+  int64_t words = 0;
+  for (int t = 0; t < m; ++t) {
+    if (!plan_radial_tab(c->dp, kinds[t], t != 1, *tabs[t])) return cudaSuccess;
+    words += (int64_t)tabs[t]->nrow * tabs[t]->stride;
+  }
+  cudaError_t e = dalloc(&c->tab_rows, words);
+  if (e != cudaSuccess) return e;
+  const uint4* at = c->tab_rows;
+  for (int t = 0; t < m; ++t) {
+    tabs[t]->rows = at;
+    at += (int64_t)tabs[t]->nrow * tabs[t]->stride;
+  }
+  return launch_radial_tables(c->dp, kinds, tabs, m, c->stream);
 }
 
 mxe_fire_params fire_params_or_default(const mxe_fire_params* fire) {
@@ -892,12 +931,10 @@ mxe_status enqueue_force_passes(mxe_ctx* c, const PassArgs& A) {
   if (half_list_forces(c)) {
     // each unordered pair once: pair kernel, then the per-site gather
     const int prec = c->precision;
-    CK(TIMED(relax_pair_name(false, prec), launch_relax_pair(prec, false, PP, c->grid, A, c->pair_rec,
-                                                              c->n_upairs, c->ent_dens, c->ent_frc, st)));
+    CK(TIMED(relax_pair_name(false, prec), relax_pair_pass(c, false, PP, A, c->ent_dens, c->ent_frc)));
     CK(TIMED(relax_gather_name(false, prec),
              launch_relax_gather(prec, false, c->nl, PP, A, c->ent_dens, c->ent_frc, st)));
-    CK(TIMED(relax_pair_name(true, prec), launch_relax_pair(prec, true, PP, c->grid, A, c->pair_rec,
-                                                             c->n_upairs, c->ent_dens, c->ent_frc, st)));
+    CK(TIMED(relax_pair_name(true, prec), relax_pair_pass(c, true, PP, A, c->ent_dens, c->ent_frc)));
     CK(TIMED(relax_gather_name(true, prec),
              launch_relax_gather(prec, true, c->nl, PP, A, c->ent_dens, c->ent_frc, st)));
   } else {
@@ -1434,6 +1471,7 @@ mxe_status mxe_create_batch(mxe_ctx** out, int32_t n_systems, const mxe_box* box
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(c->flags, 0, sizeof(int), c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->ctrl, 0, sizeof(Ctrl), c->stream);
+  if (e == cudaSuccess) e = build_radial_tabs(c);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) {
     mxe_destroy(c);
@@ -1455,6 +1493,7 @@ mxe_status mxe_destroy(mxe_ctx* c) {
   if (c->step_exec) cudaGraphExecDestroy(c->step_exec);
   dfree(c->loop_dev);
   if (c->loop_h) cudaFreeHost(c->loop_h);
+  dfree(c->tab_rows);
   dfree(c->tan_buf);
   dfree(c->emb_buf);
   dfree(c->emb_nrule);

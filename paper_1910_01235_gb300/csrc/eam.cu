@@ -31,6 +31,7 @@
 
 #include "ff.cuh"
 #include "mxe_internal.cuh"
+#include "pair_common.cuh"
 
 namespace mxe {
 
@@ -321,37 +322,6 @@ __device__ __forceinline__ void load_ab(const PassArgs& A, int64_t j, float a[S]
       b[3 < S ? 3 : 0] = v1.w;
     }
   }
-}
-
-__device__ __forceinline__ bool skin_violated(const Ctrl* c) {
-  double disp = sqrt(__longlong_as_double((long long)c->disp2_bits));
-  double smax = __longlong_as_double((long long)c->smax_bits);
-  return 2.0 * disp + kSqrt6 * (smax - c->sigma_max_build) > c->skin;
-}
-
-// Uniform early exit of the relaxation chunk.  Returns true if the kernel must
-// stop.  The skin test runs once per launch, on thread 0 of block 0 (on the
-// 1:64 FP64 pipe a test per block kept the FP64 pipe a quarter busy and held
-// every block at the barrier behind it); each block reads the halt flag
-// through one thread.  Blocks that start before block 0 sets the flag run the
-// pass on the old lists (valid arrays, so every access stays in bounds); a
-// halted pass is always evaluated again after the rebuild, so that output is
-// never used.  Every thread of the block must call this before any early
-// return.
-__device__ __forceinline__ bool chunk_halted(const PassArgs& A) {
-  if (A.ctrl == nullptr) return false;
-  __shared__ int halt;
-  if (threadIdx.x == 0) {
-    int h = A.ctrl->halted ? 1 : 0;
-    if (!h && blockIdx.x == 0 && A.check_skin && skin_violated(A.ctrl)) {
-      A.ctrl->reason = kReasonRebuild;
-      A.ctrl->halted = 1;
-      h = 1;
-    }
-    halt = h;
-  }
-  __syncthreads();
-  return halt != 0;
 }
 
 // ---------------------------------------------------------------- K2: density pass
@@ -854,34 +824,6 @@ __global__ void __launch_bounds__(256, MXE_GRADIENT_MIN_BLOCKS) k_gradient(DevPo
 // in row order and finish exactly as the density and chemical-potential
 // passes do.  Node arithmetic R: float-float (records of
 // float pairs; the FP32 modes) or FP64 (records of doubles).
-// The record of unordered pair p: owner site i, the entry of j in row i (j with
-// its image code), that entry's index tp and the index tr of the reverse
-// entry (i in row j).  The records are built from the current lists, so they
-// are consistent with them by construction; every index is still bounded
-// (a bad record sets the overflow flag and the pair is skipped).  Building
-// with MXE_DEBUG_CHECKS also checks that tp and tr lie in their rows.
-struct PairRef {
-  int64_t i, j;
-  uint32_t code;
-  int tp, tr;
-};
-__device__ __forceinline__ bool load_pair(const PassArgs& A, const int4* __restrict__ rec, int64_t p, PairRef& r) {
-  const int4 v = __ldg(&rec[p]);
-  r.i = v.x;
-  r.j = (uint32_t)v.y & kIdxMask;
-  r.code = (uint32_t)v.y >> kCodeShift;
-  r.tp = v.z;
-  r.tr = v.w;
-  bool ok = (uint64_t)(uint32_t)v.x < (uint64_t)A.n && (uint64_t)r.j < (uint64_t)A.n &&
-            (uint64_t)(uint32_t)v.z < (uint64_t)A.n_ent && (uint64_t)(uint32_t)v.w < (uint64_t)A.n_ent;
-#ifdef MXE_DEBUG_CHECKS
-  ok = ok && r.tp >= A.nb_off[r.i] && r.tp < A.nb_off[r.i + 1] && A.nb_ent[r.tp] == (uint32_t)v.y &&
-       r.tr >= A.nb_off[r.j] && r.tr < A.nb_off[r.j + 1] && (A.nb_ent[r.tr] & kIdxMask) == (uint32_t)r.i;
-#endif
-  if (!ok) atomicOr(A.flags, kFlagOverflow);
-  return ok;
-}
-
 template <typename R>
 struct GeoRec;
 template <>
@@ -1403,10 +1345,6 @@ __global__ void __launch_bounds__(256) k_pair_mu(DevPot P, PassArgs A,
 //    derivatives of both sites (over the nodes that move i and those that
 //    move j), written to the two entries of the pair;
 //  k_gather_rforce: per site the sums over its row, then the thermal term.
-struct alignas(32) Dbl4 {
-  double x, y, z, w;
-};
-
 template <typename R>
 struct Rec4;
 template <>

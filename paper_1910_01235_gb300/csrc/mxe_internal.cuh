@@ -96,6 +96,21 @@ struct Tables<1> {
 template <>
 struct Tables<2> : Tables<1> {};
 
+// The radial terms as piecewise polynomials in r^2 (radial_table.cuh): rows of
+// `stride` 16-byte words, one row per interval of width h (and per side of a
+// breakpoint), `words` words per term, density terms first.
+constexpr int64_t kTabMaxBytes = 200 * 1024;  // staged in one block's shared memory
+enum { kTabValue64 = 0, kTabDeriv64 = 1, kTabValueFF = 2 };
+struct RadialTab {
+  const uint4* rows;
+  int nrow, stride, words;
+  int nf_slots, np_slots;  // terms of a row: density, then pair terms (absent ones are zero)
+  int shift, k_lo;         // interval of w: (high word of w >> shift) - k_lo
+  unsigned rs_hi, rc_hi;   // r_switch^2, r_cut^2 as high words
+  double h;
+  double scale[5];         // value of one unit of the integer constant term
+};
+
 // Box / cell grid for positions and image codes.
 struct DevGrid {
   double L[3], invL[3], h[3];
@@ -311,6 +326,18 @@ struct GeoLayout {
 int pair_record_len(const DevPot& P);
 GeoLayout geo_layout(const DevPot& P, int64_t cap);
 int pair_threads(const PassArgs& A);
+// radial tables (radial_table.cu): the host-side plan of one table (false: the
+// potential keeps the direct kernels; with_pairs = false: density terms only)
+// and the kernel that fills the rows (nrow x stride words) of up to three
+bool plan_radial_tab(const DevPot& P, int kind, bool with_pairs, RadialTab& Tb);
+cudaError_t launch_radial_tables(const DevPot& P, const int* kinds, const RadialTab* const* tabs, int count,
+                                 cudaStream_t s);
+// tabulated passes (pair_table.cu): the geometry records of every precision,
+// and the relaxation passes of FP64 contexts
+cudaError_t launch_geo_tab(int precision, const DevPot& P, const DevGrid& g, const PassArgs& A, const RadialTab& Tb,
+                           const int4* pair_rec, int64_t npair, void* buf, int64_t cap, cudaStream_t s);
+cudaError_t launch_relax_tab(bool force, const DevPot& P, const DevGrid& g, const PassArgs& A, const RadialTab& Tb,
+                             const int4* pair_rec, int64_t npair, void* out, cudaStream_t s);
 cudaError_t launch_pair_geo(int precision, const DevPot& P, const DevGrid& g, const PassArgs& A,
                             const int4* pair_rec, int64_t npair, void* buf, int64_t cap, cudaStream_t s);
 cudaError_t launch_pair_gather(int precision, bool mu, int nl, const DevPot& P, const PassArgs& A, const void* buf,

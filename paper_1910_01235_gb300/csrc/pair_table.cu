@@ -1,0 +1,599 @@
+// pair_table.cu -- the passes over unordered pairs with tabulated radial terms
+// (radial_table.cuh): the geometry records of the accurate pass (every
+// precision) and the relaxation's density and force passes of FP64 contexts.
+//
+// What bounds them: the direct FP64 kernels sit on the FP64 pipe (2 lanes per
+// SM), the direct float-float kernel on instruction issue (two exponentials, a
+// square root and a switch in float-float per node).  Here a node costs a
+// 64-bit integer addition, a table row from shared memory (two or three
+// 16-byte loads per term) and 20 to 36 FP32 operations per term.
+//
+// Measured (event time per launch, direct -> tabulated).  FP64, 19,652-site
+// binary alloy (531 k pairs): forces 1127 -> 210 us, densities 709 -> 80 us,
+// geometry 911 -> 154 us.  Float-float geometry: 6.9 M pairs of the binary
+// alloy (which had the power form) 1.35 -> 1.22 ms, 23.3 M pairs of one species
+// 3.54 -> 1.92 ms, 241 M pairs of the interstitial slab 52.6 -> 26.6 ms.  What
+// bounds them now (ncu): the geometry kernels the shared-memory wavefronts
+// (84-89 %; 32 lanes reading random rows take about 12 wavefronts per 16-byte
+// load, 4 without bank conflicts), the force kernel the FP64 pipe (84 %), the
+// density kernel both (65 % each).
+//
+// Layout: one block per SM holds the whole table in shared memory (up to
+// 200 KB) and strides over the pairs; the table is copied before the kernel
+// waits for the previous one.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "pair_common.cuh"
+#include "radial_table.cuh"
+
+namespace mxe {
+namespace {
+
+// ---------------------------------------------------------------- geometry of a pair
+struct PairGeom {
+  double d[3], D2, s_i, s_j;
+};
+// minimum image of q_j - q_i; the division by the box only where a component
+// reaches half the box (pairs of the list are nearer than that elsewhere)
+__device__ __forceinline__ void pair_geometry(const DevGrid& g0, const PassArgs& A, int64_t i, int64_t j, PairGeom& G) {
+  const int64_t n = A.n;
+  const DevGrid* gp = A.batch.nsys ? &A.batch.grids[A.batch.sys_of[i]] : nullptr;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    double da = __ldg(&A.q[a * n + j]) - __ldg(&A.q[a * n + i]);
+    const double L = gp ? gp->L[a] : g0.L[a];
+    // high words of positive doubles order as the doubles do
+    if ((__double2hiint(da) & 0x7fffffff) >= __double2hiint(L) - (1 << 20)) {
+      const double invL = gp ? gp->invL[a] : g0.invL[a];
+      da -= L * rint(da * invL);
+    }
+    G.d[a] = da;
+  }
+  G.D2 = G.d[0] * G.d[0] + G.d[1] * G.d[1] + G.d[2] * G.d[2];
+  G.s_i = kSqrt6 * __ldg(&A.sigma[i]);
+  G.s_j = kSqrt6 * __ldg(&A.sigma[j]);
+}
+
+// squared node distances in units of 2^-56: the static point, the common part
+// of each site's nodes and the shifts 2 s |d_a|
+struct PairNodes {
+  long long w0, base[2], tw[2][3];
+};
+__device__ __forceinline__ int pair_nodes(const PairGeom& G, PairNodes& N) {
+  int big = 0;
+  N.w0 = tab_fixed(G.D2, big);
+#pragma unroll
+  for (int site = 0; site < 2; ++site) {
+    const double s = site ? G.s_j : G.s_i;
+    N.base[site] = tab_fixed(fma(s, s, G.D2), big);
+    const double s2 = s + s;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) N.tw[site][a] = tab_fixed(fabs(s2 * G.d[a]), big);
+  }
+  return big;
+}
+
+// float pair of x from its bits (no FP64 instruction): 24 bits, then the other
+// 29; magnitudes below 2^-75 give zero
+__device__ __forceinline__ ff ff_bits(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7ff);
+  if (e <= 948) return ff{0.f, 0.f};
+  const unsigned sign = hi & 0x80000000u;
+  const float h = __uint_as_float(sign | ((unsigned)(e - 896) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
+  const float sc = __uint_as_float(sign | ((unsigned)(e - 948) << 23));
+  return ff{h, (float)(lo & 0x1fffffffu) * sc};
+}
+
+// ---------------------------------------------------------------- direct evaluation
+// Pairs the table does not cover (radial_table.cuh): FP64, one term at a time.
+__device__ __noinline__ int direct_values(const DevPot& P, const PairGeom& G, double* __restrict__ st,
+                                          double* __restrict__ av, double* __restrict__ ph) {
+  int bad = G.D2 < kRMin * kRMin;
+  for (int v = 0; v < P.n_f; ++v) st[v] = av[v] = 0.0;
+  for (int u = 0; u < P.n_phi; ++u) ph[u] = 0.0;
+#pragma unroll 1
+  for (int k = 0; k < 13; ++k) {
+    double r2 = G.D2;
+    if (k < 12) {
+      const double s = k < 6 ? G.s_i : G.s_j, d = G.d[(k / 2) % 3];
+      r2 = fma(s, s, G.D2) + (k & 1 ? -2.0 : 2.0) * s * d;
+      bad |= r2 < kRMin * kRMin;
+    }
+    const double r = sqrt(r2);
+    const double t = fmin(fmax((r - P.rs) * P.inv_w, 0.0), 1.0);
+    const double S = fma(t * t * t, fma(t, fma(-6.0, t, 15.0), -10.0), 1.0);
+    for (int v = 0; v < P.n_f; ++v) {
+      const double e = P.f[v].A * exp(P.f[v].kappa - P.f[v].lambda * r) * S;
+      if (k == 12) st[v] = e;
+      else av[v] += e;
+    }
+    for (int u = 0; u < P.n_phi && k < 12; ++u) ph[u] += P.phi[u].A * exp(P.phi[u].kappa - P.phi[u].lambda * r) * S;
+  }
+  return bad;
+}
+
+// T, U[3], V[2] (force sums of the 12 nodes) and Gs (static point) of one pair
+__device__ __noinline__ void direct_forces(const DevPot& P, const PairGeom& G, const double* __restrict__ cfa,
+                                           const double* __restrict__ cfs, const double* __restrict__ cphi,
+                                           double* __restrict__ out) {
+  for (int c = 0; c < 7; ++c) out[c] = 0.0;
+#pragma unroll 1
+  for (int k = 0; k < 13; ++k) {
+    const int site = k / 6, a = (k / 2) % 3;
+    const double s = (site == 0 ? G.s_i : G.s_j) * (k & 1 ? -1.0 : 1.0);
+    const double r2 = k < 12 ? fma(s, s, G.D2) + 2.0 * s * G.d[a] : G.D2;
+    const double r = sqrt(r2);
+    const double t = fmin(fmax((r - P.rs) * P.inv_w, 0.0), 1.0), t2 = t * t, u1 = 1.0 - t;
+    const double S = fma(t2 * t, fma(t, fma(-6.0, t, 15.0), -10.0), 1.0);
+    const double dS = t2 * (u1 * u1) * (-30.0 * P.inv_w);
+    double w = 0.0;
+    for (int v = 0; v < P.n_f; ++v) {
+      const RadialFn& F = P.f[v];
+      w += (k < 12 ? cfa[v] : cfs[v]) * (F.A * exp(F.kappa - F.lambda * r) * (dS - F.lambda * S));
+    }
+    for (int u = 0; u < P.n_phi && k < 12; ++u) {
+      const RadialFn& F = P.phi[u];
+      w += cphi[u] * (F.A * exp(F.kappa - F.lambda * r) * (dS - F.lambda * S));
+    }
+    w /= r;
+    if (k == 12) {
+      out[6] = w;
+    } else {
+      out[0] += w;
+      out[1 + a] += s * w;
+      out[4 + site] += kSqrt6 * (k & 1 ? -1.0 : 1.0) * (G.d[a] + s) * w;
+    }
+  }
+}
+
+// ---------------------------------------------------------------- geometry records
+// a sum of nodes: integer constant terms and the float pair of the rest
+struct NodeSum {
+  long long c;
+  ff p;
+};
+__device__ __forceinline__ double sum_value(const NodeSum& v, double scale, double*) {
+  return fma((double)v.c, scale, (double)v.p.hi + (double)v.p.lo);
+}
+__device__ __forceinline__ ff sum_value(const NodeSum& v, double scale, ff*) {
+  // |c| < 2^62: the high word as a float, then what it left
+  const int h = (int)(v.c >> 32);
+  const float fh = (float)h;
+  const long long rest = v.c - ((long long)(int)fh << 32);  // below 2^39
+  const float fl = (float)(int)(rest >> 8);
+  const float s = (float)scale;
+  return ff{fh * (s * 4294967296.0f), fl * (s * 256.0f)} + v.p;
+}
+
+template <typename R>
+struct GeoOut;
+template <>
+struct GeoOut<ff> {
+  using T = float2;
+  static constexpr bool kFF = true;
+  static __device__ __forceinline__ T put(ff v) { return make_float2(v.hi, v.lo); }
+  static __device__ __forceinline__ uint4 two(ff a, ff b) {
+    return make_uint4(__float_as_uint(a.hi), __float_as_uint(a.lo), __float_as_uint(b.hi), __float_as_uint(b.lo));
+  }
+  static __device__ __forceinline__ ff from(double v) { return ff_from_double(v); }
+};
+template <>
+struct GeoOut<double> {
+  using T = double;
+  static constexpr bool kFF = false;
+  static __device__ __forceinline__ T put(double v) { return v; }
+  static __device__ __forceinline__ uint4 two(double a, double b) {
+    return make_uint4((unsigned)__double2loint(a), (unsigned)__double2hiint(a), (unsigned)__double2loint(b),
+                      (unsigned)__double2hiint(b));
+  }
+  static __device__ __forceinline__ double from(double v) { return v; }
+};
+
+template <int FIRST, int LAST, int W, bool FFQ>
+__device__ __forceinline__ void add_node(const RadialTab& Tb, const uint4* sm, long long w, int& low, NodeSum* s) {
+  float th, tl;
+  const uint4* row = tab_row(Tb, sm, w, th, tl, low);
+#pragma unroll
+  for (int u = FIRST; u < LAST; ++u) {
+    const uint4 a = row[u * W], b = row[u * W + 1];
+    ff p;
+    if constexpr (FFQ) p = tab_polyff(__uint_as_float(a.z), __uint_as_float(a.w), b, th, tl);
+    else p = tab_poly64(__uint_as_float(a.z), __uint_as_float(a.w), b, row[u * W + 2], th, tl);
+    s[u].c += (long long)(((unsigned long long)a.y << 32) | a.x);
+    tab_acc(s[u].p, p);
+  }
+}
+
+constexpr int kTabThreads = 512;
+
+// The record of every unordered pair (eam.cu: f_v static, 12 <f_v>, 12 <phi_u>)
+// written to both of its entries.  R ff: float-float quality rows and records
+// of float pairs (FP32 modes); R double: FP64 quality.
+template <int S, int NP, typename R>
+__global__ void __launch_bounds__(kTabThreads, 1) k_geo_tab(
+    const __grid_constant__ DevPot P, const __grid_constant__ DevGrid g0, const __grid_constant__ PassArgs A,
+    const __grid_constant__ RadialTab Tb, const int4* __restrict__ pair_rec, int64_t npair,
+    typename GeoOut<R>::T* __restrict__ buf, GeoLayout L) {
+  using O = GeoOut<R>;
+  constexpr int NF = S, NT = NF + NP, W = O::kFF ? kTabWordsFF : kTabWords64;
+  extern __shared__ uint4 sm[];
+  tab_stage(Tb, sm);
+  pdl_wait();
+  pdl_trigger();
+  __syncthreads();
+  if (chunk_halted(A)) return;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < npair; p += stride) {
+    PairRef pr;
+    if (!load_pair(A, pair_rec, p, pr)) continue;
+    PairGeom G;
+    pair_geometry(g0, A, pr.i, pr.j, G);
+    PairNodes N;
+    const int big = pair_nodes(G, N);
+    int low = 0;
+    NodeSum s[NT];
+#pragma unroll
+    for (int u = 0; u < NT; ++u) s[u] = NodeSum{0, ff{0.f, 0.f}};
+    add_node<0, NF, W, O::kFF>(Tb, sm, N.w0, low, s);
+    R val[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) val[c] = (R)0;
+#pragma unroll
+    for (int v = 0; v < NF; ++v) {
+      val[v] = sum_value(s[v], Tb.scale[v], (R*)nullptr);
+      s[v] = NodeSum{0, ff{0.f, 0.f}};
+    }
+#pragma unroll 1
+    for (int site = 0; site < 2; ++site) {
+#pragma unroll 1
+      for (int a = 0; a < 3; ++a) {
+        add_node<0, NT, W, O::kFF>(Tb, sm, N.base[0] + N.tw[0][0], low, s);
+        add_node<0, NT, W, O::kFF>(Tb, sm, N.base[0] - N.tw[0][0], low, s);
+        // the next axis (registers rotate: one copy of the node code)
+        const long long t = N.tw[0][0];
+        N.tw[0][0] = N.tw[0][1];
+        N.tw[0][1] = N.tw[0][2];
+        N.tw[0][2] = t;
+      }
+      N.base[0] = N.base[1];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) N.tw[0][a] = N.tw[1][a];
+    }
+#pragma unroll
+    for (int v = 0; v < NF; ++v) val[NF + v] = sum_value(s[v], Tb.scale[v], (R*)nullptr);
+#pragma unroll
+    for (int u = 0; u < NP; ++u) val[2 * NF + u] = sum_value(s[NF + u], Tb.scale[NF + u], (R*)nullptr);
+    if (big || low < 0) {
+      double st[2], av[2], ph[3];
+      const PairGeom H = G;
+      if (direct_values(P, H, st, av, ph)) atomicOr(A.flags, kFlagGeometry);
+#pragma unroll
+      for (int v = 0; v < NF; ++v)
+        if (v < P.n_f) {
+          val[v] = O::from(st[v]);
+          val[NF + v] = O::from(av[v]);
+        }
+#pragma unroll
+      for (int u = 0; u < NP; ++u)
+        if (u < P.n_phi) val[2 * NF + u] = O::from(ph[u]);
+    }
+    if (P.n_f == NF && (NF == 2 ? (L.ca == 4 && L.cb == 4) : (L.ca == 4 && L.cb == 0))) {
+      // 16-byte stores: plane A of each entry, and plane B (two species)
+      const uint4 v0 = O::two(val[0], val[1]), v1 = O::two(val[2], val[3]);
+      uint4* oa = reinterpret_cast<uint4*>(buf + (int64_t)pr.tp * 4);
+      uint4* oa2 = reinterpret_cast<uint4*>(buf + (int64_t)pr.tr * 4);
+      oa[0] = v0;
+      oa[1] = v1;
+      oa2[0] = v0;
+      oa2[1] = v1;
+      if constexpr (NF == 2) {
+        const uint4 v2 = O::two(val[4], val[5]), v3 = O::two(val[6], val[7]);
+        uint4* ob = reinterpret_cast<uint4*>(buf + L.b_off + (int64_t)pr.tp * 4);
+        uint4* ob2 = reinterpret_cast<uint4*>(buf + L.b_off + (int64_t)pr.tr * 4);
+        ob[0] = v2;
+        ob[1] = v3;
+        ob2[0] = v2;
+        ob2[1] = v3;
+      }
+    } else {
+      typename O::T *oa = buf + (int64_t)pr.tp * L.ca, *oa2 = buf + (int64_t)pr.tr * L.ca;
+      typename O::T *ob = L.cb ? buf + L.b_off + (int64_t)pr.tp * L.cb : oa + 2 * P.n_f;
+      typename O::T *ob2 = L.cb ? buf + L.b_off + (int64_t)pr.tr * L.cb : oa2 + 2 * P.n_f;
+#pragma unroll
+      for (int v = 0; v < NF; ++v)
+        if (v < P.n_f) {
+          oa[v] = oa2[v] = O::put(val[v]);
+          oa[P.n_f + v] = oa2[P.n_f + v] = O::put(val[NF + v]);
+        }
+#pragma unroll
+      for (int u = 0; u < NP; ++u)
+        if (u < P.n_phi) ob[u] = ob2[u] = O::put(val[2 * NF + u]);
+    }
+  }
+}
+
+// ---------------------------------------------------------------- relaxation densities, FP64
+template <int S, int TAB>
+__global__ void __launch_bounds__(kTabThreads, 1) k_rdensity_tab(
+    const __grid_constant__ DevPot P, const __grid_constant__ DevGrid g0, const __grid_constant__ PassArgs A,
+    const __grid_constant__ RadialTab Tb, const int4* __restrict__ pair_rec, int64_t npair, Dbl4* __restrict__ dens) {
+  using TB = Tables<TAB>;
+  constexpr int NF = S, W = kTabWords64;
+  extern __shared__ uint4 sm[];
+  tab_stage(Tb, sm);
+  pdl_wait();
+  pdl_trigger();
+  __syncthreads();
+  if (chunk_halted(A)) return;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < npair; p += stride) {
+    PairRef pr;
+    if (!load_pair(A, pair_rec, p, pr)) continue;
+    PairGeom G;
+    pair_geometry(g0, A, pr.i, pr.j, G);
+    PairNodes N;
+    const int big = pair_nodes(G, N);
+    int low = 0;
+    NodeSum s[NF];
+    double fst[NF], fav[NF];
+#pragma unroll
+    for (int v = 0; v < NF; ++v) s[v] = NodeSum{0, ff{0.f, 0.f}};
+    add_node<0, NF, W, false>(Tb, sm, N.w0, low, s);
+#pragma unroll
+    for (int v = 0; v < NF; ++v) {
+      fst[v] = sum_value(s[v], Tb.scale[v], (double*)nullptr);
+      s[v] = NodeSum{0, ff{0.f, 0.f}};
+    }
+#pragma unroll 1
+    for (int site = 0; site < 2; ++site) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        add_node<0, NF, W, false>(Tb, sm, N.base[0] + N.tw[0][a], low, s);
+        add_node<0, NF, W, false>(Tb, sm, N.base[0] - N.tw[0][a], low, s);
+      }
+      N.base[0] = N.base[1];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) N.tw[0][a] = N.tw[1][a];
+    }
+#pragma unroll
+    for (int v = 0; v < NF; ++v) fav[v] = sum_value(s[v], Tb.scale[v], (double*)nullptr);
+    if (big || low < 0) {
+      double st[2], av[2], ph[3];
+      const PairGeom H = G;
+      if (direct_values(P, H, st, av, ph)) atomicOr(A.flags, kFlagGeometry);
+#pragma unroll
+      for (int v = 0; v < NF; ++v)
+        if (v < P.n_f) {
+          fst[v] = st[v];
+          fav[v] = av[v];
+        }
+    }
+    double ci[4] = {0.0, 0.0, 0.0, 0.0}, cj[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int l = 0; l < S; ++l) {
+      const double xi = __ldg(&A.x[l * A.n + pr.i]), xj = __ldg(&A.x[l * A.n + pr.j]);
+#pragma unroll
+      for (int k = 0; k < S; ++k) {
+        const int fo = TB::f(P, k, l);
+#pragma unroll
+        for (int v = 0; v < NF; ++v)
+          if (fo == v) {
+            ci[k] += xj * fst[v];
+            ci[2 + k] += xj * fav[v];
+            cj[k] += xi * fst[v];
+            cj[2 + k] += xi * fav[v];
+          }
+      }
+    }
+    dens[pr.tp] = Dbl4{ci[0], ci[1], ci[2], ci[3]};
+    dens[pr.tr] = Dbl4{cj[0], cj[1], cj[2], cj[3]};
+  }
+}
+
+// ---------------------------------------------------------------- relaxation forces, FP64
+// dV/dr / r of the pair's weighted terms at one node: the constant terms in
+// FP64, the rest as a float pair
+template <int NT>
+__device__ __forceinline__ double force_node(const RadialTab& Tb, const uint4* sm, long long w, const double* C,
+                                             const ff* Cf, int& low, ff& p) {
+  float th, tl;
+  const uint4* row = tab_row(Tb, sm, w, th, tl, low);
+  double h = 0.0;
+  p = ff{0.f, 0.f};
+#pragma unroll
+  for (int u = 0; u < NT; ++u) {
+    const uint4 a = row[u * kTabWords64];
+    const ff q = tab_poly64(__uint_as_float(a.z), __uint_as_float(a.w), row[u * kTabWords64 + 1],
+                            row[u * kTabWords64 + 2], th, tl);
+    h = fma(C[u], __hiloint2double((int)a.y, (int)a.x), h);
+    ff m = two_prod(Cf[u].hi, q.hi);
+    m.lo = fmaf(Cf[u].hi, q.lo, fmaf(Cf[u].lo, q.hi, m.lo));
+    tab_acc(p, m);
+  }
+  return h;
+}
+
+__device__ __forceinline__ ff ff_times(ff a, ff b) {  // without the final renormalisation
+  ff m = two_prod(a.hi, b.hi);
+  m.lo = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, m.lo));
+  return m;
+}
+
+template <int S, int NP, int TAB>
+__global__ void __launch_bounds__(kTabThreads, 1) k_rforce_tab(
+    const __grid_constant__ DevPot P, const __grid_constant__ DevGrid g0, const __grid_constant__ PassArgs A,
+    const __grid_constant__ RadialTab Tb, const int4* __restrict__ pair_rec, int64_t npair, Dbl4* __restrict__ frc) {
+  using TB = Tables<TAB>;
+  constexpr int NF = S, NT = NF + NP;
+  extern __shared__ uint4 sm[];
+  tab_stage(Tb, sm);
+  pdl_wait();
+  pdl_trigger();
+  __syncthreads();
+  if (A.ctrl != nullptr && A.ctrl->halted) return;
+  const int64_t n = A.n, stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < npair; p += stride) {
+    PairRef pr;
+    if (!load_pair(A, pair_rec, p, pr)) continue;
+    PairGeom G;
+    pair_geometry(g0, A, pr.i, pr.j, G);
+    PairNodes N;
+    const int big = pair_nodes(G, N);
+    int low = 0;
+    // weights of the terms: nodes (C) and the static point (cfs)
+    double C[NT], cfs[NF];
+#pragma unroll
+    for (int u = 0; u < NT; ++u) C[u] = 0.0;
+#pragma unroll
+    for (int v = 0; v < NF; ++v) cfs[v] = 0.0;
+#pragma unroll
+    for (int k = 0; k < S; ++k) {
+      const double xik = __ldg(&A.x[k * n + pr.i]), aik = __ldg(&A.a[k * n + pr.i]), bik = __ldg(&A.b[k * n + pr.i]);
+      const double ajk = __ldg(&A.a[k * n + pr.j]), bjk = __ldg(&A.b[k * n + pr.j]);
+#pragma unroll
+      for (int l = 0; l < S; ++l) {
+        const double xjl = __ldg(&A.x[l * n + pr.j]), xil = __ldg(&A.x[l * n + pr.i]);
+        const int po = TB::phi(P, k, l), fo = TB::f(P, k, l);
+#pragma unroll
+        for (int u = 0; u < NP; ++u)
+          if (po == u) C[NF + u] += xik * xjl;
+#pragma unroll
+        for (int v = 0; v < NF; ++v)
+          if (fo == v) {
+            C[v] += bik * xjl + bjk * xil;
+            cfs[v] += aik * xjl + ajk * xil;
+          }
+      }
+    }
+    ff Cf[NT];
+#pragma unroll
+    for (int u = 0; u < NT; ++u) Cf[u] = ff_bits(C[u]);
+    double out[7];  // T, U[3], V[2], Gs
+    {
+      ff cs[NF], ps;
+#pragma unroll
+      for (int v = 0; v < NF; ++v) cs[v] = ff_bits(cfs[v]);
+      const double h = force_node<NF>(Tb, sm, N.w0, cfs, cs, low, ps);
+      out[6] = h + ((double)ps.hi + (double)ps.lo);
+    }
+    double T0 = 0.0, U0[3] = {0.0, 0.0, 0.0}, Vs[2];
+    ff Tp{0.f, 0.f}, Up[3] = {ff{0.f, 0.f}, ff{0.f, 0.f}, ff{0.f, 0.f}};
+    const double ad[3] = {fabs(G.d[0]), fabs(G.d[1]), fabs(G.d[2])};
+    const ff fd[3] = {ff_bits(ad[0]), ff_bits(ad[1]), ff_bits(ad[2])};
+    double s = G.s_i;
+#pragma unroll 1
+    for (int site = 0; site < 2; ++site) {
+      const ff fs = ff_bits(s);
+      double E0 = 0.0, V0 = 0.0;
+      ff Ep{0.f, 0.f}, Vp{0.f, 0.f};
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        ff p1, p2;
+        const double h1 = force_node<NT>(Tb, sm, N.base[0] + N.tw[0][a], C, Cf, low, p1);
+        const double h2 = force_node<NT>(Tb, sm, N.base[0] - N.tw[0][a], C, Cf, low, p2);
+        const double D = h1 - h2;
+        E0 += h1;
+        E0 += h2;
+        U0[a] = fma(s, D, U0[a]);
+        V0 = fma(ad[a], D, V0);
+        tab_acc(Ep, p1);
+        tab_acc(Ep, p2);
+        tab_acc(p1, ff{-p2.hi, -p2.lo});  // p1 - p2
+        tab_acc(Up[a], ff_times(fs, p1));
+        tab_acc(Vp, ff_times(fd[a], p1));
+      }
+      tab_acc(Tp, Ep);
+      tab_acc(Vp, ff_times(fs, Ep));
+      T0 += E0;
+      const double v = kSqrt6 * (fma(s, E0, V0) + ((double)Vp.hi + (double)Vp.lo));
+      Vs[1] = v;
+      if (site == 0) Vs[0] = v;
+      s = G.s_j;
+      N.base[0] = N.base[1];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) N.tw[0][a] = N.tw[1][a];
+    }
+    out[0] = T0 + ((double)Tp.hi + (double)Tp.lo);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) out[1 + a] = copysign(1.0, G.d[a]) * (U0[a] + ((double)Up[a].hi + (double)Up[a].lo));
+    out[4] = Vs[0];
+    out[5] = Vs[1];
+    if (big || low < 0) {
+      const PairGeom H = G;
+      double ca[2] = {0.0, 0.0}, cs[2] = {0.0, 0.0}, cp[3] = {0.0, 0.0, 0.0}, o[7];
+#pragma unroll
+      for (int v = 0; v < NF; ++v) {
+        ca[v] = C[v];
+        cs[v] = cfs[v];
+      }
+#pragma unroll
+      for (int u = 0; u < NP; ++u) cp[u] = C[NF + u];
+      direct_forces(P, H, ca, cs, cp, o);
+#pragma unroll
+      for (int c = 0; c < 7; ++c) out[c] = o[c];
+    }
+    const double inv12 = 1.0 / 12.0;
+    const double Tt = out[0] * inv12 + out[6];
+    const double fx = -(G.d[0] * Tt + out[1] * inv12), fy = -(G.d[1] * Tt + out[2] * inv12),
+                 fz = -(G.d[2] * Tt + out[3] * inv12);
+    frc[pr.tp] = Dbl4{fx, fy, fz, out[4] * inv12};
+    frc[pr.tr] = Dbl4{-fx, -fy, -fz, out[5] * inv12};
+  }
+}
+
+// one block per SM; few pairs: enough smaller blocks to use every SM
+template <typename... KArgs, typename... Args>
+cudaError_t launch_table_kernel(void (*kernel)(KArgs...), const RadialTab& Tb, int64_t npair, cudaStream_t s,
+                                Args... args) {
+  const size_t shm = (size_t)Tb.nrow * Tb.stride * 16;
+  cudaError_t e = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTabMaxBytes);
+  if (e != cudaSuccess) return e;
+  int dev = 0, sms = 0;
+  e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  int threads = kTabThreads;
+  while (threads > 128 && (npair + threads - 1) / threads < sms) threads /= 2;
+  const int64_t blocks = std::min<int64_t>((npair + threads - 1) / threads, sms);
+  return launch_pdl(kernel, dim3((unsigned)std::max<int64_t>(blocks, 1)), dim3(threads), shm, s, args...);
+}
+
+}  // namespace
+
+cudaError_t launch_geo_tab(int precision, const DevPot& P, const DevGrid& g, const PassArgs& A, const RadialTab& Tb,
+                           const int4* pair_rec, int64_t npair, void* buf, int64_t cap, cudaStream_t s) {
+  if (npair == 0) return cudaSuccess;
+  const GeoLayout L = geo_layout(P, cap);
+  auto run = [&](auto kernel, auto* out) {
+    return launch_table_kernel(kernel, Tb, npair, s, P, g, A, Tb, pair_rec, npair, out, L);
+  };
+  if (precision == 0) {
+    if (P.S == 1) return run(k_geo_tab<1, 1, double>, (double*)buf);
+    if (Tb.np_slots == 2) return run(k_geo_tab<2, 2, double>, (double*)buf);
+    return run(k_geo_tab<2, 3, double>, (double*)buf);
+  }
+  if (P.S == 1) return run(k_geo_tab<1, 1, ff>, (float2*)buf);
+  if (Tb.np_slots == 2) return run(k_geo_tab<2, 2, ff>, (float2*)buf);
+  return run(k_geo_tab<2, 3, ff>, (float2*)buf);
+}
+
+cudaError_t launch_relax_tab(bool force, const DevPot& P, const DevGrid& g, const PassArgs& A, const RadialTab& Tb,
+                             const int4* pair_rec, int64_t npair, void* out, cudaStream_t s) {
+  if (A.n == 0 || npair == 0) return cudaSuccess;
+  auto run = [&](auto kernel) {
+    return launch_table_kernel(kernel, Tb, npair, s, P, g, A, Tb, pair_rec, npair, (Dbl4*)out);
+  };
+  if (!force) {
+    if (P.S == 1) return run(k_rdensity_tab<1, 0>);
+    return P.tab == 1 ? run(k_rdensity_tab<2, 1>) : run(k_rdensity_tab<2, 0>);
+  }
+  if (P.S == 1) return run(k_rforce_tab<1, 1, 0>);
+  if (Tb.np_slots == 2) return run(k_rforce_tab<2, 2, 0>);
+  return P.tab == 1 ? run(k_rforce_tab<2, 3, 1>) : run(k_rforce_tab<2, 3, 0>);
+}
+
+}  // namespace mxe

@@ -1,0 +1,129 @@
+// radial_table.cuh -- the radial terms of a potential as piecewise polynomials
+// in the squared distance, for the FP64 passes and the accurate passes of the
+// FP32 modes.
+//
+// Every node of App. A's rule needs g(r) (or dg/dr / r) of each radial term at
+// r^2 = |d|^2 + s^2 +- 2 s d_a, which is known before any square root.  A term
+// with its switch is a function of w = r^2 alone, so it is tabulated once per
+// context: intervals of width h in w, on each a Taylor polynomial about the
+// centre in tau = (w - w_k)/h, |tau| <= 1/2, formed in double-double arithmetic
+// (radial_table.cu).  The square root, the exponentials and the switch leave
+// the node loop.  On GB300, whose FP64 pipe has 2 lanes per SM against 128 FP32
+// lanes, the point is the split of the polynomial: consecutive Taylor terms
+// fall by about 2^-7, so only the constant term needs 53 bits.  It is an
+// integer on a fixed grid (sums of nodes are exact 64-bit integer additions)
+// or a double (one FMA with the pair's weight); the terms tau c1 .. tau^3 c3
+// run in float-float, tau^4 c4 .. in FP32.
+//
+// The switch is only twice differentiable at r_switch and r_cut: the interval
+// that holds a breakpoint has two rows, one per side, and the row index steps
+// by one at each breakpoint; from r_cut on every w takes one row of zeros.
+//
+// w is a 64-bit integer in units of 2^-56 (w < 128): node distances are integer
+// additions, the interval is a shift, and tau is the remaining bits.  Pairs
+// with a node below the first row (r < r_cut / 4), with |d|^2 >= 64 or with a
+// non-finite coordinate take the direct evaluation.
+#pragma once
+
+#include "mxe_internal.cuh"
+
+namespace mxe {
+
+// A row of one term, FP64 quality: c0 (int64 or double), c1, c2, c3 as float
+// pairs, c4..c7 floats: three 16-byte words.  Float-float quality (degree 4):
+// c0 int64, c1, c2 float pairs, c3, c4: two words.
+constexpr int kTabWords64 = 3, kTabWordsFF = 2;
+constexpr int kTabFixedBits = 56;   // w in units of 2^-56
+constexpr int kTabSumBits = 58;     // |c0| < 2^58 on its grid: 13 nodes sum without overflow
+constexpr double kTabRLow = 0.25;   // first row at (r_cut / 4)^2
+
+// 16-byte words between the rows of consecutive intervals: all terms of an
+// interval lie side by side; an odd count spreads random intervals over the
+// eight 16-byte bank groups of shared memory.
+inline int tab_stride(int nterm, int words) { return (nterm * words) | 1; }
+
+__device__ __forceinline__ void tab_stage(const RadialTab& Tb, uint4* __restrict__ sm) {
+  const int n = Tb.nrow * Tb.stride;
+  for (int t = threadIdx.x; t < n; t += blockDim.x) {
+    const unsigned dst = (unsigned)__cvta_generic_to_shared(sm + t);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(Tb.rows + t) : "memory");
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// x >= 0 in units of 2^-56, truncated; `big` collects x >= 64, infinities and NaN
+__device__ __forceinline__ long long tab_fixed(double x, int& big) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)(b >> 52);  // biased exponent (x >= 0)
+  big |= e >= 1023 + 6;
+  const unsigned long long m = (b << 11) | 0x8000000000000000ull;
+  const int sh = 1023 + 7 - e;
+  return (long long)(sh > 63 ? 0ull : m >> (sh < 1 ? 1 : sh));
+}
+
+// Row of w and the offset from the row's centre; `low` collects w below the
+// first row.  The index is clamped, so every access stays inside the table
+// whatever w is.
+__device__ __forceinline__ const uint4* tab_row(const RadialTab& Tb, const uint4* sm, long long w, float& th, float& tl,
+                                                int& low) {
+  const unsigned hi = (unsigned)((unsigned long long)w >> 32), lo = (unsigned)w;
+  int k = (int)(hi >> Tb.shift) - Tb.k_lo;
+  low |= k;  // negative below the first row
+  k += hi >= Tb.rs_hi ? 1 : 0;
+  if (hi >= Tb.rc_hi) k = Tb.nrow - 1;
+  k = min(max(k, 0), Tb.nrow - 1);
+  const unsigned f1 = __funnelshift_r(lo, hi, Tb.shift + 9) & 0x7fffffu;
+  const unsigned f2 = (lo >> (Tb.shift - 14)) & 0x7fffffu;
+  th = __uint_as_float(0x3f800000u | f1) - 1.5f;
+  // the next 23 bits, at the middle of what they truncate
+  tl = fmaf(__uint_as_float(0x3f800000u | f2), 0x1p-23f, -0x1p-23f * (1.0f - 0x1p-24f));
+  return sm + k * Tb.stride;
+}
+
+// tau c1 + ... + tau^7 c7 as a float pair (the row without its constant term)
+__device__ __forceinline__ ff tab_poly64(float c1h, float c1l, uint4 b, uint4 c, float th, float tl) {
+  float e = fmaf(__uint_as_float(c.w), th, __uint_as_float(c.z));
+  e = fmaf(e, th, __uint_as_float(c.y));
+  e = fmaf(e, th, __uint_as_float(c.x));
+  ff s = fast_two_sum(__uint_as_float(b.z), e * th);
+  s.lo += __uint_as_float(b.w);
+  auto times_tau = [&](ff v) {
+    ff m = two_prod(v.hi, th);
+    m.lo = fmaf(v.lo, th, fmaf(v.hi, tl, m.lo));
+    return m;
+  };
+  ff m = times_tau(s);
+  s = two_sum(__uint_as_float(b.x), m.hi);
+  s.lo += m.lo + __uint_as_float(b.y);
+  m = times_tau(s);
+  s = two_sum(c1h, m.hi);
+  s.lo += m.lo + c1l;
+  return times_tau(s);
+}
+
+// the float-float quality row: tau c1 + ... + tau^5 c5; the low part of c2 and
+// c5 need 8 bits and share a word
+__device__ __forceinline__ ff tab_polyff(float c1h, float c1l, uint4 b, float th, float tl) {
+  float e = fmaf(__uint_as_float(b.y << 16), th, __uint_as_float(b.w));
+  e = fmaf(e, th, __uint_as_float(b.z)) * th;
+  auto times_tau = [&](ff v) {
+    ff m = two_prod(v.hi, th);
+    m.lo = fmaf(v.lo, th, fmaf(v.hi, tl, m.lo));
+    return m;
+  };
+  ff s = two_sum(__uint_as_float(b.x), e);
+  s.lo += __uint_as_float(b.y & 0xffff0000u);
+  const ff m = times_tau(s);
+  s = two_sum(c1h, m.hi);
+  s.lo += m.lo + c1l;
+  return times_tau(s);
+}
+
+// running sum of float pairs without renormalisation
+__device__ __forceinline__ void tab_acc(ff& a, ff v) {
+  const ff s = two_sum(a.hi, v.hi);
+  a.hi = s.hi;
+  a.lo += s.lo + v.lo;
+}
+
+}  // namespace mxe
