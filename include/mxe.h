@@ -61,7 +61,8 @@ typedef enum {
 typedef enum {
     MXE_FP64 = 0,        /* every step in FP64 */
     MXE_FP32_MIXED = 1,  /* node arithmetic (distance, switch, exp, derivatives) in FP32;
-                            each pair's 13-node partial sums added into FP64 per-site sums;
+                            each pair's 13-node partial sums added into per-site sums of
+                            at least FP64 precision (FP64, or three floats rounded to FP64 once);
                             FP64 for per-site results, totals, mu differences, x, FIRE */
     MXE_FP32_FF = 2      /* as MXE_FP32_MIXED, but the per-site sums are carried as
                             unevaluated float pairs (float-float, >= 44-bit significand)

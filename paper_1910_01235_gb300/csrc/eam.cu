@@ -90,6 +90,42 @@ struct AccFF {
   }
 };
 
+// Unevaluated sum of three floats (TwoSum cascade, about 70 bits): the
+// per-site sums of the mixed mode's gathers, at least as exact as an FP64 sum.
+// A conversion and an FP64 addition per value cost 128 FP32 issue slots on
+// GB300 (2 FP64 lanes per SM) and kept the gathers on the FP64 pipe; this takes
+// 13 (float) or 20 (float pair).
+struct AccT {
+  float h, m, l;
+  __device__ __forceinline__ void zero() { h = m = l = 0.f; }
+  __device__ __forceinline__ void add(float x) {
+    const ff s = two_sum(h, x), t = two_sum(m, s.lo);
+    h = s.hi;
+    m = t.hi;
+    l += t.lo;
+  }
+  __device__ __forceinline__ void add(ff x) {
+    const ff s = two_sum(h, x.hi), t = two_sum(m, s.lo), u = two_sum(t.hi, x.lo);
+    h = s.hi;
+    m = u.hi;
+    l += t.lo + u.lo;
+  }
+  __device__ __forceinline__ double get() const { return (double)h + ((double)m + (double)l); }
+  __device__ __forceinline__ float2 get_pair() const {
+    const ff s = two_sum(h, m);
+    const ff t = fast_two_sum(s.hi, s.lo + l);
+    return make_float2(t.hi, t.lo);
+  }
+  __device__ __forceinline__ void team_reduce(int nl) {
+    for (int o = nl >> 1; o > 0; o >>= 1) {
+      const float oh = __shfl_xor_sync(0xffffffffu, h, o), om = __shfl_xor_sync(0xffffffffu, m, o),
+                  ol = __shfl_xor_sync(0xffffffffu, l, o);
+      add(ff{oh, om});
+      l += ol;
+    }
+  }
+};
+
 template <int PREC>
 struct Traits;
 template <>
@@ -1071,7 +1107,7 @@ __global__ void __launch_bounds__(256) k_pair_geo(DevPot P, DevGrid g0, PassArgs
 
 // per-site sums of the float-float gathers in float-float on the FP32 pipe (a
 // conversion to FP64 per term would load GB300's slow FP64 pipe); the mixed
-// and FP64 contexts sum in FP64 (AccD)
+// contexts sum in three floats (AccT), the FP64 contexts in FP64 (AccD)
 struct AccF2 {
   ff v;
   __device__ __forceinline__ void zero() { v = ff(0.f, 0.f); }
@@ -1337,7 +1373,7 @@ __global__ void __launch_bounds__(256) k_pair_mu(DevPot P, PassArgs A,
 //    symmetric in i, j), weighted by the other site's fractions, written to
 //    both entries of the pair;
 //  k_gather_rdensity: per site the sums over its row (float-float in PREC 2,
-//    FP64 otherwise), then the embedding coefficients (a, b): packed FP32
+//    three floats in PREC 1, FP64 in PREC 0), then the embedding coefficients (a, b): packed FP32
 //    records (PREC 1, 2) or the FP64 arrays (PREC 0);
 //  k_pair_rforce: with the pair's weights (x, a, b of both sites) the force
 //    on the row-owner site i, F_i = -(d T + U / 12), d = q_j - q_i (the other
@@ -1373,23 +1409,22 @@ struct Rec4<double> {
   }
 };
 
-// value type of the relaxation records: FP32 in PREC 2 (float-float sums);
-// doubles in PREC 0 and in PREC 1, whose FP32 node values are converted to
-// FP64 by the pair kernel (its FP64 pipe is idle) rather than by the gathers
-// (bound by the FP64 pipe: a conversion and an add per component)
+// value type of the relaxation records: the node arithmetic's
 template <int PREC>
 struct RelaxRec {
-  using V = double;
-};
-template <>
-struct RelaxRec<2> {
-  using V = float;
+  using V = typename Traits<PREC>::R;
 };
 
-// per-site sums of the relaxation gathers: float-float in PREC 2, FP64 otherwise
+// per-site sums of the relaxation gathers: float-float in PREC 2, three floats
+// in PREC 1 (FP32 records either way), FP64 in PREC 0.  PREC 1 with doubles in
+// both places: 58 and 56 us per gather at 55,296 sites, FP64-pipe bound
 template <int PREC>
 struct RelaxAcc {
   using T = AccD;
+};
+template <>
+struct RelaxAcc<1> {
+  using T = AccT;
 };
 template <>
 struct RelaxAcc<2> {
@@ -2655,7 +2690,7 @@ cudaError_t pair_gather_p(int precision, bool mu, const DevPot& P, const PassArg
                           cudaStream_t s) {
   switch (precision) {
     case 0: return pair_gather_t<S, NL, double, AccD>(mu, P, A, buf, C, s);
-    case 1: return pair_gather_t<S, NL, ff, AccD>(mu, P, A, buf, C, s);
+    case 1: return pair_gather_t<S, NL, ff, AccT>(mu, P, A, buf, C, s);
     case 2: return pair_gather_t<S, NL, ff, AccF2>(mu, P, A, buf, C, s);
     default: return cudaErrorInvalidValue;
   }
@@ -2797,7 +2832,7 @@ int64_t resident_grid(const void* kernel, int threads, int64_t work_items) {
   return std::max<int64_t>(1, std::min<int64_t>(need, wave));
 }
 
-size_t relax_record_bytes(int precision) { return precision == 2 ? sizeof(float4) : sizeof(Dbl4); }
+size_t relax_record_bytes(int precision) { return precision == 0 ? sizeof(Dbl4) : sizeof(float4); }
 
 cudaError_t launch_relax_pair(int precision, bool force, const DevPot& P, const DevGrid& g, const PassArgs& A,
                               const int4* pair_rec, int64_t npair, void* dens, void* frc, cudaStream_t s) {
