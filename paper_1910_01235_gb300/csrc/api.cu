@@ -152,6 +152,13 @@ struct mxe_ctx {
   double* tan_buf = nullptr;   // a, b, e values and tangents: 6 [S][n]
   double* th_buf = nullptr;    // per-site term sensitivities, values and tangents: 2 x [2 T][n]
   double* th_sum = nullptr;    // [4 T]: sums of the values, then of the tangents
+  // pair form of the passes (tangent_table.cu): rows, records of every entry
+  uint4* tan_rows = nullptr;
+  RadialTab tan_dens{}, tan_tab{};
+  double* tan_rec = nullptr;
+  int64_t tan_rec_cap = 0;     // entries
+  double* tan_part = nullptr;  // partial sums of the term sensitivities
+  int64_t tan_part_len = 0;
   double* dot_part = nullptr;  // partial sums of dot products
   double* dot_out = nullptr;   // [2]
   double* dot_h = nullptr;     // pinned [2]
@@ -1208,6 +1215,52 @@ mxe_status enqueue_tune_work(mxe_ctx* c, const mxe_state* s) {
 // ---------------------------------------------------------------- second order
 int n_terms(const mxe_ctx* c) { return c->dp.n_phi + c->dp.n_f; }
 
+// The tangent passes run over unordered pairs when the potential has Taylor
+// rows and the records of every entry (12 doubles for two species) fit the
+// device; else over the full list (one thread per site).
+bool ensure_tangent_pairs(mxe_ctx* c) {
+  if (!has_pair_index(c) || !c->pair_rec) return false;
+  if (!c->tan_rows) {
+    if (!plan_radial_tab(c->dp, kTabTaylor64, false, c->tan_dens) ||
+        !plan_radial_tab(c->dp, kTabTaylor64, true, c->tan_tab))
+      return false;
+    const int64_t nd = (int64_t)c->tan_dens.nrow * c->tan_dens.stride;
+    if (dalloc(&c->tan_rows, nd + (int64_t)c->tan_tab.nrow * c->tan_tab.stride) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    c->tan_dens.rows = c->tan_rows;
+    c->tan_tab.rows = c->tan_rows + nd;
+    const int kinds[2] = {kTabTaylor64, kTabTaylor64};
+    RadialTab* tabs[2] = {&c->tan_dens, &c->tan_tab};
+    if (launch_radial_tables(c->dp, kinds, tabs, 2, c->stream) != cudaSuccess) {
+      cudaGetLastError();
+      dfree(c->tan_rows);
+      return false;
+    }
+  }
+  if (c->tan_rec_cap < c->pair_cap) {
+    dfree(c->tan_rec);
+    c->tan_rec_cap = 0;
+    if (dalloc(&c->tan_rec, c->pair_cap * tangent_record_len(c->dp)) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    c->tan_rec_cap = c->pair_cap;
+  }
+  const int64_t part = 4LL * (c->tan_tab.nf_slots + c->tan_tab.np_slots) * tangent_blocks(c->n_upairs);
+  if (c->tan_part_len < part) {
+    dfree(c->tan_part);
+    c->tan_part_len = 0;
+    if (dalloc(&c->tan_part, part) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    c->tan_part_len = part;
+  }
+  return true;
+}
+
 mxe_status ensure_tangent(mxe_ctx* c) {
   if (c->tan_buf) return MXE_OK;
   const int64_t n = c->n, S = c->S, T = n_terms(c);
@@ -1257,6 +1310,13 @@ mxe_status enqueue_tangent(mxe_ctx* c, const mxe_state* s, const double* dq, con
   }
   A.flags = c->flags;
   A.batch = c->B;
+  A.n_ent = c->n_pairs;
+  if (ensure_tangent_pairs(c)) {
+    CK(TIMED("tangent_pairs", launch_tangent_pairs(c->dp, c->grid, A, c->tan_dens, c->tan_tab, c->pair_rec,
+                                                   c->n_upairs, c->tan_rec, c->tan_part, T > 0 ? th_out : nullptr,
+                                                   c->stream)));
+    return MXE_OK;
+  }
   CK(TIMED("tangent", launch_tangent(c->dp, c->grid, A, c->stream)));
   if (th_out && T > 0) {
     CK(launch_col_sum(A.th_v, (int)(2 * T), n, th_out, c->stream));
@@ -1500,6 +1560,9 @@ mxe_status mxe_destroy(mxe_ctx* c) {
   dfree(c->loop_dev);
   if (c->loop_h) cudaFreeHost(c->loop_h);
   dfree(c->tab_rows);
+  dfree(c->tan_rows);
+  dfree(c->tan_rec);
+  dfree(c->tan_part);
   dfree(c->tan_buf);
   dfree(c->emb_buf);
   dfree(c->emb_nrule);

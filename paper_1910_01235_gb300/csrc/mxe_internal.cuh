@@ -100,7 +100,7 @@ struct Tables<2> : Tables<1> {};
 // `stride` 16-byte words, one row per interval of width h (and per side of a
 // breakpoint), `words` words per term, density terms first.
 constexpr int64_t kTabMaxBytes = 200 * 1024;  // staged in one block's shared memory
-enum { kTabValue64 = 0, kTabDeriv64 = 1, kTabValueFF = 2 };
+enum { kTabValue64 = 0, kTabDeriv64 = 1, kTabValueFF = 2, kTabTaylor64 = 3 };
 struct RadialTab {
   const uint4* rows;
   int nrow, stride, words;
@@ -410,7 +410,17 @@ struct TanArgs {
   double *th_v, *th_t;                       // [2 T][n] per-site term sensitivities (null: skip)
   int* flags;
   Batch batch;
+  int64_t n_ent;
 };
+// tangent_table.cu: the same passes over unordered pairs with tabulated terms.
+// dens_tab holds the density terms, tab every term (kind kTabTaylor64); rec:
+// [entries] records of tangent_record_len doubles; th_part: tangent_blocks x
+// 4 T partial sums, th_out [4 T] (null: no term sensitivities)
+int tangent_record_len(const DevPot& P);
+int tangent_blocks(int64_t npair);
+cudaError_t launch_tangent_pairs(const DevPot& P, const DevGrid& g, const TanArgs& A, const RadialTab& dens_tab,
+                                 const RadialTab& tab, const int4* pair_rec, int64_t npair, double* rec,
+                                 double* th_part, double* th_out, cudaStream_t s);
 cudaError_t launch_tangent(const DevPot& P, const DevGrid& g, const TanArgs& A, cudaStream_t s);
 cudaError_t launch_col_sum(const double* col, int ncol, int64_t n, double* out, cudaStream_t s);
 cudaError_t launch_flux_vjp(const double* x, const double* T, const double* mu, const int* bd_off, const int* bd_idx,

@@ -48,7 +48,8 @@ struct PairRef {
   uint32_t code;
   int tp, tr;
 };
-__device__ __forceinline__ bool load_pair(const PassArgs& A, const int4* __restrict__ rec, int64_t p, PairRef& r) {
+template <typename Args>
+__device__ __forceinline__ bool load_pair(const Args& A, const int4* __restrict__ rec, int64_t p, PairRef& r) {
   const int4 v = __ldg(&rec[p]);
   r.i = v.x;
   r.j = (uint32_t)v.y & kIdxMask;
@@ -68,5 +69,32 @@ __device__ __forceinline__ bool load_pair(const PassArgs& A, const int4* __restr
 struct alignas(32) Dbl4 {
   double x, y, z, w;
 };
+
+// ---------------------------------------------------------------- geometry of a pair
+// separation and node offsets (sqrt(6) sigma) of a pair from the FP64 state
+struct PairGeom {
+  double d[3], D2, s_i, s_j;
+};
+// minimum image of q_j - q_i; the division by the box only where a component
+// reaches half the box (pairs of the list are nearer than that elsewhere)
+template <typename Args>
+__device__ __forceinline__ void pair_geometry(const DevGrid& g0, const Args& A, int64_t i, int64_t j, PairGeom& G) {
+  const int64_t n = A.n;
+  const DevGrid* gp = A.batch.nsys ? &A.batch.grids[A.batch.sys_of[i]] : nullptr;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    double da = __ldg(&A.q[a * n + j]) - __ldg(&A.q[a * n + i]);
+    const double L = gp ? gp->L[a] : g0.L[a];
+    // high words of positive doubles order as the doubles do
+    if ((__double2hiint(da) & 0x7fffffff) >= __double2hiint(L) - (1 << 20)) {
+      const double invL = gp ? gp->invL[a] : g0.invL[a];
+      da -= L * rint(da * invL);
+    }
+    G.d[a] = da;
+  }
+  G.D2 = G.d[0] * G.d[0] + G.d[1] * G.d[1] + G.d[2] * G.d[2];
+  G.s_i = kSqrt6 * __ldg(&A.sigma[i]);
+  G.s_j = kSqrt6 * __ldg(&A.sigma[j]);
+}
 
 }  // namespace mxe

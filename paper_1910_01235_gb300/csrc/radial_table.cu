@@ -12,7 +12,7 @@
 namespace mxe {
 namespace {
 
-constexpr int kDeg = 8;  // series order (coefficients 0..8)
+constexpr int kDeg = 9;  // series order (coefficients 0..9)
 
 struct dd {
   double h, l;
@@ -79,12 +79,13 @@ __device__ __forceinline__ void mul(const double* a, const double* b, double* o)
 }
 
 // Taylor coefficients of a term with its switch about w = wc in units of h.
-// The first two carry the constant terms of the value and derivative tables:
-// double-double; the others weigh at most 2^-13 of them: FP64.
+// The first three carry the constant terms of the value and derivative tables:
+// double-double (V0..V2); the others weigh at most 2^-7 of them: FP64.
 __device__ void term_series(const RadialFn& F, double wc, double h, bool beyond_rs, double rs, double rc, dd& V0,
-                            dd& V1, double* V) {
+                            dd& V1, dd& V2, double* V) {
   const dd r0 = dd_sqrt(wc);
   const dd r1 = (0.5 * h) * dd_recip(r0);
+  const dd r2 = (-0.25 * h) * (r1 * dd_recip(dd_of(wc)));
   // r = sqrt(wc + h tau), binomial series
   double r[kDeg + 1];
   r[0] = r0.h;
@@ -94,6 +95,7 @@ __device__ void term_series(const RadialFn& F, double wc, double h, bool beyond_
   // E = A exp(kappa - lambda r): n E_n = -lambda sum_i i r_i E_{n-i}
   const dd e0 = F.A * dd_exp(dd_of(F.kappa) - F.lambda * r0);
   const dd e1 = -(F.lambda * (r1 * e0));
+  const dd e2 = -((0.5 * F.lambda) * (r1 * e1 + 2.0 * (r2 * e0)));
   double E[kDeg + 1];
   E[0] = e0.h;
 #pragma unroll
@@ -105,6 +107,7 @@ __device__ void term_series(const RadialFn& F, double wc, double h, bool beyond_
   }
   V0 = e0;
   V1 = e1;
+  V2 = e2;
   if (!beyond_rs) {
 #pragma unroll
     for (int n = 0; n <= kDeg; ++n) V[n] = E[n];
@@ -114,9 +117,14 @@ __device__ void term_series(const RadialFn& F, double wc, double h, bool beyond_
   const dd iw = dd_recip(dd_of(rc) - dd_of(rs));
   const dd z0 = (r0 - dd_of(rs)) * iw, z02 = z0 * z0, u = dd_of(1.0) - z0;
   const dd S0 = dd_of(1.0) - (z02 * z0) * (dd_of(10.0) - z0 * (dd_of(15.0) - 6.0 * z0));
-  const dd S1 = (-30.0) * ((z02 * (u * u)) * (r1 * iw));
+  const dd dS = (-30.0) * (z02 * (u * u));                              // dS/dz
+  const dd d2S = (-60.0) * ((z0 * u) * (dd_of(1.0) - 2.0 * z0));        // d2S/dz2
+  const dd z1 = r1 * iw;
+  const dd S1 = dS * z1;
+  const dd S2 = 0.5 * (d2S * (z1 * z1)) + dS * (r2 * iw);
   V0 = e0 * S0;
   V1 = e1 * S0 + e0 * S1;
+  V2 = e2 * S0 + e1 * S1 + e0 * S2;
   double z[kDeg + 1], z2[kDeg + 1], z3[kDeg + 1], p[kDeg + 1], t[kDeg + 1];
 #pragma unroll
   for (int n = 0; n <= kDeg; ++n) z[n] = n == 0 ? z0.h : r[n] * iw.h;
@@ -174,17 +182,27 @@ __global__ void __launch_bounds__(32) k_radial_table(const __grid_constant__ Dev
   const bool beyond = row > ks;
   const int k = row - (beyond ? 1 : 0);
   const double wc = ((double)(k + Tb.k_lo) + 0.5) * h;
-  dd V0, V1;
+  dd V0, V1, V2;
   double V[kDeg + 1];
-  term_series(*F, wc, h, beyond, P.rs, P.rc, V0, V1, V);
+  term_series(*F, wc, h, beyond, P.rs, P.rc, V0, V1, V2, V);
+  if (kind == kTabTaylor64) {
+    double2* o = reinterpret_cast<double2*>(out);
+    o[0] = make_double2(V0.h, V1.h);
+    o[1] = make_double2(V2.h, V[3]);
+    o[2] = make_double2(V[4], V[5]);
+    o[3] = make_double2(V[6], V[7]);
+    o[4] = make_double2(V[8], V[9]);
+    return;
+  }
   dd c0 = V0;
-  double c[8] = {0.0, V1.h, V[2], V[3], V[4], V[5], V[6], V[7]};
+  double c[8] = {0.0, V1.h, V2.h, V[3], V[4], V[5], V[6], V[7]};
   double c1l = V1.l;
   if (kind == kTabDeriv64) {  // dV/dr / r = 2 dV/dw
     c0 = (2.0 / h) * V1;
+    c[1] = (4.0 / h) * V2.h;
+    c1l = (4.0 / h) * V2.l;
 #pragma unroll
-    for (int n = 1; n < 8; ++n) c[n] = (2.0 / h) * (n + 1) * V[n + 1];
-    c1l = 0.0;
+    for (int n = 2; n < 8; ++n) c[n] = (2.0 / h) * (n + 1) * V[n + 1];
   } else if (kind == kTabValueFF) {
     // Chebyshev economisation of tau^6 on |tau| <= 1/2 (a = 1/2):
     // x^6 -> 3/2 a^2 x^4 - 9/16 a^4 x^2 + a^6/32
@@ -238,11 +256,13 @@ bool plan_radial_tab(const DevPot& P, int kind, bool with_pairs, RadialTab& Tb) 
   for (int u = 0; u < P.n_phi; ++u) rate(P.phi[u]);
   for (int v = 0; v < P.n_f; ++v) rate(P.f[v]);
   if (!(lam < 1e3) || grow < 0.0) return false;
-  const int bits_h = 5;
-  const double h = std::ldexp(1.0, -bits_h), r_lo = kTabRLow * P.rc;
-  if (!(lam * h <= 0.016 * 4.0 * r_lo)) return false;
-  if (!(h <= 0.004 * 4.0 * P.rs * (P.rc - P.rs))) return false;
-  Tb.words = kind == kTabValueFF ? kTabWordsFF : kTabWords64;
+  // all-FP64 rows of degree 9 afford intervals twice as wide
+  const bool taylor = kind == kTabTaylor64;
+  const int bits_h = taylor ? 4 : 5;
+  const double h = std::ldexp(1.0, -bits_h), r_lo = kTabRLow * P.rc, wide = taylor ? 2.0 : 1.0;
+  if (!(lam * h <= 0.016 * wide * 4.0 * r_lo)) return false;
+  if (!(h <= 0.004 * wide * 4.0 * P.rs * (P.rc - P.rs))) return false;
+  Tb.words = taylor ? kTabWordsTaylor : kind == kTabValueFF ? kTabWordsFF : kTabWords64;
   Tb.nf_slots = P.S;
   Tb.np_slots = !with_pairs ? 0 : P.S == 1 ? 1 : (P.n_phi <= 2 ? 2 : 3);
   Tb.stride = tab_stride(Tb.nf_slots + Tb.np_slots, Tb.words);

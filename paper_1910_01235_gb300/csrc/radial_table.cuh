@@ -32,7 +32,8 @@ namespace mxe {
 // A row of one term, FP64 quality: c0 (int64 or double), c1, c2, c3 as float
 // pairs, c4..c7 floats: three 16-byte words.  Float-float quality (degree 4):
 // c0 int64, c1, c2 float pairs, c3, c4: two words.
-constexpr int kTabWords64 = 3, kTabWordsFF = 2;
+// All FP64 (degree 9, c0..c9; the tangent passes): five words.
+constexpr int kTabWords64 = 3, kTabWordsFF = 2, kTabWordsTaylor = 5;
 constexpr int kTabFixedBits = 56;   // w in units of 2^-56
 constexpr int kTabSumBits = 58;     // |c0| < 2^58 on its grid: 13 nodes sum without overflow
 constexpr double kTabRLow = 0.25;   // first row at (r_cut / 4)^2

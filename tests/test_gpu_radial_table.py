@@ -132,3 +132,37 @@ def test_geometry_status_below_half_angstrom():
         with pytest.raises(M.MxeError) as e:
             g.free_energy_grad()
         assert e.value.status == M.ERR_GEOMETRY
+
+
+@pytest.mark.parametrize("name", ["single", "binary", "slab", "asymmetric", "ragged_cut", "close"])
+def test_tangent_pairs(name):
+    """Hessian products of the pair-wise tangent passes against central
+    differences of the oracle's gradients (step 1e-5 along a unit-size
+    direction: truncation ~h^2 |third derivative| ~1e-8 relative, rounding
+    ~1e-16 / h ~1e-11: 1e-6 of the largest component bounds both), the values
+    against the oracle, and the Hessian-only form against the full one (the
+    same sums in another order: 1e-12)."""
+    s, skin = CASES[name]()
+    g = M.MxeSystem(s, "fp64", skin=skin)
+    g.build_neighbors()
+    rng = np.random.default_rng(3)
+    dq, ds, dx = rng.normal(size=s.q.shape), rng.normal(size=s.n) * 0.3, rng.normal(size=s.x.shape) * 0.01
+    d = [torch.as_tensor(v, dtype=torch.float64, device="cuda") for v in (dq, ds, dx)]
+    out = g.tangent(*d)
+    st, offs, idx = O.neighbors(s.q, s.L, g.r_list)
+    fe = O.free_energy(s, (offs, idx))
+    for k in ("gq", "gs", "mu_ex"):
+        assert off(out[k], fe[k]) <= TOL
+    h, lo_hi = 1e-5, []
+    for sign in (1.0, -1.0):
+        t = s.copy()
+        t.q, t.sigma, t.x = s.q + sign * h * dq, s.sigma + sign * h * ds, s.x + sign * h * dx
+        lo_hi.append(O.free_energy(t, (offs, idx)))
+    for k in ("gq", "gs", "mu_ex"):
+        assert off(out[k + "_t"], (lo_hi[0][k] - lo_hi[1][k]) / (2 * h)) <= 1e-6
+    # Hessian products alone
+    gq_t, gs_t = torch.zeros_like(out["gq_t"]), torch.zeros_like(out["gs_t"])
+    ptr = [M._ptr(v) for v in d]
+    assert M.mxe_tangent(g.ctx, g.state, *ptr, 0, 0, 0, M._ptr(gq_t), M._ptr(gs_t), 0, 0) == M.OK
+    assert off(gq_t, out["gq_t"].cpu().numpy()) <= 1e-12
+    assert off(gs_t, out["gs_t"].cpu().numpy()) <= 1e-12
