@@ -752,11 +752,13 @@ EmbArgs emb_args(mxe_ctx* c) {
 // chemical potentials, whichever A carries).
 mxe_status enqueue_emb_exact(mxe_ctx* c, const PassArgs& A, bool fp64) {
   const EmbArgs E = emb_args(c);
-  CK(TIMED(fp64 ? "emb_nodes_fp64" : "emb_nodes_fp32",
-           launch_emb_exact(false, fp64, c->nl, c->dp, c->grid, A, E, c->stream)));
-  if (A.gq || A.gs || A.mu_ex || A.mu)
-    CK(TIMED(fp64 ? "emb_grad_fp64" : "emb_grad_fp32",
-             launch_emb_exact(true, fp64, c->nl, c->dp, c->grid, A, E, c->stream)));
+  const bool tab = fp64 && c->tan_rows;  // rows built by mxe_set_embedding
+  auto pass = [&](bool second) {
+    return tab ? launch_emb_tab(second, c->dp, c->grid, A, E, c->tan_dens, c->stream)
+               : launch_emb_exact(second, fp64, c->nl, c->dp, c->grid, A, E, c->stream);
+  };
+  CK(TIMED(fp64 ? "emb_nodes_fp64" : "emb_nodes_fp32", pass(false)));
+  if (A.gq || A.gs || A.mu_ex || A.mu) CK(TIMED(fp64 ? "emb_grad_fp64" : "emb_grad_fp32", pass(true)));
   return MXE_OK;
 }
 
@@ -1215,30 +1217,35 @@ mxe_status enqueue_tune_work(mxe_ctx* c, const mxe_state* s) {
 // ---------------------------------------------------------------- second order
 int n_terms(const mxe_ctx* c) { return c->dp.n_phi + c->dp.n_f; }
 
+// FP64 Taylor rows of the potential (tangent passes, exact embedding average):
+// built on first use and kept.
+bool ensure_taylor_rows(mxe_ctx* c) {
+  if (c->tan_rows) return true;
+  if (!plan_radial_tab(c->dp, kTabTaylor64, false, c->tan_dens) ||
+      !plan_radial_tab(c->dp, kTabTaylor64, true, c->tan_tab))
+    return false;
+  const int64_t nd = (int64_t)c->tan_dens.nrow * c->tan_dens.stride;
+  if (dalloc(&c->tan_rows, nd + (int64_t)c->tan_tab.nrow * c->tan_tab.stride) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  c->tan_dens.rows = c->tan_rows;
+  c->tan_tab.rows = c->tan_rows + nd;
+  const int kinds[2] = {kTabTaylor64, kTabTaylor64};
+  RadialTab* tabs[2] = {&c->tan_dens, &c->tan_tab};
+  if (launch_radial_tables(c->dp, kinds, tabs, 2, c->stream) != cudaSuccess) {
+    cudaGetLastError();
+    dfree(c->tan_rows);
+    return false;
+  }
+  return true;
+}
+
 // The tangent passes run over unordered pairs when the potential has Taylor
 // rows and the records of every entry (12 doubles for two species) fit the
 // device; else over the full list (one thread per site).
 bool ensure_tangent_pairs(mxe_ctx* c) {
-  if (!has_pair_index(c) || !c->pair_rec) return false;
-  if (!c->tan_rows) {
-    if (!plan_radial_tab(c->dp, kTabTaylor64, false, c->tan_dens) ||
-        !plan_radial_tab(c->dp, kTabTaylor64, true, c->tan_tab))
-      return false;
-    const int64_t nd = (int64_t)c->tan_dens.nrow * c->tan_dens.stride;
-    if (dalloc(&c->tan_rows, nd + (int64_t)c->tan_tab.nrow * c->tan_tab.stride) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    c->tan_dens.rows = c->tan_rows;
-    c->tan_tab.rows = c->tan_rows + nd;
-    const int kinds[2] = {kTabTaylor64, kTabTaylor64};
-    RadialTab* tabs[2] = {&c->tan_dens, &c->tan_tab};
-    if (launch_radial_tables(c->dp, kinds, tabs, 2, c->stream) != cudaSuccess) {
-      cudaGetLastError();
-      dfree(c->tan_rows);
-      return false;
-    }
-  }
+  if (!has_pair_index(c) || !c->pair_rec || !ensure_taylor_rows(c)) return false;
   if (c->tan_rec_cap < c->pair_cap) {
     dfree(c->tan_rec);
     c->tan_rec_cap = 0;
@@ -2297,6 +2304,7 @@ mxe_status mxe_set_embedding(mxe_ctx* c, int32_t mode) {
     CK(dalloc(&c->emb_buf, 9 * (int64_t)c->S * c->n));
     CK(dalloc(&c->emb_nrule, c->n));
   }
+  if (mode == MXE_EMBED_EXACT) ensure_taylor_rows(c);  // without rows: the direct kernels
   c->embedding = mode;
   c->list_gen += 1;  // a captured staggered step is captured again
   return MXE_OK;

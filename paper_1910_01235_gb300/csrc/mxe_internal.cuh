@@ -368,6 +368,10 @@ struct EmbArgs {
 // A.mu), the first adds the embedding energy into A.site_E
 cudaError_t launch_emb_exact(bool second, bool fp64, int nl, const DevPot& P, const DevGrid& g, const PassArgs& A,
                              const EmbArgs& E, cudaStream_t s);
+// embed_table.cu: the same in FP64 with the density terms from Taylor rows (tab:
+// kind kTabTaylor64, density terms only)
+cudaError_t launch_emb_tab(bool second, const DevPot& P, const DevGrid& g, const PassArgs& A, const EmbArgs& E,
+                           const RadialTab& tab, cudaStream_t s);
 cudaError_t launch_pack_ab(const double* a, const double* b, int64_t n, int S, float4* ab32, cudaStream_t s);
 cudaError_t launch_energy_reduce(const double* site_E, int64_t n, double* partials, double* F4, cudaStream_t s);
 // batches: F4 [nsys][4], one block per system in a fixed order

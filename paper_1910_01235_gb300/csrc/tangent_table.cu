@@ -21,68 +21,12 @@
 
 #include "pair_common.cuh"
 #include "radial_table.cuh"
+#include "taylor_rows.cuh"
 
 namespace mxe {
 namespace {
 
 constexpr int kTanThreads = 256;
-
-struct V3 {  // a term and its derivatives in tau = (w - w_k) / h: V, dV/dtau, 1/2 d2V/dtau2
-  double v, d1, h2;
-};
-
-// the term at w from its formula (w below the first row, or not finite)
-__device__ __noinline__ V3 direct_term(const RadialFn& F, double rs, double rc, double w, double h) {
-  const double r = sqrt(w), iw = 1.0 / (rc - rs);
-  const double z = fmin(fmax((r - rs) * iw, 0.0), 1.0), u = 1.0 - z;
-  const double S = 1.0 - z * z * z * (10.0 - z * (15.0 - 6.0 * z));
-  const double S1 = -30.0 * z * z * u * u * iw, S2 = -60.0 * z * u * (1.0 - 2.0 * z) * iw * iw;
-  const double E = F.A * exp(F.kappa - F.lambda * r), lam = F.lambda;
-  const double Vr = E * (S1 - lam * S), Vrr = E * (S2 - 2.0 * lam * S1 + lam * lam * S);
-  return V3{E * S, h * Vr / (2.0 * r), 0.5 * h * h * (Vrr - Vr / r) / (4.0 * w)};
-}
-
-struct TanTab {
-  RadialTab t;
-  double rs2, rc2, w_lo, ih;
-};
-
-// row of w; null: direct evaluation
-__device__ __forceinline__ const double2* tan_row(const TanTab& Tb, const uint4* sm, double w, double& tau) {
-  const double y = w * Tb.ih, f = floor(y);
-  tau = (y - f) - 0.5;
-  if (!(w >= Tb.w_lo)) return nullptr;
-  int k = w < Tb.rc2 ? (int)f - Tb.t.k_lo + (w >= Tb.rs2 ? 1 : 0) : Tb.t.nrow - 1;
-  k = min(max(k, 0), Tb.t.nrow - 1);
-  return reinterpret_cast<const double2*>(sm + k * Tb.t.stride);
-}
-
-__device__ __forceinline__ V3 horner(const double2* __restrict__ row, double t) {
-  const double2 a = row[0], b = row[1], c = row[2], d = row[3], e = row[4];
-  const double k[9] = {e.x, d.y, d.x, c.y, c.x, b.y, b.x, a.y, a.x};  // c8 .. c0
-  double v = fma(e.y, t, k[0]), d1 = e.y, h2 = e.y;
-  d1 = fma(d1, t, v);
-  v = fma(v, t, k[1]);
-#pragma unroll
-  for (int n = 2; n < 9; ++n) {
-    h2 = fma(h2, t, d1);
-    d1 = fma(d1, t, v);
-    v = fma(v, t, k[n]);
-  }
-  return V3{v, d1, h2};
-}
-
-// slot u of a row: density terms, then pair terms
-__device__ __forceinline__ const RadialFn* slot_fn(const DevPot& P, const RadialTab& T, int u) {
-  if (u < T.nf_slots) return u < P.n_f ? &P.f[u] : nullptr;
-  return u - T.nf_slots < P.n_phi ? &P.phi[u - T.nf_slots] : nullptr;
-}
-__device__ __forceinline__ V3 term_at(const DevPot& P, const TanTab& Tb, const double2* row, int u, double w,
-                                      double tau) {
-  if (row) return horner(row + u * kTabWordsTaylor, tau);
-  const RadialFn* F = slot_fn(P, Tb.t, u);
-  return F ? direct_term(*F, P.rs, P.rc, w, Tb.t.h) : V3{0.0, 0.0, 0.0};
-}
 
 // tangent of the separation and of the node offsets
 struct PairRate {
@@ -103,7 +47,7 @@ __device__ __forceinline__ double rate_of(const double* __restrict__ t, int64_t 
 template <int S>
 __global__ void __launch_bounds__(kTanThreads) k_tan_pair_density(
     const __grid_constant__ DevPot P, const __grid_constant__ DevGrid g0, const __grid_constant__ TanArgs A,
-    const __grid_constant__ TanTab Tb, const int4* __restrict__ pair_rec, int64_t npair, double* __restrict__ rec) {
+    const __grid_constant__ TaylorTab Tb, const int4* __restrict__ pair_rec, int64_t npair, double* __restrict__ rec) {
   constexpr int NF = S;
   extern __shared__ uint4 sm[];
   tab_stage(Tb.t, sm);
@@ -121,7 +65,7 @@ __global__ void __launch_bounds__(kTanThreads) k_tan_pair_density(
     double fst[NF], fst_t[NF], fav[NF], fav_t[NF];
     {
       double tau;
-      const double2* row = tan_row(Tb, sm, G.D2, tau);
+      const double2* row = taylor_row(Tb, sm, G.D2, tau);
       const double td = 2.0 * D.dd * ih;
 #pragma unroll
       for (int v = 0; v < NF; ++v) {
@@ -145,7 +89,7 @@ __global__ void __launch_bounds__(kTanThreads) k_tan_pair_density(
       const double td = 2.0 * (D.dd + fma(sd, s + da, s * dda)) * ih;
       bad |= w < kRMin * kRMin;
       double tau;
-      const double2* row = tan_row(Tb, sm, w, tau);
+      const double2* row = taylor_row(Tb, sm, w, tau);
 #pragma unroll
       for (int v = 0; v < NF; ++v) {
         const V3 f = term_at(P, Tb, row, v, w, tau);
@@ -262,7 +206,7 @@ constexpr int grad_len() {
 template <int S, int NP, bool FULL>
 __global__ void __launch_bounds__(kTanThreads) k_tan_pair_grad(
     const __grid_constant__ DevPot P, const __grid_constant__ DevGrid g0, const __grid_constant__ TanArgs A,
-    const __grid_constant__ TanTab Tb, const int4* __restrict__ pair_rec, int64_t npair, double* __restrict__ rec,
+    const __grid_constant__ TaylorTab Tb, const int4* __restrict__ pair_rec, int64_t npair, double* __restrict__ rec,
     double* __restrict__ th_part) {
   constexpr int NF = S, NT = NF + NP, RL = grad_len<S, FULL>();
   extern __shared__ uint4 sm[];
@@ -322,7 +266,7 @@ __global__ void __launch_bounds__(kTanThreads) k_tan_pair_grad(
     double fst[NF], fst_t[NF], A1 = 0.0, A1d = 0.0;
     {
       double tau;
-      const double2* row = tan_row(Tb, sm, G.D2, tau);
+      const double2* row = taylor_row(Tb, sm, G.D2, tau);
       const double td = 2.0 * D.dd * ih;
       double r = 0.0, rd = 0.0;
       if (theta) {
@@ -370,7 +314,7 @@ __global__ void __launch_bounds__(kTanThreads) k_tan_pair_grad(
           const double td = 2.0 * (D.dd + fma(sgd, sg + da, sg * dda)) * ih;
           bad |= w < kRMin * kRMin;
           double tau;
-          const double2* row = tan_row(Tb, sm, w, tau);
+          const double2* row = taylor_row(Tb, sm, w, tau);
           double r = 0.0, rd = 0.0;
           if (theta) {
             const double ir = rsqrt(w);
@@ -586,21 +530,19 @@ cudaError_t launch_staged(void (*kernel)(KArgs...), const RadialTab& Tb, int blo
   return cudaGetLastError();
 }
 
-TanTab tan_tab(const DevPot& P, const RadialTab& T) { return TanTab{T, P.rs * P.rs, P.rc * P.rc, T.k_lo * T.h, 1.0 / T.h}; }
-
 template <int S, int NP>
 cudaError_t tangent_pairs(const DevPot& P, const DevGrid& g, const TanArgs& A, const RadialTab& dens_tab,
                           const RadialTab& tab, const int4* pair_rec, int64_t npair, double* rec, double* th_part,
                           double* th_out, cudaStream_t s) {
   const int blocks = tangent_blocks(npair);
   const unsigned gblocks = (unsigned)((A.n * kTanLanes + 255) / 256);
-  cudaError_t e = launch_staged(k_tan_pair_density<S>, dens_tab, blocks, s, P, g, A, tan_tab(P, dens_tab), pair_rec,
+  cudaError_t e = launch_staged(k_tan_pair_density<S>, dens_tab, blocks, s, P, g, A, taylor_tab(P, dens_tab), pair_rec,
                                 npair, rec);
   if (e != cudaSuccess) return e;
   k_tan_density_gather<S><<<gblocks, 256, 0, s>>>(P, A, rec);
   const bool full = th_out || A.gq_v || A.gs_v || A.mu_v || A.mu_t;
   if (full) {
-    e = launch_staged(k_tan_pair_grad<S, NP, true>, tab, blocks, s, P, g, A, tan_tab(P, tab), pair_rec, npair, rec,
+    e = launch_staged(k_tan_pair_grad<S, NP, true>, tab, blocks, s, P, g, A, taylor_tab(P, tab), pair_rec, npair, rec,
                       th_out ? th_part : nullptr);
     if (e != cudaSuccess) return e;
     k_tan_grad_gather<S, true><<<gblocks, 256, 0, s>>>(A, rec);
@@ -608,7 +550,7 @@ cudaError_t tangent_pairs(const DevPot& P, const DevGrid& g, const TanArgs& A, c
       k_tan_theta<<<dim3(P.n_phi + P.n_f, 4), 32, 0, s>>>(P, tab.nf_slots, tab.nf_slots + tab.np_slots, blocks,
                                                           th_part, th_out);
   } else {
-    e = launch_staged(k_tan_pair_grad<S, NP, false>, tab, blocks, s, P, g, A, tan_tab(P, tab), pair_rec, npair, rec,
+    e = launch_staged(k_tan_pair_grad<S, NP, false>, tab, blocks, s, P, g, A, taylor_tab(P, tab), pair_rec, npair, rec,
                       (double*)nullptr);
     if (e != cudaSuccess) return e;
     k_tan_grad_gather<S, false><<<gblocks, 256, 0, s>>>(A, rec);
