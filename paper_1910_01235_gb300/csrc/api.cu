@@ -522,14 +522,19 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
   const double r_list = (c->pot.r_cut + kSqrt6 * smax) + skin;
   if (!std::isfinite(r_list)) return MXE_ERR_ARG;
   DevGrid& g = c->grid;
-  double Lmax = 0.0;
+  double Lmax = 0.0, h_max = 0.0;  // h_max: widest cell of the grids with >= 3 cells per axis
   int64_t ncell = 0;
+  auto widest = [&](const DevGrid& gr) {
+    if (gr.nc[0] >= 3 && gr.nc[1] >= 3 && gr.nc[2] >= 3)
+      for (int a = 0; a < 3; ++a) h_max = std::max(h_max, gr.h[a]);
+  };
   if (c->nsys == 0) {
     for (int a = 0; a < 3; ++a) {
       if (!(c->box.L[a] >= 2.0 * r_list)) return MXE_ERR_BOX_TOO_SMALL;
       Lmax = std::max(Lmax, c->box.L[a]);
     }
     ncell = plan_grid(c->box.L, r_list, 8 * n + 4096, g);
+    widest(g);
   } else {
     // one grid per system, cells numbered system after system
     for (int b = 0; b < c->nsys; ++b) {
@@ -540,6 +545,7 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
       const int64_t nb = c->sys_off_h[b + 1] - c->sys_off_h[b];
       c->cell_base_h[b] = (int)ncell;
       ncell += plan_grid(c->boxes[b].L, r_list, 8 * nb + 64, c->grids_h[b]);
+      widest(c->grids_h[b]);
       if (ncell > (int64_t)1 << 30) return MXE_ERR_NBR_OVERFLOW;
     }
     c->cell_base_h[c->nsys] = (int)ncell;
@@ -559,6 +565,12 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
   const double delta = std::max(2.0 * (6.0 * u * qmax + u * Lmax + u * r_list), 8.0 * u * Lmax / 3.0);
   const double band_d = 2.0 * (2.0 * std::sqrt(3.0) * r_list * delta + 3.0 * delta * delta + 4.0 * u * r_list * r_list);
   const float band = (float)(band_d * (1.0 + 1e-6));
+  // The home-frame test alone: 8 u h, plus 2^-50 of the FP64 coordinates for
+  // their own rounding.  With the general bound, which grows with the box, the
+  // FP64 rule ran for a few candidates of most sites of a large box.
+  const double delta_h = 8.0 * u * h_max + std::ldexp(qmax + Lmax, -50);
+  const double home_d = 2.0 * (2.0 * std::sqrt(3.0) * r_list * delta_h + 3.0 * delta_h * delta_h + 4.0 * u * r_list * r_list);
+  const float2 bands = make_float2(band, (float)(std::min(home_d, band_d) * (1.0 + 1e-6)));
   mxe_status ms = ensure_cells(c, ncell);
   if (ms != MXE_OK) return ms;
   if (c->nsys) {
@@ -575,7 +587,7 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
   // largest stencil candidate set: the cell-staged kernels hold it in shared
   // memory.  A rebuild that can skip the count pass (the previous build's
   // longest row bounds this one's) sizes it from the previous build's largest
-  // stencil plus a margin and checks the true size, computed on the device
+  // stencil plus a fifth and checks the true size, computed on the device
   // meanwhile, together with the totals: a larger stencil discards that fill
   // (count + fill instead).  Otherwise the host waits for the size here.
   CK(cudaMemsetAsync(c->max_row, 0, 3 * sizeof(int), st));
@@ -587,7 +599,7 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
                           !std::getenv("MXE_NEIGHBOR_COUNT");
   int cand_cap;
   if (try_direct) {
-    cand_cap = c->cand_cap_prev + c->cand_cap_prev / 8 + 8;
+    cand_cap = c->cand_cap_prev + c->cand_cap_prev / 5 + 8;
   } else {
     CK(cudaMemcpyAsync(c->ints_h + 2, c->max_row + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -600,7 +612,9 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
   bool direct = false;
   int stride = 0;
   if (staged && try_direct) {
-    stride = (c->max_row_h + 16 + 3) & ~3;
+    // a growing r_list takes in whole shells of a lattice (24 of 54 neighbours
+    // at once in FCC): half a row more, at least 32
+    stride = std::min((c->max_row_h + std::max(32, c->max_row_h / 2) + 3) & ~3, 256);
     if ((int64_t)n * stride > c->rows_cap) {
       dfree(c->rows_tmp);
       dfree(c->brows_tmp);
@@ -612,7 +626,7 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
     // a stencil above cand_cap is cut and reported in max_row[2] (not in the
     // context's flags): the check below then discards this fill
     CK(TIMED("build_fill", launch_cell_fill_direct(s->q, c->qf, s->sublattice, s->mobile_mask, n, ncell, g, B,
-                                                   c->cell_start, c->cell_sites, c->abs_cell, rl2, rb2, band, cand_cap,
+                                                   c->cell_start, c->cell_sites, c->abs_cell, rl2, rb2, bands, cand_cap,
                                                    stride, c->rows_tmp, c->brows_tmp, c->nb_cnt, c->bd_cnt,
                                                    pi ? c->n_below : nullptr, pi ? c->pair_cnt : nullptr,
                                                    c->max_row, c->max_row + 2, st)));
@@ -645,7 +659,7 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
     // counts, offsets and totals are in place
   } else if (staged) {
     CK(TIMED("build_count", launch_cell_count(s->q, c->qf, s->sublattice, s->mobile_mask, n, ncell, g, B, c->cell_start,
-                                              c->cell_sites, rl2, rb2, band, cand_cap, c->nb_cnt, c->bd_cnt,
+                                              c->cell_sites, rl2, rb2, bands, cand_cap, c->nb_cnt, c->bd_cnt,
                                               c->max_row, c->flags, st)));
   } else {
     CK(TIMED("build_count", launch_nbr_count(s->q, c->qf, s->sublattice, s->mobile_mask, n, g, B, c->cell_of,
@@ -695,7 +709,7 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
                                               c->bd_idx, st)));
   } else if (staged && max_row <= 256) {
     CK(TIMED("build_fill", launch_cell_fill(s->q, c->qf, s->sublattice, s->mobile_mask, n, ncell, g, B, c->cell_start,
-                                            c->cell_sites, c->abs_cell, rl2, rb2, band, cand_cap, c->nb_off,
+                                            c->cell_sites, c->abs_cell, rl2, rb2, bands, cand_cap, c->nb_off,
                                             c->nb_ent, c->bd_off, c->bd_idx, max_row, c->flags, st)));
   } else {
     CK(TIMED("build_fill", launch_nbr_fill(s->q, c->qf, s->sublattice, s->mobile_mask, n, g, B, c->cell_of,

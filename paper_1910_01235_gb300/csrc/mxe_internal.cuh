@@ -219,7 +219,9 @@ cudaError_t launch_nbr_fill(const double* q, const float4* qf, const uint8_t* su
                             const DevGrid& g, const Batch& B, const int* cell_of, const int* cell_start, const int* cell_sites,
                             const int* abs_cell, double rl2, double rb2, float band, const int* nb_off,
                             uint32_t* nb_ent, const int* bd_off, int* bd_idx, int max_row, cudaStream_t s);
-// cell-staged variants (one block per cell, candidates staged in shared memory)
+// cell-staged variants (one block per cell, candidates staged in shared memory);
+// band: x for the general test, y for the home-frame test (grids of >= 3 cells
+// per axis)
 cudaError_t launch_cand_max(int64_t ncell, const DevGrid& g, const Batch& B, const int* cell_start, int* out,
                             cudaStream_t s);
 size_t cell_stage_bytes(int cand_cap, int max_row, bool fill);
@@ -227,11 +229,11 @@ size_t cell_stage_bytes(int cand_cap, int max_row, bool fill);
 cudaError_t launch_segment_ids(const int* base, int nseg, int64_t count, int* out, cudaStream_t s);
 cudaError_t launch_cell_count(const double* q, const float4* qf, const uint8_t* sub, uint32_t mobile_mask, int64_t n,
                               int64_t ncell, const DevGrid& g, const Batch& B, const int* cell_start, const int* cell_sites,
-                              double rl2, double rb2, float band, int cand_cap, int* nb_cnt, int* bd_cnt,
+                              double rl2, double rb2, float2 band, int cand_cap, int* nb_cnt, int* bd_cnt,
                               int* max_row, int* flags, cudaStream_t s);
 cudaError_t launch_cell_fill(const double* q, const float4* qf, const uint8_t* sub, uint32_t mobile_mask, int64_t n,
                              int64_t ncell, const DevGrid& g, const Batch& B, const int* cell_start, const int* cell_sites,
-                             const int* abs_cell, double rl2, double rb2, float band, int cand_cap,
+                             const int* abs_cell, double rl2, double rb2, float2 band, int cand_cap,
                              const int* nb_off, uint32_t* nb_ent, const int* bd_off, int* bd_idx, int max_row,
                              int* flags, cudaStream_t s);
 // unordered-pair index of a symmetric list (rows sorted by j): n_below[i] =
@@ -251,7 +253,7 @@ cudaError_t launch_pair_fill(const int* nb_off, const uint32_t* nb_ent, int64_t 
 // tail lengths of every row
 cudaError_t launch_cell_fill_direct(const double* q, const float4* qf, const uint8_t* sub, uint32_t mobile_mask,
                                     int64_t n, int64_t ncell, const DevGrid& g, const Batch& B, const int* cell_start,
-                                    const int* cell_sites, const int* abs_cell, double rl2, double rb2, float band,
+                                    const int* cell_sites, const int* abs_cell, double rl2, double rb2, float2 band,
                                     int cand_cap, int stride, uint32_t* rows, int* brows, int* nb_cnt, int* bd_cnt,
                                     int* n_below, int* pair_cnt, int* row_max, int* flags, cudaStream_t s);
 cudaError_t launch_row_compact(const uint32_t* rows, const int* brows, int stride, int64_t n, const int* nb_off,

@@ -483,7 +483,7 @@ __device__ __forceinline__ void warp_sort_row(const uint32_t* __restrict__ buf, 
 __global__ void __launch_bounds__(kCellThreads) k_cell_count(
     const double* __restrict__ q, const float4* __restrict__ qf, const uint8_t* __restrict__ sub, uint32_t mobile_mask,
     int64_t n, DevGrid g0, Batch B, const int* __restrict__ cell_start, const int* __restrict__ cell_sites, double rl2,
-    double rb2, float band, int cand_cap, int* __restrict__ nb_cnt, int* __restrict__ bd_cnt,
+    double rb2, float2 bands, int cand_cap, int* __restrict__ nb_cnt, int* __restrict__ bd_cnt,
     int* __restrict__ max_row, int* __restrict__ flags) {
   extern __shared__ unsigned char smem[];
   __shared__ int s_off[28], s_beg[27];
@@ -501,7 +501,7 @@ __global__ void __launch_bounds__(kCellThreads) k_cell_count(
   const CellStage cs =
       stage_cell(cell, base, g, n, cell_start, cell_sites, qf, cq, cj, s_off, s_beg, s_sh, cand_cap, flags);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  const float rl2f = (float)rl2, rb2f = (float)rb2;
+  const float rl2f = (float)rl2, rb2f = (float)rb2, band = cs.fast ? bands.y : bands.x;
   for (int h = hbeg + warp; h < hend; h += nwarps) {
     const int64_t i = cell_sites[h];
     const double qi[3] = {q[i], q[n + i], q[2 * n + i]};
@@ -538,7 +538,7 @@ template <bool DIRECT>
 __global__ void __launch_bounds__(kCellThreads, 8) k_cell_fill(
     const double* __restrict__ q, const float4* __restrict__ qf, const uint8_t* __restrict__ sub, uint32_t mobile_mask,
     int64_t n, DevGrid g0, Batch B, const int* __restrict__ cell_start, const int* __restrict__ cell_sites,
-    const int* __restrict__ abs_cell, double rl2, double rb2, float band, int cand_cap,
+    const int* __restrict__ abs_cell, double rl2, double rb2, float2 bands, int cand_cap,
     const int* __restrict__ nb_off, uint32_t* __restrict__ nb_ent, const int* __restrict__ bd_off,
     int* __restrict__ bd_idx, int max_row, int* __restrict__ nb_cnt, int* __restrict__ bd_cnt,
     int* __restrict__ n_below, int* __restrict__ pair_cnt, int* __restrict__ row_max, int* __restrict__ flags) {
@@ -595,7 +595,7 @@ __global__ void __launch_bounds__(kCellThreads, 8) k_cell_fill(
     }
     __syncthreads();
   }
-  const float rl2f = (float)rl2, rb2f = (float)rb2;
+  const float rl2f = (float)rl2, rb2f = (float)rb2, band = cs.fast ? bands.y : bands.x;
   for (int h = hbeg + warp; h < hend; h += nwarps) {
     const int64_t i = cell_sites[h];
     const double qi[3] = {q[i], q[n + i], q[2 * n + i]};
@@ -971,7 +971,7 @@ size_t cell_stage_bytes(int cand_cap, int max_row, bool fill) {
 
 cudaError_t launch_cell_count(const double* q, const float4* qf, const uint8_t* sub, uint32_t mobile_mask, int64_t n,
                               int64_t ncell, const DevGrid& g, const Batch& B, const int* cell_start, const int* cell_sites,
-                              double rl2, double rb2, float band, int cand_cap, int* nb_cnt, int* bd_cnt,
+                              double rl2, double rb2, float2 band, int cand_cap, int* nb_cnt, int* bd_cnt,
                               int* max_row, int* flags, cudaStream_t s) {
   if (n == 0 || ncell == 0) return cudaSuccess;
   const size_t shm = cell_stage_bytes(cand_cap, 0, false);
@@ -984,7 +984,7 @@ cudaError_t launch_cell_count(const double* q, const float4* qf, const uint8_t* 
 
 cudaError_t launch_cell_fill(const double* q, const float4* qf, const uint8_t* sub, uint32_t mobile_mask, int64_t n,
                              int64_t ncell, const DevGrid& g, const Batch& B, const int* cell_start, const int* cell_sites,
-                             const int* abs_cell, double rl2, double rb2, float band, int cand_cap,
+                             const int* abs_cell, double rl2, double rb2, float2 band, int cand_cap,
                              const int* nb_off, uint32_t* nb_ent, const int* bd_off, int* bd_idx, int max_row,
                              int* flags, cudaStream_t s) {
   if (n == 0 || ncell == 0) return cudaSuccess;
@@ -1001,7 +1001,7 @@ cudaError_t launch_cell_fill(const double* q, const float4* qf, const uint8_t* s
 
 cudaError_t launch_cell_fill_direct(const double* q, const float4* qf, const uint8_t* sub, uint32_t mobile_mask,
                                     int64_t n, int64_t ncell, const DevGrid& g, const Batch& B, const int* cell_start,
-                                    const int* cell_sites, const int* abs_cell, double rl2, double rb2, float band,
+                                    const int* cell_sites, const int* abs_cell, double rl2, double rb2, float2 band,
                                     int cand_cap, int stride, uint32_t* rows, int* brows, int* nb_cnt, int* bd_cnt,
                                     int* n_below, int* pair_cnt, int* row_max, int* flags, cudaStream_t s) {
   if (n == 0 || ncell == 0) return cudaSuccess;
