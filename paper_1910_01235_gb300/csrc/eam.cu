@@ -2840,8 +2840,8 @@ cudaError_t launch_relax_pair(int precision, bool force, const DevPot& P, const 
   if (!pair_kernels_supported(P)) return cudaErrorInvalidValue;
   switch (precision) {
     case 0: return relax_pair_p<0>(force, P, g, A, pair_rec, npair, dens, frc, s);
-    case 1: return relax_pair_p<1>(force, P, g, A, pair_rec, npair, dens, frc, s);
-    case 2: return relax_pair_p<2>(force, P, g, A, pair_rec, npair, dens, frc, s);
+    case 1:
+    case 2: return launch_relax_pair32(force, P, g, A, pair_rec, npair, force ? frc : dens, s);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -353,6 +353,9 @@ bool pair_kernels_supported(const DevPot& P);
 size_t relax_record_bytes(int precision);
 cudaError_t launch_relax_pair(int precision, bool force, const DevPot& P, const DevGrid& g, const PassArgs& A,
                               const int4* pair_rec, int64_t npair, void* dens, void* frc, cudaStream_t s);
+// the FP32 modes' pair passes (pair_fp32.cu)
+cudaError_t launch_relax_pair32(bool force, const DevPot& P, const DevGrid& g, const PassArgs& A, const int4* pair_rec,
+                                int64_t npair, void* out, cudaStream_t s);
 cudaError_t launch_relax_gather(int precision, bool force, int nl, const DevPot& P, const PassArgs& A,
                                 const void* dens, const void* frc, cudaStream_t s);
 // exact phase average of the embedding term (App. B.2: App. A's rule over a
