@@ -18,7 +18,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libmxe.so")
-SOURCES = ["api.cu", "neighbors.cu", "eam.cu", "radial_table.cu", "pair_table.cu", "pair_fp32.cu", "tangent_table.cu", "embed_table.cu", "relax.cu", "flux.cu", "noalloc.cu", "deriv.cu"]
+SOURCES = ["api.cu", "neighbors.cu", "eam.cu", "radial_table.cu", "pair_table.cu", "pair_fp32.cu", "gathers.cu", "tangent_table.cu", "embed_table.cu", "relax.cu", "flux.cu", "noalloc.cu", "deriv.cu"]
 HEADERS = sorted(os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cuh")) + [os.path.join(ROOT, "include", "mxe.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",

@@ -100,9 +100,10 @@ struct mxe_ctx {
   int64_t rows_cap = 0;
 
   // per-site work arrays
-  double *rho_bar = nullptr, *rho_avg = nullptr, *a = nullptr, *b = nullptr, *e = nullptr;
+  double *a = nullptr, *b = nullptr, *e = nullptr;
   float4 *pos32 = nullptr, *x32 = nullptr, *ab32 = nullptr;
-  float4 *pos32lo = nullptr, *x32lo = nullptr, *ab32lo = nullptr;  // float-float remainders (FP32 modes)
+  float4* pos32lo = nullptr;  // float-pair remainders (direct float-float pass)
+  double* srec = nullptr;     // site records of the accurate gathers
   double *gq = nullptr, *gs = nullptr, *mu_ex = nullptr;
   double* site_E = nullptr;
   double* partials = nullptr;
@@ -432,18 +433,15 @@ void fill_pass(mxe_ctx* c, const mxe_state* s, PassArgs& A) {
   A.pos32 = c->pos32;
   A.x32 = c->x32;
   A.pos32lo = c->pos32lo;
-  A.x32lo = c->x32lo;
   A.nb_off = c->nb_off;
   A.nb_ent = c->nb_ent;
   A.n = c->n;
   A.n_ent = c->n_pairs;
-  A.rho_bar = c->rho_bar;
-  A.rho_avg = c->rho_avg;
   A.a = c->a;
   A.b = c->b;
   A.e = c->e;
   A.ab32 = c->ab32;
-  A.ab32lo = c->ab32lo;
+  A.srec = c->srec;
   A.gq = c->gq;
   A.gs = c->gs;
   A.mu_ex = c->mu_ex;
@@ -687,7 +685,9 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
     dfree(c->pair_buf);
     const int64_t cap = std::max<int64_t>(c->nb_cap, npairs);
     CK(dalloc(&c->pair_rec, cap / 2 + 64));
-    CK(dalloc(&c->pair_buf, cap * (int64_t)pair_record_len(c->dp)));  // one record per entry
+    // one record per entry, wide enough for the force records a free-energy call puts there
+    const int64_t rec = std::max<int64_t>(pair_record_len(c->dp) * (int64_t)sizeof(double), relax_record_bytes(c->precision));
+    CK(dalloc_bytes((void**)&c->pair_buf, cap * rec));
     dfree(c->ent_dens);
     dfree(c->ent_frc);
     if (c->relax_records) {
@@ -818,7 +818,8 @@ mxe_status enqueue_passes(mxe_ctx* c, const mxe_state* s, PassArgs& A, bool want
   const DevPot& PP = c->embedding ? c->dp_pair : c->dp;
   if (fp32)
     CK(TIMED("pack", launch_pack(s->q, s->sigma, s->x, c->abs_cell, c->n, c->S, c->grid, c->B, c->pos32, c->x32,
-                   hl && want_mu ? c->pos32lo : nullptr, hl && want_mu ? c->x32lo : nullptr, st)));
+                   hl && want_mu && !c->tab_rows ? c->pos32lo : nullptr, hl && want_mu ? c->srec : nullptr,
+                   site_record_len(c->dp), st)));
   if (!hl) {  // full-list passes
     if (!fp32) {
       CK(TIMED(cls_name("density", 0), launch_density(0, c->nl, PP, c->grid, A, st)));
@@ -844,7 +845,6 @@ mxe_status enqueue_passes(mxe_ctx* c, const mxe_state* s, PassArgs& A, bool want
     PassArgs G = A;
     if (!fp32) {  // FP64: no packed records
       G.ab32 = nullptr;
-      G.ab32lo = nullptr;
     }
     CK(TIMED(prec == MXE_FP64 ? "pair_geo64" : "pair_ff",
              c->tab_rows ? launch_geo_tab(prec, PP, c->grid, G, c->tab_geo, c->pair_rec, c->n_upairs, c->pair_buf,
@@ -863,17 +863,9 @@ mxe_status enqueue_passes(mxe_ctx* c, const mxe_state* s, PassArgs& A, bool want
     // Before the first relaxation its records go where the geometry records
     // were (the gathers above have read them), so the call allocates nothing.
     // Against the full-list kernel at 108,000 sites FP64: 19.0 -> 1.4 ms.
-    void* frc = half_list_forces(c) ? c->ent_frc
-                : pair_record_len(PP) * sizeof(double) >= relax_record_bytes(prec) ? (void*)c->pair_buf
-                                                                                   : nullptr;
-    if (frc) {
-      CK(TIMED(relax_pair_name(true, prec), relax_pair_pass(c, true, PP, F, nullptr, frc)));
-      CK(TIMED(relax_gather_name(true, prec),
-               launch_relax_gather(prec, true, c->nl, PP, F, nullptr, frc, st)));
-    } else {
-      CK(TIMED(cls_name("gradient", prec, kGradForceNoE),
-               launch_gradient(prec, kGradForceNoE, c->nl, PP, c->grid, F, st)));
-    }
+    void* frc = half_list_forces(c) ? c->ent_frc : (void*)c->pair_buf;
+    CK(TIMED(relax_pair_name(true, prec), relax_pair_pass(c, true, PP, F, nullptr, frc)));
+    CK(TIMED(relax_gather_name(true, prec), launch_relax_gather(prec, true, c->nl, PP, F, nullptr, frc, st)));
   }
   // the accurate pass: the exact average in FP64
   return c->embedding ? enqueue_emb_exact(c, A, true) : MXE_OK;
@@ -1068,7 +1060,7 @@ mxe_status fire_loop(mxe_ctx* c, mxe_state* s, int max_iter, int chunk, Ctrl& H)
     H.sigma_max_build = c->sigma_max_build;
     CK(cudaMemcpyAsync(c->ctrl, &H, sizeof(Ctrl), cudaMemcpyHostToDevice, st));
     if (c->precision != MXE_FP64)
-      CK(TIMED("pack", launch_pack(s->q, s->sigma, s->x, c->abs_cell, c->n, c->S, c->grid, c->B, c->pos32, c->x32, nullptr, nullptr, st)));
+      CK(TIMED("pack", launch_pack(s->q, s->sigma, s->x, c->abs_cell, c->n, c->S, c->grid, c->B, c->pos32, c->x32, nullptr, nullptr, 0, st)));
     // the rebuild may have reallocated the lists: take the current pointers
     relax_pass_args(c, s, A);
   }
@@ -1119,7 +1111,7 @@ mxe_status enqueue_staggered_step(mxe_ctx* c, mxe_state* s, const StepKey& k) {
                      c->mu_eff, c->nsys ? c->dt_sys : nullptr, c->nsys ? c->sys_of : nullptr, c->ctrl, st));
   CK(launch_commit_x(s->x, c->x_new, (int64_t)c->S * c->n, c->step_flags, c->flags, c->ctrl, st));
   if (c->precision != MXE_FP64)
-    CK(launch_pack(s->q, s->sigma, s->x, c->abs_cell, c->n, c->S, c->grid, c->B, c->pos32, c->x32, nullptr, nullptr, st));
+    CK(launch_pack(s->q, s->sigma, s->x, c->abs_cell, c->n, c->S, c->grid, c->B, c->pos32, c->x32, nullptr, nullptr, 0, st));
   CK(launch_fire_zero_v(c->vq, c->vs, c->n, c->ctrl, st));
   if (c->nsys) CK(launch_fire_seg_init(c->sf, c->nsys, k.dt0, k.alpha0, c->ctrl, st));
   PassArgs A;
@@ -1220,7 +1212,7 @@ mxe_status enqueue_tune_work(mxe_ctx* c, const mxe_state* s) {
   fill_pass(c, s, A);
   A.site_E = nullptr;
   A.lean = 1;
-  if (c->precision != MXE_FP64) CK(launch_pack(s->q, s->sigma, s->x, c->abs_cell, c->n, c->S, c->grid, c->B, c->pos32, c->x32, nullptr, nullptr, c->stream));
+  if (c->precision != MXE_FP64) CK(launch_pack(s->q, s->sigma, s->x, c->abs_cell, c->n, c->S, c->grid, c->B, c->pos32, c->x32, nullptr, nullptr, 0, c->stream));
   for (int r = 0; r < 2; ++r) {
     ms = enqueue_force_passes(c, A);
     if (ms != MXE_OK) return ms;
@@ -1484,8 +1476,6 @@ mxe_status mxe_create_batch(mxe_ctx** out, int32_t n_systems, const mxe_box* box
   A(dalloc(&c->smax_bits, 2));
   A(dalloc(&c->qf, 2 * n));
   A(dalloc(&c->q_build, 3 * n));
-  A(dalloc(&c->rho_bar, S * n));
-  A(dalloc(&c->rho_avg, S * n));
   A(dalloc(&c->a, S * n));
   A(dalloc(&c->b, S * n));
   A(dalloc(&c->e, S * n));
@@ -1498,11 +1488,8 @@ mxe_status mxe_create_batch(mxe_ctx** out, int32_t n_systems, const mxe_box* box
     A(dalloc(&c->n_below, n));
     A(dalloc(&c->pair_cnt, n));
     A(dalloc(&c->pair_off, n + 1));
-    if (precision != MXE_FP64) {
-      A(dalloc(&c->pos32lo, n));
-      A(dalloc(&c->x32lo, n));
-      A(dalloc(&c->ab32lo, 2 * n));
-    }
+    if (precision != MXE_FP64) A(dalloc(&c->pos32lo, n));
+    A(dalloc(&c->srec, n * site_record_len(c->dp)));
   }
   A(init_ff_exp_table());
   A(dalloc(&c->gq, 3 * n));
@@ -1621,8 +1608,6 @@ mxe_status mxe_destroy(mxe_ctx* c) {
   dfree(c->smax_bits);
   dfree(c->qf);
   dfree(c->q_build);
-  dfree(c->rho_bar);
-  dfree(c->rho_avg);
   dfree(c->a);
   dfree(c->b);
   dfree(c->e);
@@ -1630,8 +1615,7 @@ mxe_status mxe_destroy(mxe_ctx* c) {
   dfree(c->x32);
   dfree(c->ab32);
   dfree(c->pos32lo);
-  dfree(c->x32lo);
-  dfree(c->ab32lo);
+  dfree(c->srec);
   dfree(c->gq);
   dfree(c->gs);
   dfree(c->mu_ex);
@@ -2149,7 +2133,7 @@ mxe_status mxe_relax(mxe_ctx* c, mxe_state* s, double ftol, int32_t max_iter, co
   CK(cudaMemcpyAsync(c->ctrl, &H, sizeof(Ctrl), cudaMemcpyHostToDevice, st));
   if (c->nsys) CK(launch_fire_seg_init(c->sf, c->nsys, fp.dt0, fp.alpha0, nullptr, st));
   if (c->precision != MXE_FP64)
-    CK(TIMED("pack", launch_pack(s->q, s->sigma, s->x, c->abs_cell, n, c->S, c->grid, c->B, c->pos32, c->x32, nullptr, nullptr, st)));
+    CK(TIMED("pack", launch_pack(s->q, s->sigma, s->x, c->abs_cell, n, c->S, c->grid, c->B, c->pos32, c->x32, nullptr, nullptr, 0, st)));
   mxe_status result = fire_loop(c, s, max_iter, fp.check_every > 0 ? fp.check_every : 16, H);
   mxe_status info = record_relax_info(c, H);
   if (info != MXE_OK && result == MXE_OK) result = info;
@@ -2235,7 +2219,7 @@ mxe_status mxe_run_staggered(mxe_ctx* c, mxe_state* s, int32_t n_steps, double d
       // (velocities, dt and alpha kept) outside the graph
       CK(cudaMemcpyAsync(c->ctrl, &H, sizeof(Ctrl), cudaMemcpyHostToDevice, st));
       if (c->precision != MXE_FP64)
-        CK(TIMED("pack", launch_pack(s->q, s->sigma, s->x, c->abs_cell, c->n, c->S, c->grid, c->B, c->pos32, c->x32, nullptr, nullptr, st)));
+        CK(TIMED("pack", launch_pack(s->q, s->sigma, s->x, c->abs_cell, c->n, c->S, c->grid, c->B, c->pos32, c->x32, nullptr, nullptr, 0, st)));
       ms = fire_loop(c, s, max_iter, chunk, H);
       if (ms != MXE_OK && ms != MXE_ERR_NO_CONVERGE) {
         result = ms;

@@ -29,6 +29,7 @@
 #include <mutex>
 #include <vector>
 
+#include "accum.cuh"
 #include "ff.cuh"
 #include "mxe_internal.cuh"
 #include "pair_common.cuh"
@@ -48,83 +49,6 @@ cudaError_t init_ff_exp_table() {
 }
 
 namespace {
-
-// ---------------------------------------------------------------- accumulators
-struct AccD {
-  double v;
-  __device__ __forceinline__ void zero() { v = 0.0; }
-  __device__ __forceinline__ void add(double x) { v += x; }
-  __device__ __forceinline__ void add(float x) { v += (double)x; }
-  __device__ __forceinline__ void add(ff x) { v += ff_to_double(x); }
-  __device__ __forceinline__ double get() const { return v; }
-  __device__ __forceinline__ float2 get_pair() const {
-    const float h = (float)v;
-    return make_float2(h, (float)(v - (double)h));
-  }
-  __device__ __forceinline__ void team_reduce(int nl) {
-    for (int o = nl >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  }
-};
-
-// Unevaluated sum hi + lo of floats; TwoSum (Knuth) keeps the rounding error
-// of every addition, so the pair carries about twice the float significand.
-struct AccFF {
-  float hi, lo;
-  __device__ __forceinline__ void zero() { hi = 0.f; lo = 0.f; }
-  __device__ __forceinline__ void add(float x) {
-    float s = hi + x;
-    float bp = s - hi;
-    float err = (hi - (s - bp)) + (x - bp);
-    hi = s;
-    lo += err;
-  }
-  __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
-  __device__ __forceinline__ float2 get_pair() const { return make_float2(hi, lo); }
-  __device__ __forceinline__ void team_reduce(int nl) {
-    for (int o = nl >> 1; o > 0; o >>= 1) {
-      float oh = __shfl_xor_sync(0xffffffffu, hi, o);
-      float ol = __shfl_xor_sync(0xffffffffu, lo, o);
-      add(oh);
-      lo += ol;
-    }
-  }
-};
-
-// Unevaluated sum of three floats (TwoSum cascade, about 70 bits): the
-// per-site sums of the mixed mode's gathers, at least as exact as an FP64 sum.
-// A conversion and an FP64 addition per value cost 128 FP32 issue slots on
-// GB300 (2 FP64 lanes per SM) and kept the gathers on the FP64 pipe; this takes
-// 13 (float) or 20 (float pair).
-struct AccT {
-  float h, m, l;
-  __device__ __forceinline__ void zero() { h = m = l = 0.f; }
-  __device__ __forceinline__ void add(float x) {
-    const ff s = two_sum(h, x), t = two_sum(m, s.lo);
-    h = s.hi;
-    m = t.hi;
-    l += t.lo;
-  }
-  __device__ __forceinline__ void add(ff x) {
-    const ff s = two_sum(h, x.hi), t = two_sum(m, s.lo), u = two_sum(t.hi, x.lo);
-    h = s.hi;
-    m = u.hi;
-    l += t.lo + u.lo;
-  }
-  __device__ __forceinline__ double get() const { return (double)h + ((double)m + (double)l); }
-  __device__ __forceinline__ float2 get_pair() const {
-    const ff s = two_sum(h, m);
-    const ff t = fast_two_sum(s.hi, s.lo + l);
-    return make_float2(t.hi, t.lo);
-  }
-  __device__ __forceinline__ void team_reduce(int nl) {
-    for (int o = nl >> 1; o > 0; o >>= 1) {
-      const float oh = __shfl_xor_sync(0xffffffffu, h, o), om = __shfl_xor_sync(0xffffffffu, m, o),
-                  ol = __shfl_xor_sync(0xffffffffu, l, o);
-      add(ff{oh, om});
-      l += ol;
-    }
-  }
-};
 
 template <int PREC>
 struct Traits;
@@ -272,11 +196,7 @@ __device__ __forceinline__ void load_site(const PassArgs& A, int64_t j, SiteData
   d.p[0] = ff(P.x, Pl.x);
   d.p[1] = ff(P.y, Pl.y);
   d.p[2] = ff(P.z, Pl.z);
-  d.sig = ff(P.w, Pl.w);
-  const float4 X = __ldg(&A.x32[j]), Xl = __ldg(&A.x32lo[j]);
-  const float xs[4] = {X.x, X.y, X.z, X.w}, xl[4] = {Xl.x, Xl.y, Xl.z, Xl.w};
-#pragma unroll
-  for (int k = 0; k < S; ++k) d.x[k] = ff(xs[k], xl[k]);
+  d.sig = ff(P.w, Pl.w);  // the geometry pass needs no fractions
 }
 template <int PREC, int S>
 __device__ __forceinline__ void load_site(const PassArgs& A, int64_t j, SiteData<PREC, S>& d) {
@@ -327,16 +247,6 @@ __device__ __forceinline__ void load_ab(const PassArgs& A, int64_t j, double a[S
   for (int k = 0; k < S; ++k) {
     a[k] = A.a[k * A.n + j];
     b[k] = A.b[k * A.n + j];
-  }
-}
-template <int S>
-__device__ __forceinline__ void load_ab(const PassArgs& A, int64_t j, ff a[S], ff b[S], SiteData<3, S>*) {
-  const float4 v0 = __ldg(&A.ab32[2 * j]), l0 = __ldg(&A.ab32lo[2 * j]);
-  a[0] = ff(v0.x, l0.x);
-  b[0] = ff(v0.y, l0.y);
-  if (S > 1) {
-    a[1 < S ? 1 : 0] = ff(v0.z, l0.z);
-    b[1 < S ? 1 : 0] = ff(v0.w, l0.w);
   }
 }
 template <int PREC, int S>
@@ -404,7 +314,7 @@ __global__ void __launch_bounds__(256, MXE_DENSITY_MIN_BLOCKS) k_density(DevPot 
       const R D2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
       // every node lies at least |d| - max(s_i, s_j) from the origin site:
       // only a pair closer than 0.5 A + that shift needs its nodes checked
-      constexpr bool kNodeCheck = PREC == 0 || PREC == 3;
+      constexpr bool kNodeCheck = PREC == 0;
       const R s_max = s_i < s_j ? s_j : s_i;
       const R near = (R)kRMin + s_max;
       const bool close = D2 < near * near;
@@ -422,13 +332,11 @@ __global__ void __launch_bounds__(256, MXE_DENSITY_MIN_BLOCKS) k_density(DevPot 
         }
       }
       // 12 nodes: site i moved (base_i), site j moved (base_j), each +-s along each axis
-      // float-float node arithmetic is long: keep its node loops rolled so the
-      // kernel fits the instruction cache
-#pragma unroll(PREC == 3 ? 1 : 2)
+#pragma unroll
       for (int site = 0; site < 2; ++site) {
         const R s = site == 0 ? s_i : s_j;
         const R base = D2 + s * s;
-#pragma unroll(PREC == 3 ? 1 : 3)
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
           const R tw = (R)2 * s * d[a];
 #pragma unroll
@@ -526,7 +434,7 @@ __global__ void __launch_bounds__(256, MXE_DENSITY_MIN_BLOCKS) k_density(DevPot 
     if (P.E[k] == 0.0) {
       // no embedding energy for this element
     } else if (rbar > kRhoMin) {
-      if (PREC == 0 || PREC == 3) {
+      if (PREC == 0) {
         const double sq = sqrt(rbar);
         const double F = -P.E[k] * sq;
         const double dF = -P.E[k] / (2.0 * sq);
@@ -549,8 +457,6 @@ __global__ void __launch_bounds__(256, MXE_DENSITY_MIN_BLOCKS) k_density(DevPot 
     } else {
       flag |= kFlagGeometry;
     }
-    A.rho_bar[k * n + i] = rbar;
-    A.rho_avg[k * n + i] = ravg;
     A.e[k * n + i] = e;
     A.a[k * n + i] = ak;
     A.b[k * n + i] = bk;
@@ -560,16 +466,6 @@ __global__ void __launch_bounds__(256, MXE_DENSITY_MIN_BLOCKS) k_density(DevPot 
   if (PREC != 0) {
     A.ab32[2 * i] = make_float4(ab[0], ab[1], ab[2], ab[3]);
     if (S > 2) A.ab32[2 * i + 1] = make_float4(ab[4], ab[5], ab[6], ab[7]);
-  }
-  if (PREC == 3) {
-    float lo[4];
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const double av = k < S ? A.a[k * n + i] : 0.0, bv = k < S ? A.b[k * n + i] : 0.0;
-      lo[2 * k] = (float)(av - (double)(float)av);
-      lo[2 * k + 1] = (float)(bv - (double)(float)bv);
-    }
-    A.ab32lo[2 * i] = make_float4(lo[0], lo[1], lo[2], lo[3]);
   }
   if (flag) atomicOr(A.flags, flag);
 }
@@ -678,13 +574,11 @@ __global__ void __launch_bounds__(256, MXE_GRADIENT_MIN_BLOCKS) k_gradient(DevPo
 #pragma unroll
       for (int v = 0; v < NF; ++v) af[v] = (R)0;
       R T = (R)0, U[3] = {(R)0, (R)0, (R)0}, Vs = (R)0;
-      // float-float node arithmetic is long: keep its node loops rolled so the
-      // kernel fits the instruction cache
-#pragma unroll(PREC == 3 ? 1 : 2)
+#pragma unroll
       for (int site = 0; site < 2; ++site) {
         const R s = site == 0 ? s_i : s_j;
         const R base = D2 + s * s;
-#pragma unroll(PREC == 3 ? 1 : 3)
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
           const R tw = (R)2 * s * d[a];
           R w2[2];
@@ -963,13 +857,12 @@ __global__ void __launch_bounds__(256) k_pair_geo(DevPot P, DevGrid g0, PassArgs
   const R D2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
   int bad = D2 < (R)(kRMin * kRMin);
   // component c of the record, at both entries of the pair: the densities (c
-  // below 2 n_f) in plane A, the pair terms in plane B when the record is
-  // split, else after the densities
+  // below 2 n_f) in plane A, the pair terms in plane B
   typename GeoRec<R>::T* oa = buf + pr_.tp * (int64_t)L.ca;
   typename GeoRec<R>::T* oa2 = buf + pr_.tr * (int64_t)L.ca;
   const int c_b = 2 * P.n_f;
-  typename GeoRec<R>::T* ob = L.cb ? buf + L.b_off + pr_.tp * (int64_t)L.cb : oa + c_b;
-  typename GeoRec<R>::T* ob2 = L.cb ? buf + L.b_off + pr_.tr * (int64_t)L.cb : oa2 + c_b;
+  typename GeoRec<R>::T* ob = buf + L.b_off + pr_.tp * (int64_t)L.cb;
+  typename GeoRec<R>::T* ob2 = buf + L.b_off + pr_.tr * (int64_t)L.cb;
   auto put = [&](int c, R v) {
     const typename GeoRec<R>::T w = GeoRec<R>::put(v);
     if (c < c_b) {
@@ -1105,342 +998,28 @@ __global__ void __launch_bounds__(256) k_pair_geo(DevPot P, DevGrid g0, PassArgs
   if (bad) atomicOr(A.flags, kFlagGeometry);
 }
 
-// per-site sums of the float-float gathers in float-float on the FP32 pipe (a
-// conversion to FP64 per term would load GB300's slow FP64 pipe); the mixed
-// contexts sum in three floats (AccT), the FP64 contexts in FP64 (AccD)
-struct AccF2 {
-  ff v;
-  __device__ __forceinline__ void zero() { v = ff(0.f, 0.f); }
-  __device__ __forceinline__ void add(ff x) { v = v + x; }
-  __device__ __forceinline__ double get() const { return ff_to_double(v); }
-  __device__ __forceinline__ void team_reduce(int nl) {
-    for (int o = nl >> 1; o > 0; o >>= 1) {
-      const ff w(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
-      v = v + w;
-    }
-  }
-};
-
-// molar fractions of a neighbour in the accurate passes
-template <int S>
-__device__ __forceinline__ void load_x(const PassArgs& A, int64_t j, ff x[S]) {
-  const float4 X = __ldg(&A.x32[j]), Xl = __ldg(&A.x32lo[j]);
-  const float xs[4] = {X.x, X.y, X.z, X.w}, xl[4] = {Xl.x, Xl.y, Xl.z, Xl.w};
-#pragma unroll
-  for (int k = 0; k < S; ++k) x[k] = ff(xs[k], xl[k]);
-}
-template <int S>
-__device__ __forceinline__ void load_x(const PassArgs& A, int64_t j, double x[S]) {
-#pragma unroll
-  for (int k = 0; k < S; ++k) x[k] = __ldg(&A.x[k * A.n + j]);
-}
-
-template <int S, int NL, typename R, typename Acc>
-__global__ void __launch_bounds__(256) k_pair_density(DevPot P, PassArgs A,
-                                                      const typename GeoRec<R>::T* __restrict__ buf, GeoLayout GL) {
-  if (A.ctrl != nullptr && A.ctrl->halted) return;
-  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t i = tid / NL;
-  const int lane = (int)(tid % NL);
-  const bool active = i < A.n;
-  Acc rb[S], ra[S];
-#pragma unroll
-  for (int k = 0; k < S; ++k) {
-    rb[k].zero();
-    ra[k].zero();
-  }
-  if (active) {
-    const int beg = A.nb_off[i], end = A.nb_off[i + 1];
-#pragma unroll 4
-    for (int t = beg + lane; t < end; t += NL) {
-      const int64_t j = __ldg(&A.nb_ent[t]) & kIdxMask;
-      const typename GeoRec<R>::T* rec = buf + (int64_t)t * GL.ca;  // densities: plane A
-      R xj[S];
-      load_x<S>(A, j, xj);
-#pragma unroll
-      for (int k = 0; k < S; ++k) {
-        R sb = (R)0, sa = (R)0;
-#pragma unroll
-        for (int l = 0; l < S; ++l) {
-          const int v = P.f_of[k][l];
-          if (v < 0) continue;
-          sb += xj[l] * GeoRec<R>::get(rec, v);
-          sa += xj[l] * GeoRec<R>::get(rec, P.n_f + v);
-        }
-        rb[k].add(sb);
-        ra[k].add(sa);
-      }
-    }
-  }
-  if (NL > 1) {
-#pragma unroll
-    for (int k = 0; k < S; ++k) {
-      rb[k].team_reduce(NL);
-      ra[k].team_reduce(NL);
-    }
-  }
-  // Per-site tail: team lane k < S takes species k (the FP64 square root and
-  // divisions then issue once per warp, not S times); the sums are those of
-  // team lane 0, so the result does not depend on which lane finishes it.
-  // Every lane reaches every shuffle.
-  static_assert(S <= 2 && NL >= S, "one team lane per species");
-  const int src = (int)(threadIdx.x & 31) - lane;
-  double rbar = 0.0, rsum = 0.0;
-#pragma unroll
-  for (int k = 0; k < S; ++k) {
-    const double wb = __shfl_sync(0xffffffffu, rb[k].get(), src);
-    const double wa = __shfl_sync(0xffffffffu, ra[k].get(), src);
-    if (lane == k) {
-      rbar = wb;
-      rsum = wa;
-    }
-  }
-  const int64_t n = A.n;
-  const bool mine = active && lane < S;
-  float abk = 0.f, bbk = 0.f, lak = 0.f, lbk = 0.f;
-  if (mine) {
-    const int k = lane;
-    const double Ek = (S > 1 && k == 1) ? P.E[S > 1 ? 1 : 0] : P.E[0];
-    const double ravg = rsum * (1.0 / 12.0);
-    const double xk = A.x[k * n + i];
-    double e = 0.0, ak = 0.0, bk = 0.0;
-    if (Ek == 0.0) {
-      // no embedding energy for this element
-    } else if (rbar > kRhoMin) {
-      const double sq = sqrt(rbar);
-      const double F = -Ek * sq;
-      const double dF = -Ek / (2.0 * sq);
-      const double d2F = Ek / (4.0 * rbar * sq);
-      e = F + dF * (ravg - rbar);
-      ak = xk * d2F * (ravg - rbar);
-      bk = xk * dF;
-    } else {
-      atomicOr(A.flags, kFlagGeometry);
-    }
-    A.rho_bar[k * n + i] = rbar;
-    A.rho_avg[k * n + i] = ravg;
-    A.e[k * n + i] = e;
-    A.a[k * n + i] = ak;
-    A.b[k * n + i] = bk;
-    abk = (float)ak;
-    bbk = (float)bk;
-    lak = (float)(ak - (double)abk);
-    lbk = (float)(bk - (double)bbk);
-  }
-  if (A.ab32 == nullptr) return;  // FP64 contexts: no packed records
-  // the packed FP32 (a, b) records of both species, written by team lane 0
-  float ab[4] = {abk, bbk, 0.f, 0.f}, lo[4] = {lak, lbk, 0.f, 0.f};
-  if (S > 1) {
-    ab[2] = __shfl_sync(0xffffffffu, abk, src + 1);
-    ab[3] = __shfl_sync(0xffffffffu, bbk, src + 1);
-    lo[2] = __shfl_sync(0xffffffffu, lak, src + 1);
-    lo[3] = __shfl_sync(0xffffffffu, lbk, src + 1);
-  }
-  if (!active || lane != 0) return;
-  A.ab32[2 * i] = make_float4(ab[0], ab[1], ab[2], ab[3]);
-  if (A.ab32lo) A.ab32lo[2 * i] = make_float4(lo[0], lo[1], lo[2], lo[3]);
-}
-
-template <int S, int NL, typename R, typename Acc>
-__global__ void __launch_bounds__(256) k_pair_mu(DevPot P, PassArgs A,
-                                                 const typename GeoRec<R>::T* __restrict__ buf, GeoLayout GL) {
-  constexpr int PR = GeoPrec<R>::P;
-  if (A.ctrl != nullptr && A.ctrl->halted) return;
-  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t i = tid / NL;
-  const int lane = (int)(tid % NL);
-  const bool active = i < A.n;
-  Acc mu[S], epair;
-  epair.zero();
-#pragma unroll
-  for (int k = 0; k < S; ++k) mu[k].zero();
-  if (active) {
-    R xi[S];
-    load_x<S>(A, i, xi);
-    const R inv12 = (R)(1.0 / 12.0);
-    const R half = (R)0.5;
-    const int beg = A.nb_off[i], end = A.nb_off[i + 1];
-    for (int t = beg + lane; t < end; t += NL) {
-      const int64_t j = __ldg(&A.nb_ent[t]) & kIdxMask;
-      const typename GeoRec<R>::T* rec = buf + (int64_t)t * GL.ca;
-      // pair terms: plane B when the record is split, else after the densities
-      const typename GeoRec<R>::T* recp = GL.cb ? buf + GL.b_off + (int64_t)t * GL.cb : rec + 2 * P.n_f;
-      R xj[S];
-      load_x<S>(A, j, xj);
-      R aj[S], bj[S];
-      load_ab(A, j, aj, bj, (SiteData<PR, S>*)nullptr);
-      R ep = (R)0;
-#pragma unroll
-      for (int k = 0; k < S; ++k) {
-        R m = (R)0;
-#pragma unroll
-        for (int l = 0; l < S; ++l) {
-          const int u = P.phi_of[k][l];
-          if (u >= 0) {
-            const R ph = GeoRec<R>::get(recp, u);
-            m += xj[l] * ph * inv12;
-            ep += xi[k] * xj[l] * ph;
-          }
-          // density at j of species l from this site holding species k: f_lk
-          const int v = P.f_of[l][k];
-          if (v >= 0) m += aj[l] * GeoRec<R>::get(rec, v) + bj[l] * GeoRec<R>::get(rec, P.n_f + v) * inv12;
-        }
-        mu[k].add(m);
-      }
-      epair.add(half * inv12 * ep);
-    }
-  }
-  if (NL > 1) {
-    epair.team_reduce(NL);
-#pragma unroll
-    for (int k = 0; k < S; ++k) mu[k].team_reduce(NL);
-  }
-  // Per-site tail on the first S + 2 team lanes, one FP64 logarithm each:
-  // lane k < S ln x_k (with the floor of the chemical potential), lane S
-  // ln x_v, lane S + 1 ln sigma; x ln x of the mixing entropy reuses them
-  // (a separate logarithm only for 0 < x below the floor).  The sums are
-  // those of team lane 0; every lane reaches every shuffle.
-  static_assert(NL >= S + 2, "one team lane per logarithm");
-  const int src = (int)(threadIdx.x & 31) - lane;
-  double mk = 0.0;
-#pragma unroll
-  for (int k = 0; k < S; ++k) {
-    const double w = __shfl_sync(0xffffffffu, mu[k].get(), src);
-    if (lane == k) mk = w;
-  }
-  const int64_t n = A.n;
-  double xk = 0.0, xv = 1.0;
-  if (active) {
-#pragma unroll
-    for (int k = 0; k < S; ++k) {
-      const double v = A.x[k * n + i];
-      xv -= v;
-      if (lane == k) xk = v;
-    }
-  }
-  double arg = 1.0;
-  if (active) {
-    if (lane < S) arg = fmax(xk, kLogFloor);
-    else if (lane == S) arg = fmax(xv, kLogFloor);
-    else if (lane == S + 1 && A.site_E) arg = A.sigma[i];
-  }
-  const double L = log(arg);
-  const double lv = __shfl_sync(0xffffffffu, L, src + S);
-  bool finite = true;
-  if (active && lane < S) {
-    const double kT = kKB * A.T[i];
-    const double m = mk + A.e[lane * n + i];
-    finite = isfinite(m);
-    if (A.mu_ex) A.mu_ex[lane * n + i] = m;
-    if (A.mu) A.mu[lane * n + i] = m + kT * (L - lv);
-  }
-  if (A.site_E) {
-    const double xs = lane < S ? xk : xv;
-    double t = 0.0;
-    if (active && lane <= S && xs > 0.0) t = xs * (xs >= kLogFloor ? L : log(xs));
-    double tk[S + 1];
-#pragma unroll
-    for (int k = 0; k <= S; ++k) tk[k] = __shfl_sync(0xffffffffu, t, src + k);
-    const double Ls = __shfl_sync(0xffffffffu, L, src + S + 1);
-    const double ept = __shfl_sync(0xffffffffu, epair.get(), src);
-    if (active && lane == 0) {
-      const double kT = kKB * A.T[i];
-      double mix = 0.0, emb = 0.0;
-#pragma unroll
-      for (int k = 0; k < S; ++k) {
-        const double x = A.x[k * n + i];
-        if (x > 0.0) mix += tk[k];
-        emb += x * A.e[k * n + i];
-      }
-      if (xv > 0.0) mix += tk[S];
-      const double EV = ept + emb;
-      const double Fv = -3.0 * kT * Ls;
-      const double Fm = kT * mix;
-      A.site_E[i] = EV;
-      A.site_E[n + i] = Fv;
-      A.site_E[2 * n + i] = Fm;
-      finite = finite && isfinite(EV) && isfinite(Fv) && isfinite(Fm);
-    }
-  }
-  if (!finite) atomicOr(A.flags, kFlagNonfinite);
-}
-
-// ---------------------------------------------------------------- half-list relaxation passes
-// The relaxation's density and force passes, each unordered pair evaluated
-// once (PREC 1, 2: FP32 node arithmetic, float4 records; PREC 0: FP64, records
-// of four doubles):
+// ---------------------------------------------------------------- half-list relaxation passes, direct FP64
+// FP64 contexts whose potential has no radial table (pair_table.cu otherwise;
+// the FP32 modes: pair_fp32.cu).  Each unordered pair once, records of doubles
+// summed by gathers.cu:
 //  k_pair_rdensity: f_v(r_ij) and the sum of f_v over the 12 nodes (both
 //    symmetric in i, j), weighted by the other site's fractions, written to
 //    both entries of the pair;
-//  k_gather_rdensity: per site the sums over its row (float-float in PREC 2,
-//    three floats in PREC 1, FP64 in PREC 0), then the embedding coefficients (a, b): packed FP32
-//    records (PREC 1, 2) or the FP64 arrays (PREC 0);
 //  k_pair_rforce: with the pair's weights (x, a, b of both sites) the force
 //    on the row-owner site i, F_i = -(d T + U / 12), d = q_j - q_i (the other
 //    site receives -F_i: the pair functions are symmetric), and the width
 //    derivatives of both sites (over the nodes that move i and those that
-//    move j), written to the two entries of the pair;
-//  k_gather_rforce: per site the sums over its row, then the thermal term.
-template <typename R>
-struct Rec4;
-template <>
-struct Rec4<float> {
-  using T = float4;
-  static __device__ __forceinline__ T make(float a, float b, float c, float d) { return make_float4(a, b, c, d); }
-  static __device__ __forceinline__ void load(const T* __restrict__ p, float v[4]) {
-    const float4 r = __ldg(p);
-    v[0] = r.x;
-    v[1] = r.y;
-    v[2] = r.z;
-    v[3] = r.w;
-  }
-};
-template <>
-struct Rec4<double> {
-  using T = Dbl4;
-  static __device__ __forceinline__ T make(double a, double b, double c, double d) { return Dbl4{a, b, c, d}; }
-  static __device__ __forceinline__ void load(const T* __restrict__ p, double v[4]) {
-    const double2* q = reinterpret_cast<const double2*>(p);
-    const double2 r0 = __ldg(q), r1 = __ldg(q + 1);
-    v[0] = r0.x;
-    v[1] = r0.y;
-    v[2] = r1.x;
-    v[3] = r1.y;
-  }
-};
-
-// value type of the relaxation records: the node arithmetic's
-template <int PREC>
-struct RelaxRec {
-  using V = typename Traits<PREC>::R;
-};
-
-// per-site sums of the relaxation gathers: float-float in PREC 2, three floats
-// in PREC 1 (FP32 records either way), FP64 in PREC 0.  PREC 1 with doubles in
-// both places: 58 and 56 us per gather at 55,296 sites, FP64-pipe bound
-template <int PREC>
-struct RelaxAcc {
-  using T = AccD;
-};
-template <>
-struct RelaxAcc<1> {
-  using T = AccT;
-};
-template <>
-struct RelaxAcc<2> {
-  using T = AccFF;
-};
-
+//    move j), written to the two entries of the pair.
 template <int PREC, int S, int TAB>
 __device__ __forceinline__ void pair_rdensity_one(const DevPot& P, const DevGrid& g0, const PassArgs& A,
                                                 const int4* __restrict__ pair_rec, int64_t p,
-                                                typename Rec4<typename RelaxRec<PREC>::V>::T* __restrict__ dens);
+                                                Dbl4* __restrict__ dens);
 
 // grid-stride over the unordered pairs (a resident grid: see resident_grid)
 template <int PREC, int S, int TAB>
 __global__ void __launch_bounds__(256) k_pair_rdensity(DevPot P, DevGrid g0, PassArgs A,
                                                        const int4* __restrict__ pair_rec, int64_t npair,
-                                                       typename Rec4<typename RelaxRec<PREC>::V>::T* __restrict__ dens) {
+                                                       Dbl4* __restrict__ dens) {
   pdl_wait();
   pdl_trigger();
   if (chunk_halted(A)) return;
@@ -1452,9 +1031,8 @@ __global__ void __launch_bounds__(256) k_pair_rdensity(DevPot P, DevGrid g0, Pas
 template <int PREC, int S, int TAB>
 __device__ __forceinline__ void pair_rdensity_one(const DevPot& P, const DevGrid& g0, const PassArgs& A,
                                                 const int4* __restrict__ pair_rec, int64_t p,
-                                                typename Rec4<typename RelaxRec<PREC>::V>::T* __restrict__ dens) {
+                                                Dbl4* __restrict__ dens) {
   using R = typename Traits<PREC>::R;
-  using RT = Rec4<typename RelaxRec<PREC>::V>;
   using TB = Tables<TAB>;
   constexpr int NF = S * S;
   PairRef pr_;
@@ -1528,114 +1106,28 @@ __device__ __forceinline__ void pair_rdensity_one(const DevPot& P, const DevGrid
           cj[2 + k] += si.x[l] * fav[w];
         }
     }
-  using RV = typename RelaxRec<PREC>::V;
-  dens[tp] = RT::make((RV)ci[0], (RV)ci[1], (RV)ci[2], (RV)ci[3]);
-  dens[tr] = RT::make((RV)cj[0], (RV)cj[1], (RV)cj[2], (RV)cj[3]);
-  if (bad) atomicOr(A.flags, kFlagGeometry);
-}
-
-template <int PREC, int S, int NL>
-__global__ void __launch_bounds__(256) k_gather_rdensity(DevPot P, PassArgs A,
-                                                         const typename Rec4<typename RelaxRec<PREC>::V>::T* __restrict__ dens) {
-  pdl_wait();
-  pdl_trigger();
-  using R = typename Traits<PREC>::R;
-  using Acc = typename RelaxAcc<PREC>::T;
-  if (A.ctrl != nullptr && A.ctrl->halted) return;
-  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t i = tid / NL;
-  const int lane = (int)(tid % NL);
-  const bool active = i < A.n;
-  Acc rb[S], ra[S];
-#pragma unroll
-  for (int k = 0; k < S; ++k) {
-    rb[k].zero();
-    ra[k].zero();
-  }
-  if (active) {
-    const int beg = A.nb_off[i], end = A.nb_off[i + 1];
-#pragma unroll 4
-    for (int t = beg + lane; t < end; t += NL) {
-      typename RelaxRec<PREC>::V rec[4];
-      Rec4<typename RelaxRec<PREC>::V>::load(&dens[t], rec);
-      rb[0].add(rec[0]);
-      ra[0].add(rec[2]);
-      if (S > 1) {
-        rb[S > 1 ? 1 : 0].add(rec[1]);
-        ra[S > 1 ? 1 : 0].add(rec[3]);
-      }
-    }
-  }
-  if (NL > 1) {
-#pragma unroll
-    for (int k = 0; k < S; ++k) {
-      rb[k].team_reduce(NL);
-      ra[k].team_reduce(NL);
-    }
-  }
-  if (!active || lane != 0) return;
-  int flag = 0;
-  const int64_t n = A.n;
-  if constexpr (PREC == 0) {
-    // FP64 embedding coefficients, as the FP64 density pass forms them
-#pragma unroll
-    for (int k = 0; k < S; ++k) {
-      const double rbar = rb[k].get();
-      const double ravg = ra[k].get() * (1.0 / 12.0);
-      const double xk = A.x[k * n + i];
-      double ak = 0.0, bk = 0.0;
-      if (P.E[k] == 0.0) {
-        // no embedding energy for this element
-      } else if (rbar > kRhoMin) {
-        const double sq = sqrt(rbar);
-        const double dF = -P.E[k] / (2.0 * sq);
-        const double d2F = P.E[k] / (4.0 * rbar * sq);
-        ak = xk * d2F * (ravg - rbar);
-        bk = xk * dF;
-      } else {
-        flag |= kFlagGeometry;
-      }
-      A.a[k * n + i] = ak;
-      A.b[k * n + i] = bk;
-    }
+  if constexpr (S == 1 || TAB == 1) {  // one density for every species
+    double2* d2 = reinterpret_cast<double2*>(dens);
+    d2[tp] = make_double2(ci[0], ci[2]);
+    d2[tr] = make_double2(cj[0], cj[2]);
   } else {
-    float ab[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    const float4 X = A.x32[i];
-    const float xs[4] = {X.x, X.y, X.z, X.w};
-#pragma unroll
-    for (int k = 0; k < S; ++k) {
-      const float2 b2 = rb[k].get_pair(), a2 = ra[k].get_pair();
-      const float rf = b2.x + b2.y;
-      const float df = fmaf(a2.x, 1.0f / 12.0f, -b2.x) + fmaf(a2.y, 1.0f / 12.0f, -b2.y);
-      if (P.E[k] == 0.0) {
-        // no embedding energy for this element
-      } else if (rf > (float)kRhoMin) {
-        const float Ef = (float)P.E[k];
-        const float isq = rsqrt_approx(rf);
-        const float dF = -0.5f * Ef * isq;
-        const float d2F = 0.25f * Ef * isq * isq * isq;
-        ab[2 * k] = xs[k] * d2F * df;
-        ab[2 * k + 1] = xs[k] * dF;
-      } else {
-        flag |= kFlagGeometry;
-      }
-    }
-    A.ab32[2 * i] = make_float4(ab[0], ab[1], ab[2], ab[3]);
+    dens[tp] = Dbl4{ci[0], ci[1], ci[2], ci[3]};
+    dens[tr] = Dbl4{cj[0], cj[1], cj[2], cj[3]};
   }
-  if (flag) atomicOr(A.flags, flag);
+  if (bad) atomicOr(A.flags, kFlagGeometry);
 }
 
 template <int PREC, int S, int TAB>
 __device__ __forceinline__ void pair_rforce_one(const DevPot& P, const DevGrid& g0, const PassArgs& A,
                                                 const int4* __restrict__ pair_rec, int64_t p,
-                                                typename Rec4<typename RelaxRec<PREC>::V>::T* __restrict__ frc);
+                                                Dbl4* __restrict__ frc);
 
 // one thread per unordered pair (a grid-stride loop here held 48 registers
 // against 40 and ran 9 % slower)
 template <int PREC, int S, int TAB>
 __global__ void __launch_bounds__(256) k_pair_rforce(DevPot P, DevGrid g0, PassArgs A,
                                                        const int4* __restrict__ pair_rec, int64_t npair,
-                                                       typename Rec4<typename RelaxRec<PREC>::V>::T* __restrict__ frc) {
+                                                       Dbl4* __restrict__ frc) {
   pdl_wait();
   pdl_trigger();
   if (A.ctrl != nullptr && A.ctrl->halted) return;
@@ -1646,9 +1138,8 @@ __global__ void __launch_bounds__(256) k_pair_rforce(DevPot P, DevGrid g0, PassA
 template <int PREC, int S, int TAB>
 __device__ __forceinline__ void pair_rforce_one(const DevPot& P, const DevGrid& g0, const PassArgs& A,
                                                 const int4* __restrict__ pair_rec, int64_t p,
-                                                typename Rec4<typename RelaxRec<PREC>::V>::T* __restrict__ frc) {
+                                                Dbl4* __restrict__ frc) {
   using R = typename Traits<PREC>::R;
-  using RT = Rec4<typename RelaxRec<PREC>::V>;
   using TB = Tables<TAB>;
   constexpr int NF = S * S;
   constexpr int NP = S * (S + 1) / 2;
@@ -1779,74 +1270,8 @@ __device__ __forceinline__ void pair_rforce_one(const DevPot& P, const DevGrid& 
   // this entry: the force on i and its width derivative; the reverse entry:
   // the force on j (Newton's third law) and j's width derivative
   const R Fx = -(d[0] * Tt + U[0] * inv12), Fy = -(d[1] * Tt + U[1] * inv12), Fz = -(d[2] * Tt + U[2] * inv12);
-  using RV = typename RelaxRec<PREC>::V;
-  const RV fx = (RV)Fx, fy = (RV)Fy, fz = (RV)Fz;
-  frc[tp] = RT::make(fx, fy, fz, (RV)(Vs[0] * inv12));
-  frc[tr] = RT::make(-fx, -fy, -fz, (RV)(Vs[1] * inv12));
-}
-
-template <int PREC, int S, int NL>
-__global__ void __launch_bounds__(256) k_gather_rforce(PassArgs A,
-                                                       const typename Rec4<typename RelaxRec<PREC>::V>::T* __restrict__ frc) {
-  pdl_wait();
-  pdl_trigger();
-  using R = typename Traits<PREC>::R;
-  using Acc = typename RelaxAcc<PREC>::T;
-  if (A.ctrl != nullptr && A.ctrl->halted) return;
-  const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t i = tid / NL;
-  const int lane = (int)(tid % NL);
-  const bool active = i < A.n;
-  Acc g[3], gsig;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) g[c].zero();
-  gsig.zero();
-  if (active) {
-    const int beg = A.nb_off[i], end = A.nb_off[i + 1];
-#pragma unroll 4
-    for (int t = beg + lane; t < end; t += NL) {
-      typename RelaxRec<PREC>::V f[4];
-      Rec4<typename RelaxRec<PREC>::V>::load(&frc[t], f);
-      g[0].add(f[0]);
-      g[1].add(f[1]);
-      g[2].add(f[2]);
-      gsig.add(f[3]);
-    }
-  }
-  if (NL > 1) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) g[c].team_reduce(NL);
-    gsig.team_reduce(NL);
-  }
-  // Per-site tail: team lanes 0-2 the force components, lane 3 the width
-  // derivative with its thermal term, so the conversions and the FP64 division
-  // issue once per warp.  After the butterfly every team lane holds the whole
-  // sum (a lane's own rounding order: fixed, so runs repeat exactly).
-  static_assert(NL >= 4, "one team lane per output");
-  if (!active || lane > 3) return;
-  const int64_t n = A.n;
-  double v;
-  if constexpr (PREC == 0) {
-    v = lane == 0 ? g[0].get() : lane == 1 ? g[1].get() : lane == 2 ? g[2].get()
-                  : gsig.get() - 3.0 * kKB * A.T[i] / A.sigma[i];
-  } else {
-    float2 h = g[0].get_pair();
-    if (lane == 1) h = g[1].get_pair();
-    else if (lane == 2) h = g[2].get_pair();
-    else if (lane == 3) {
-      // FP32 modes: the thermal term in FP32 (no FP64 division)
-      const float2 gp = gsig.get_pair();
-      const float th = 3.0f * (float)kKB * (float)A.T[i] / (float)A.sigma[i];
-      h = make_float2((gp.x - th) + gp.y, 0.f);
-    }
-    v = (double)h.x + (double)h.y;
-  }
-  if (lane < 3) {
-    if (A.gq) A.gq[lane * n + i] = v;
-  } else if (A.gs) {
-    A.gs[i] = v;
-  }
-  if (!isfinite(v)) atomicOr(A.flags, kFlagNonfinite);
+  frc[tp] = Dbl4{Fx, Fy, Fz, Vs[0] * inv12};
+  frc[tr] = Dbl4{-Fx, -Fy, -Fz, Vs[1] * inv12};
 }
 
 // ---------------------------------------------------------------- exact embedding average
@@ -2399,7 +1824,7 @@ __global__ void __launch_bounds__(256) k_emb_grad(DevPot P, DevGrid g0, PassArgs
 __global__ void k_pack(const double* __restrict__ q, const double* __restrict__ sigma, const double* __restrict__ x,
                        const int* __restrict__ abs_cell, int64_t n, int S, DevGrid g0, Batch B,
                        float4* __restrict__ pos32, float4* __restrict__ x32, float4* __restrict__ pos32lo,
-                       float4* __restrict__ x32lo) {
+                       float4* __restrict__ srec, int srec_len) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   const DevGrid g = site_grid(g0, B, i);
@@ -2421,10 +1846,8 @@ __global__ void k_pack(const double* __restrict__ q, const double* __restrict__ 
     xl[k] = (float)(xv - (double)xs[k]);
   }
   x32[i] = make_float4(xs[0], xs[1], xs[2], xs[3]);
-  if (pos32lo) {
-    pos32lo[i] = make_float4(pl[0], pl[1], pl[2], pl[3]);
-    x32lo[i] = make_float4(xl[0], xl[1], xl[2], xl[3]);
-  }
+  if (pos32lo) pos32lo[i] = make_float4(pl[0], pl[1], pl[2], pl[3]);
+  if (srec) srec[i * (srec_len / 2)] = make_float4(xs[0], xl[0], xs[1], xl[1]);
 }
 
 // FP64 embedding coefficients -> the packed FP32 records the FP32 gradient pass gathers
@@ -2530,10 +1953,7 @@ cudaError_t launch_gradient_t(int mode, const DevPot& P, const DevGrid& g, const
   const int threads = a.tpb > 0 ? a.tpb : 256;
   const int64_t work = a.n * NL;
   const unsigned blocks = (unsigned)((work + threads - 1) / threads);
-  if constexpr (PREC == 3) {  // float-float: chemical potentials and energies only
-    if (mode != kGradMu) return cudaErrorInvalidValue;
-    k_gradient<3, S, NL, kGradMu><<<blocks, threads, 0, s>>>(P, g, a);
-  } else if constexpr (PREC == 0) {
+  if constexpr (PREC == 0) {
     if (mode == kGradForce)
       k_gradient<0, S, NL, kGradForce><<<blocks, threads, 0, s>>>(P, g, a);
     else if (mode == kGradForceNoE)
@@ -2582,7 +2002,6 @@ cudaError_t dispatch(int mode, int precision, int nl, const DevPot& P, const Dev
     case 0: return dispatch_s<0>(mode, nl, P, g, a, s);
     case 1: return dispatch_s<1>(mode, nl, P, g, a, s);
     case 2: return dispatch_s<2>(mode, nl, P, g, a, s);
-    case 3: return dispatch_s<3>(mode, nl, P, g, a, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -2591,9 +2010,10 @@ cudaError_t dispatch(int mode, int precision, int nl, const DevPot& P, const Dev
 
 cudaError_t launch_pack(const double* q, const double* sigma, const double* x, const int* abs_cell, int64_t n,
                         int S, const DevGrid& g, const Batch& B, float4* pos32, float4* x32, float4* pos32lo,
-                        float4* x32lo, cudaStream_t s) {
+                        void* srec, int srec_len, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  k_pack<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(q, sigma, x, abs_cell, n, S, g, B, pos32, x32, pos32lo, x32lo);
+  k_pack<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(q, sigma, x, abs_cell, n, S, g, B, pos32, x32, pos32lo,
+                                                     (float4*)srec, srec_len);
   return cudaGetLastError();
 }
 
@@ -2627,17 +2047,14 @@ cudaError_t launch_energy_seg(const double* site_E, int64_t n, const Batch& B, d
   return cudaGetLastError();
 }
 
-namespace {
-bool geo_split(const DevPot& P) { return 2 * P.n_f + P.n_phi > 4; }
-}  // namespace
 int pair_record_len(const DevPot& P) {
-  if (geo_split(P)) return ((2 * P.n_f + 3) & ~3) + ((P.n_phi + 3) & ~3);
-  return (2 * P.n_f + P.n_phi + 3) & ~3;
+  const GeoLayout L = geo_layout(P, 0);
+  return L.ca + L.cb;
 }
 GeoLayout geo_layout(const DevPot& P, int64_t cap) {
-  if (!geo_split(P)) return GeoLayout{pair_record_len(P), 0, 0};
-  const int ca = (2 * P.n_f + 3) & ~3;
-  return GeoLayout{ca, (P.n_phi + 3) & ~3, cap * ca};
+  // even counts (16-byte loads), or the single pair term of one species
+  const int ca = 2 * P.n_f, cb = P.n_phi == 1 ? 1 : (P.n_phi + 1) & ~1;
+  return GeoLayout{ca, cb, cap * ca};
 }
 
 // threads per block of the pair kernels: the unordered pairs one block takes
@@ -2676,78 +2093,10 @@ cudaError_t launch_pair_geo(int precision, const DevPot& P, const DevGrid& g, co
 }
 
 namespace {
-template <int S, int NL, typename R, typename Acc>
-cudaError_t pair_gather_t(bool mu, const DevPot& P, const PassArgs& A, const void* buf, GeoLayout C, cudaStream_t s) {
-  const int threads = A.tpb > 0 ? A.tpb : 256;
-  const unsigned blocks = (unsigned)((A.n * NL + threads - 1) / threads);
-  using T = typename GeoRec<R>::T;
-  if (mu) k_pair_mu<S, NL, R, Acc><<<blocks, threads, 0, s>>>(P, A, (const T*)buf, C);
-  else k_pair_density<S, NL, R, Acc><<<blocks, threads, 0, s>>>(P, A, (const T*)buf, C);
-  return cudaGetLastError();
-}
-template <int S, int NL>
-cudaError_t pair_gather_p(int precision, bool mu, const DevPot& P, const PassArgs& A, const void* buf, GeoLayout C,
-                          cudaStream_t s) {
-  switch (precision) {
-    case 0: return pair_gather_t<S, NL, double, AccD>(mu, P, A, buf, C, s);
-    case 1: return pair_gather_t<S, NL, ff, AccT>(mu, P, A, buf, C, s);
-    case 2: return pair_gather_t<S, NL, ff, AccF2>(mu, P, A, buf, C, s);
-    default: return cudaErrorInvalidValue;
-  }
-}
-template <int S>
-cudaError_t pair_gather_s(int precision, bool mu, int nl, const DevPot& P, const PassArgs& A, const void* buf, GeoLayout C,
-                          cudaStream_t s) {
-  switch (nl) {
-    case 4: return pair_gather_p<S, 4>(precision, mu, P, A, buf, C, s);
-    case 8: return pair_gather_p<S, 8>(precision, mu, P, A, buf, C, s);
-    case 16: return pair_gather_p<S, 16>(precision, mu, P, A, buf, C, s);
-    default: return cudaErrorInvalidValue;
-  }
-}
-}  // namespace
-
-cudaError_t launch_pair_gather(int precision, bool mu, int nl, const DevPot& P, const PassArgs& A, const void* buf,
-                               int64_t cap, cudaStream_t s) {
-  if (A.n == 0) return cudaSuccess;
-  const GeoLayout C = geo_layout(P, cap);
-  switch (P.S) {
-    case 1: return pair_gather_s<1>(precision, mu, nl, P, A, buf, C, s);
-    case 2: return pair_gather_s<2>(precision, mu, nl, P, A, buf, C, s);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-namespace {
-template <int PREC, int S, int NL>
-cudaError_t relax_gather_t(bool force, const DevPot& P, const PassArgs& A, const void* dens, const void* frc,
-                           cudaStream_t s) {
-  using T = typename Rec4<typename RelaxRec<PREC>::V>::T;
-  const int threads = A.tpb > 0 ? A.tpb : 256;
-  const unsigned blocks = (unsigned)((A.n * NL + threads - 1) / threads);
-  if (force) return launch_pdl(k_gather_rforce<PREC, S, NL>, dim3(blocks), dim3(threads), 0, s, A, (const T*)frc);
-  return launch_pdl(k_gather_rdensity<PREC, S, NL>, dim3(blocks), dim3(threads), 0, s, P, A, (const T*)dens);
-}
-template <int PREC, int S>
-cudaError_t relax_gather_s(bool force, int nl, const DevPot& P, const PassArgs& A, const void* dens, const void* frc,
-                           cudaStream_t s) {
-  switch (nl) {
-    case 4: return relax_gather_t<PREC, S, 4>(force, P, A, dens, frc, s);
-    case 8: return relax_gather_t<PREC, S, 8>(force, P, A, dens, frc, s);
-    case 16: return relax_gather_t<PREC, S, 16>(force, P, A, dens, frc, s);
-    default: return cudaErrorInvalidValue;
-  }
-}
-template <int PREC>
-cudaError_t relax_gather_p(bool force, int nl, const DevPot& P, const PassArgs& A, const void* dens, const void* frc,
-                           cudaStream_t s) {
-  if (P.S == 1) return relax_gather_s<PREC, 1>(force, nl, P, A, dens, frc, s);
-  return relax_gather_s<PREC, 2>(force, nl, P, A, dens, frc, s);
-}
 template <int PREC>
 cudaError_t relax_pair_p(bool force, const DevPot& P, const DevGrid& g, const PassArgs& A, const int4* pair_rec,
                          int64_t npair, void* dens, void* frc, cudaStream_t s) {
-  using T = typename Rec4<typename RelaxRec<PREC>::V>::T;
+  using T = Dbl4;
   const int pt = pair_threads(A);
   // the density pass strides over a resident grid in a single system; the
   // force pass, and every pass of a batch (a stride would take each thread
@@ -2842,18 +2191,6 @@ cudaError_t launch_relax_pair(int precision, bool force, const DevPot& P, const 
     case 0: return relax_pair_p<0>(force, P, g, A, pair_rec, npair, dens, frc, s);
     case 1:
     case 2: return launch_relax_pair32(force, P, g, A, pair_rec, npair, force ? frc : dens, s);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-cudaError_t launch_relax_gather(int precision, bool force, int nl, const DevPot& P, const PassArgs& A,
-                                const void* dens, const void* frc, cudaStream_t s) {
-  if (A.n == 0) return cudaSuccess;
-  if (!pair_kernels_supported(P)) return cudaErrorInvalidValue;
-  switch (precision) {
-    case 0: return relax_gather_p<0>(force, nl, P, A, dens, frc, s);
-    case 1: return relax_gather_p<1>(force, nl, P, A, dens, frc, s);
-    case 2: return relax_gather_p<2>(force, nl, P, A, dens, frc, s);
     default: return cudaErrorInvalidValue;
   }
 }

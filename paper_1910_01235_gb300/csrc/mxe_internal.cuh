@@ -267,10 +267,11 @@ cudaError_t launch_site_max(const double* sigma, const double* q, int64_t n, uns
                             cudaStream_t s);
 
 // eam.cu
-// pos32/x32: FP32 records; pos32lo/x32lo (optional): the float-pair remainders
+// pos32/x32: FP32 records; pos32lo (optional): the float-pair remainders of
+// pos32; srec (optional): the x part of the site records (float pairs)
 cudaError_t launch_pack(const double* q, const double* sigma, const double* x, const int* abs_cell, int64_t n,
                         int S, const DevGrid& g, const Batch& B, float4* pos32, float4* x32, float4* pos32lo,
-                        float4* x32lo, cudaStream_t s);
+                        void* srec, int srec_len, cudaStream_t s);
 cudaError_t init_ff_exp_table();
 struct PassArgs {
   const double* q;
@@ -279,20 +280,17 @@ struct PassArgs {
   const double* T;
   const float4* pos32;
   const float4* x32;
-  const float4* pos32lo;  // float-float passes: remainders of pos32, x32, ab32
-  const float4* x32lo;
+  const float4* pos32lo;  // direct float-float pass: remainders of pos32
   const int* nb_off;
   const uint32_t* nb_ent;
   int64_t n;
   int64_t n_ent;    // neighbour entries of the list (bound of every entry index)
   // pass-1 outputs / pass-2 inputs
-  double* rho_bar;
-  double* rho_avg;
   double* a;
   double* b;
   double* e;
   float4* ab32;     // [n][2] packed (a_k, b_k) for the mixed pass-2 gathers
-  float4* ab32lo;
+  void* srec;       // [n] site records of the accurate gathers (site_record_len values)
   // pass-2 outputs
   double* gq;
   double* gs;
@@ -318,11 +316,11 @@ cudaError_t launch_gradient(int precision, int mode, int nl, const DevPot& P, co
 // the density (mu = false) or chemical-potential gather over each site's own
 // row (per-site sums in float-float for MXE_FP32_FF, FP64 otherwise).  Record
 // components [0, 2 n_f) (the densities) and [2 n_f, 2 n_f + n_phi) (the pair
-// terms) lie in two planes when they do not fit one 32-byte group: plane A
-// [cap][ca] at buf, plane B [cap][cb] at buf + b_off (cap: entries allocated),
-// so that the density gather reads plane A only.
+// terms) lie in two planes: plane A [cap][ca] at buf, plane B [cap][cb] at
+// buf + b_off (cap: entries allocated), so that the density gather reads plane
+// A only.
 struct GeoLayout {
-  int ca, cb;      // values per entry in plane A and plane B (cb 0: one plane)
+  int ca, cb;      // values per entry in plane A and plane B
   int64_t b_off;   // plane B's first value
 };
 int pair_record_len(const DevPot& P);
@@ -342,6 +340,9 @@ cudaError_t launch_relax_tab(bool force, const DevPot& P, const DevGrid& g, cons
                              const int4* pair_rec, int64_t npair, void* out, cudaStream_t s);
 cudaError_t launch_pair_geo(int precision, const DevPot& P, const DevGrid& g, const PassArgs& A,
                             const int4* pair_rec, int64_t npair, void* buf, int64_t cap, cudaStream_t s);
+// values per site of PassArgs::srec (gathers.cu): x of both species, then the
+// embedding coefficients a, b of every distinct density
+int site_record_len(const DevPot& P);
 cudaError_t launch_pair_gather(int precision, bool mu, int nl, const DevPot& P, const PassArgs& A, const void* buf,
                                int64_t cap, cudaStream_t s);
 // half-list relaxation passes (FP32 node math in the FP32 modes, FP64 in FP64

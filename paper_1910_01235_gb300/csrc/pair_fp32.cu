@@ -219,8 +219,14 @@ __global__ void __launch_bounds__(256) k_rdensity32(const __grid_constant__ Pot3
             cj[2 + k] += si.x[l] * fa;
           }
       }
-    dens[pr.tp] = make_float4(ci[0], ci[1], ci[2], ci[3]);
-    dens[pr.tr] = make_float4(cj[0], cj[1], cj[2], cj[3]);
+    if constexpr (S == 1 || TAB != 0) {  // one density for every species
+      float2* d2 = reinterpret_cast<float2*>(dens);
+      d2[pr.tp] = make_float2(ci[0], ci[2]);
+      d2[pr.tr] = make_float2(cj[0], cj[2]);
+    } else {
+      dens[pr.tp] = make_float4(ci[0], ci[1], ci[2], ci[3]);
+      dens[pr.tr] = make_float4(cj[0], cj[1], cj[2], cj[3]);
+    }
     if (bad) atomicOr(A.flags, kFlagGeometry);
   }
 }

@@ -255,28 +255,24 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_geo_tab(
       for (int u = 0; u < NP; ++u)
         if (u < P.n_phi) val[2 * NF + u] = O::from(ph[u]);
     }
-    if (P.n_f == NF && (NF == 2 ? (L.ca == 4 && L.cb == 4) : (L.ca == 4 && L.cb == 0))) {
-      // 16-byte stores: plane A of each entry, and plane B (two species)
-      const uint4 v0 = O::two(val[0], val[1]), v1 = O::two(val[2], val[3]);
-      uint4* oa = reinterpret_cast<uint4*>(buf + (int64_t)pr.tp * 4);
-      uint4* oa2 = reinterpret_cast<uint4*>(buf + (int64_t)pr.tr * 4);
-      oa[0] = v0;
-      oa[1] = v1;
-      oa2[0] = v0;
-      oa2[1] = v1;
-      if constexpr (NF == 2) {
-        const uint4 v2 = O::two(val[4], val[5]), v3 = O::two(val[6], val[7]);
-        uint4* ob = reinterpret_cast<uint4*>(buf + L.b_off + (int64_t)pr.tp * 4);
-        uint4* ob2 = reinterpret_cast<uint4*>(buf + L.b_off + (int64_t)pr.tr * 4);
-        ob[0] = v2;
-        ob[1] = v3;
-        ob2[0] = v2;
-        ob2[1] = v3;
+    if (P.n_f == NF && P.n_phi == NP) {
+      // 16-byte stores to plane A of each entry, then plane B
+      uint4* oa = reinterpret_cast<uint4*>(buf + (int64_t)pr.tp * L.ca);
+      uint4* oa2 = reinterpret_cast<uint4*>(buf + (int64_t)pr.tr * L.ca);
+      typename O::T *ob = buf + L.b_off + (int64_t)pr.tp * L.cb, *ob2 = buf + L.b_off + (int64_t)pr.tr * L.cb;
+#pragma unroll
+      for (int v = 0; v < NF; ++v) oa[v] = oa2[v] = O::two(val[2 * v], val[2 * v + 1]);
+      if constexpr (NP == 1) {
+        *ob = *ob2 = O::put(val[2 * NF]);
+      } else {
+#pragma unroll
+        for (int u = 0; u < (NP + 1) / 2; ++u)
+          reinterpret_cast<uint4*>(ob)[u] = reinterpret_cast<uint4*>(ob2)[u] =
+              O::two(val[2 * NF + 2 * u], val[2 * NF + 2 * u + 1]);
       }
     } else {
       typename O::T *oa = buf + (int64_t)pr.tp * L.ca, *oa2 = buf + (int64_t)pr.tr * L.ca;
-      typename O::T *ob = L.cb ? buf + L.b_off + (int64_t)pr.tp * L.cb : oa + 2 * P.n_f;
-      typename O::T *ob2 = L.cb ? buf + L.b_off + (int64_t)pr.tr * L.cb : oa2 + 2 * P.n_f;
+      typename O::T *ob = buf + L.b_off + (int64_t)pr.tp * L.cb, *ob2 = buf + L.b_off + (int64_t)pr.tr * L.cb;
 #pragma unroll
       for (int v = 0; v < NF; ++v)
         if (v < P.n_f) {
@@ -363,8 +359,14 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_rdensity_tab(
           }
       }
     }
-    dens[pr.tp] = Dbl4{ci[0], ci[1], ci[2], ci[3]};
-    dens[pr.tr] = Dbl4{cj[0], cj[1], cj[2], cj[3]};
+    if constexpr (S == 1 || TAB == 1) {  // one density for every species
+      double2* d2 = reinterpret_cast<double2*>(dens);
+      d2[pr.tp] = make_double2(ci[0], ci[2]);
+      d2[pr.tr] = make_double2(cj[0], cj[2]);
+    } else {
+      dens[pr.tp] = Dbl4{ci[0], ci[1], ci[2], ci[3]};
+      dens[pr.tr] = Dbl4{cj[0], cj[1], cj[2], cj[3]};
+    }
   }
 }
 
