@@ -510,7 +510,7 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
   cudaStream_t st = c->stream;
   c->have_list = false;
   // max sigma -> r_list; max |q| -> error band of the FP32 prefilter
-  CK(cudaMemsetAsync(c->smax_bits, 0, 2 * sizeof(unsigned long long), st));
+  CK(cudaMemsetAsync(c->smax_bits, 0, 4 * sizeof(unsigned long long), st));  // and max_row
   CK(TIMED("build_misc", launch_site_max(s->sigma, s->q, n, c->smax_bits, st)));
   CK(cudaMemcpyAsync(c->bits_h, c->smax_bits, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
@@ -580,7 +580,7 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
   // cell lists
   CK(cudaMemsetAsync(c->cell_count, 0, sizeof(int) * ncell, st));
   CK(TIMED("build_misc", launch_cell_assign(s->q, n, g, B, c->cell_of, c->cell_slot, c->cell_count, c->abs_cell, c->qf, st)));
-  CK(TIMED("build_misc", launch_scan(c->cell_count, c->cell_start, ncell, c->totals + 0, (int*)c->scan_tmp, c->scan_len, st)));
+  CK(TIMED("build_misc", launch_scan(ScanJobs{{c->cell_count}, {c->cell_start}, {c->totals}}, 1, ncell, c->scan_tmp, c->scan_len, st)));
   CK(TIMED("build_misc", launch_cell_place(n, c->cell_of, c->cell_slot, c->cell_start, c->cell_sites, st)));
   // largest stencil candidate set: the cell-staged kernels hold it in shared
   // memory.  A rebuild that can skip the count pass (the previous build's
@@ -588,7 +588,6 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
   // stencil plus a fifth and checks the true size, computed on the device
   // meanwhile, together with the totals: a larger stencil discards that fill
   // (count + fill instead).  Otherwise the host waits for the size here.
-  CK(cudaMemsetAsync(c->max_row, 0, 3 * sizeof(int), st));
   CK(TIMED("build_misc", launch_cand_max(ncell, g, B, c->cell_start, c->max_row + 1, st)));
   // MXE_NEIGHBOR_PER_SITE forces the warp-per-site kernels (they are the
   // fallback for stencils too dense for shared memory; tests compare both)
@@ -607,6 +606,9 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
   // counts: from a fill at a fixed stride when the previous build's longest row
   // bounds it (no count pass), else a count pass before the fill
   const double rl2 = r_list * r_list, rb2 = r_bond * r_bond;
+  const ScanJobs rows_scan{{c->nb_cnt, c->bd_cnt, c->pair_cnt},
+                           {c->nb_off, c->bd_off, c->pair_off},
+                           {c->totals + 1, c->totals + 2, c->totals + 3}};
   bool direct = false;
   int stride = 0;
   if (staged && try_direct) {
@@ -628,10 +630,7 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
                                                    stride, c->rows_tmp, c->brows_tmp, c->nb_cnt, c->bd_cnt,
                                                    pi ? c->n_below : nullptr, pi ? c->pair_cnt : nullptr,
                                                    c->max_row, c->max_row + 2, st)));
-    CK(TIMED("build_misc", launch_scan(c->nb_cnt, c->nb_off, n, c->totals + 1, (int*)c->scan_tmp, c->scan_len, st)));
-    CK(TIMED("build_misc", launch_scan(c->bd_cnt, c->bd_off, n, c->totals + 2, (int*)c->scan_tmp, c->scan_len, st)));
-    if (pi)
-      CK(TIMED("build_misc", launch_scan(c->pair_cnt, c->pair_off, n, c->totals + 3, (int*)c->scan_tmp, c->scan_len, st)));
+    CK(TIMED("build_misc", launch_scan(rows_scan, pi ? 3 : 2, n, c->scan_tmp, c->scan_len, st)));
     CK(cudaMemcpyAsync(c->totals_h, c->totals, sizeof(long long) * 4, cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(c->ints_h, c->max_row, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -665,8 +664,7 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
                                              c->max_row, st)));
   }
   if (!direct) {
-    CK(TIMED("build_misc", launch_scan(c->nb_cnt, c->nb_off, n, c->totals + 1, (int*)c->scan_tmp, c->scan_len, st)));
-    CK(TIMED("build_misc", launch_scan(c->bd_cnt, c->bd_off, n, c->totals + 2, (int*)c->scan_tmp, c->scan_len, st)));
+    CK(TIMED("build_misc", launch_scan(rows_scan, 2, n, c->scan_tmp, c->scan_len, st)));
     CK(cudaMemcpyAsync(c->totals_h, c->totals, sizeof(long long) * 3, cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(c->ints_h, c->max_row, sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -724,7 +722,8 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
     // total came with the list's); otherwise count them from the rows.
     if (!direct) {
       CK(TIMED("build_misc", launch_pair_count(c->nb_off, c->nb_ent, n, c->n_below, c->pair_cnt, st)));
-      CK(TIMED("build_misc", launch_scan(c->pair_cnt, c->pair_off, n, c->totals + 3, (int*)c->scan_tmp, c->scan_len, st)));
+      CK(TIMED("build_misc", launch_scan(ScanJobs{{c->pair_cnt}, {c->pair_off}, {c->totals + 3}}, 1, n, c->scan_tmp,
+                                            c->scan_len, st)));
       CK(cudaMemcpyAsync(c->totals_h + 3, c->totals + 3, sizeof(long long), cudaMemcpyDeviceToHost, st));
       CK(cudaStreamSynchronize(st));
     }
@@ -1472,8 +1471,9 @@ mxe_status mxe_create_batch(mxe_ctx** out, int32_t n_systems, const mxe_box* box
   A(dalloc(&c->nb_off, n + 1));
   A(dalloc(&c->bd_off, n + 1));
   A(dalloc(&c->totals, 4));
-  A(dalloc(&c->max_row, 4));  // longest row, largest stencil, flags of a fill that may be discarded
-  A(dalloc(&c->smax_bits, 2));
+  A(dalloc(&c->smax_bits, 4));  // maxima of sigma and |q|, then max_row
+  // longest row, largest stencil, flags of a fill that may be discarded
+  c->max_row = c->smax_bits ? reinterpret_cast<int*>(c->smax_bits + 2) : nullptr;
   A(dalloc(&c->qf, 2 * n));
   A(dalloc(&c->q_build, 3 * n));
   A(dalloc(&c->a, S * n));
@@ -1505,7 +1505,7 @@ mxe_status mxe_create_batch(mxe_ctx** out, int32_t n_systems, const mxe_box* box
   A(dalloc(&c->x_new, S * n));
   A(dalloc(&c->flux_tmp, flux_scratch_len(n, (int)S)));
   A(dalloc(&c->mu_eff, S * n));
-  A(dalloc(&c->flags, 1));
+  A(dalloc(&c->flags, 2));  // status bits, ticket of the energy sums
   A(dalloc(&c->step_flags, 1));
   A(dalloc(&c->ctrl, 1));
   A(cudaMallocHost((void**)&c->ctrl_h, sizeof(Ctrl)));
@@ -1543,7 +1543,7 @@ mxe_status mxe_create_batch(mxe_ctx** out, int32_t n_systems, const mxe_box* box
     c->B.cell_sys = nullptr;  // set with the cell arrays
     c->B.sys_off = c->sys_off;
   }
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->flags, 0, sizeof(int), c->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->flags, 0, 2 * sizeof(int), c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->ctrl, 0, sizeof(Ctrl), c->stream);
   if (e == cudaSuccess) e = build_radial_tabs(c);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -1604,7 +1604,6 @@ mxe_status mxe_destroy(mxe_ctx* c) {
   dfree(c->bd_idx);
   dfree(c->scan_tmp);
   dfree(c->totals);
-  dfree(c->max_row);
   dfree(c->smax_bits);
   dfree(c->qf);
   dfree(c->q_build);
@@ -2098,7 +2097,8 @@ mxe_status mxe_free_energy_grad_async(mxe_ctx* c, const mxe_state* s, double* F4
   mxe_status ms = enqueue_passes(c, s, A, want_mu);
   if (ms != MXE_OK) return ms;
   if (c->nsys) CK(TIMED("energy_reduce", launch_energy_seg(c->site_E, c->n, c->B, F4_dev, c->stream)));
-  else CK(TIMED("energy_reduce", launch_energy_reduce(c->site_E, c->n, c->partials, F4_dev, c->stream)));
+  else CK(TIMED("energy_reduce", launch_energy_reduce(c->site_E, c->n, c->partials, (unsigned*)(c->flags + 1),
+                                                             F4_dev, c->stream)));
   return MXE_OK;
 }
 

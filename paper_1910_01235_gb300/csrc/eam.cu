@@ -1866,50 +1866,54 @@ __global__ void k_pack_ab(const double* __restrict__ a, const double* __restrict
 
 // ---------------------------------------------------------------- K6: energy totals
 // Fixed grouping (kReduceGroup sites per partial, fixed tree inside a group,
-// groups summed in order by one block), so the totals do not depend on any
-// launch shape.
-__global__ void k_energy_partials(const double* __restrict__ site_E, int64_t n, int64_t ngroups,
-                                  double* __restrict__ partials) {
-  __shared__ double sh[3][kReduceGroup / 4];
+// the partials summed in a fixed order), so the totals do not depend on any
+// launch shape.  The last block to finish (ticket) adds the partials: a second
+// launch would cost more than the sums of a small system.
+__global__ void __launch_bounds__(256) k_energy(const double* __restrict__ site_E, int64_t n, int64_t ngroups,
+                                                double* __restrict__ partials, unsigned* __restrict__ ticket,
+                                                double* __restrict__ F4) {
+  static_assert(kReduceGroup == 4 * 256, "four sites per thread");
+  __shared__ double sh[3][256];
+  __shared__ int s_last;
   const int64_t grp = blockIdx.x;
-  const int tid = threadIdx.x;  // blockDim = kReduceGroup / 4
+  const int tid = threadIdx.x;
+  auto block_sum = [&]() {
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+      if (tid < w)
+        for (int c = 0; c < 3; ++c) sh[c][tid] += sh[c][tid + w];
+      __syncthreads();
+    }
+  };
   for (int c = 0; c < 3; ++c) {
     double v = 0.0;
     for (int r = 0; r < 4; ++r) {
-      int64_t i = grp * kReduceGroup + r * (kReduceGroup / 4) + tid;
+      const int64_t i = grp * kReduceGroup + r * 256 + tid;
       if (i < n) v += site_E[c * n + i];
     }
     sh[c][tid] = v;
   }
-  __syncthreads();
-  for (int w = kReduceGroup / 8; w > 0; w >>= 1) {
-    if (tid < w)
-      for (int c = 0; c < 3; ++c) sh[c][tid] += sh[c][tid + w];
-    __syncthreads();
-  }
-  if (tid == 0)
+  block_sum();
+  if (tid == 0) {
     for (int c = 0; c < 3; ++c) partials[c * ngroups + grp] = sh[c][0];
-}
-
-__global__ void k_energy_final(const double* __restrict__ partials, int64_t ngroups, double* __restrict__ F4) {
-  __shared__ double sh[3][256];
-  const int tid = threadIdx.x;
+    __threadfence();  // partials before the ticket
+    s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
   for (int c = 0; c < 3; ++c) {
     double v = 0.0;
-    for (int64_t gi = tid; gi < ngroups; gi += 256) v += partials[c * ngroups + gi];
+    for (int64_t gi = tid; gi < ngroups; gi += 256) v += __ldcg(&partials[c * ngroups + gi]);
     sh[c][tid] = v;
   }
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (tid < w)
-      for (int c = 0; c < 3; ++c) sh[c][tid] += sh[c][tid + w];
-    __syncthreads();
-  }
+  block_sum();
   if (tid == 0) {
     F4[0] = sh[0][0];
     F4[1] = sh[1][0];
     F4[2] = sh[2][0];
     F4[3] = (sh[0][0] + sh[1][0]) + sh[2][0];
+    *ticket = 0u;
   }
 }
 
@@ -2033,11 +2037,10 @@ cudaError_t launch_pack_ab(const double* a, const double* b, int64_t n, int S, f
   return cudaGetLastError();
 }
 
-cudaError_t launch_energy_reduce(const double* site_E, int64_t n, double* partials, double* F4, cudaStream_t s) {
-  int64_t ng = (n + kReduceGroup - 1) / kReduceGroup;
-  if (ng < 1) ng = 1;
-  k_energy_partials<<<(unsigned)ng, kReduceGroup / 4, 0, s>>>(site_E, n, ng, partials);
-  k_energy_final<<<1, 256, 0, s>>>(partials, ng, F4);
+cudaError_t launch_energy_reduce(const double* site_E, int64_t n, double* partials, unsigned* ticket, double* F4,
+                                 cudaStream_t s) {
+  const int64_t ng = std::max<int64_t>((n + kReduceGroup - 1) / kReduceGroup, 1);
+  k_energy<<<(unsigned)ng, 256, 0, s>>>(site_E, n, ng, partials, ticket, F4);
   return cudaGetLastError();
 }
 

@@ -258,9 +258,14 @@ cudaError_t launch_cell_fill_direct(const double* q, const float4* qf, const uin
                                     int* n_below, int* pair_cnt, int* row_max, int* flags, cudaStream_t s);
 cudaError_t launch_row_compact(const uint32_t* rows, const int* brows, int stride, int64_t n, const int* nb_off,
                                const int* bd_off, uint32_t* nb_ent, int* bd_idx, cudaStream_t s);
-// exclusive scan of n int32 counts into out[0..n] (out[n] = total, int64 total in *total64)
-cudaError_t launch_scan(const int* in, int* out, int64_t n, long long* total64, int* tmp, int64_t tmp_len,
-                        cudaStream_t s);
+// exclusive scans of n int32 counts each into out[0..n] (out[n] = total, int64
+// total in *total); up to three of the same length together
+struct ScanJobs {
+  const int* in[3];
+  int* out[3];
+  long long* total[3];
+};
+cudaError_t launch_scan(const ScanJobs& J, int count, int64_t n, long long* tmp, int64_t tmp_len, cudaStream_t s);
 int64_t scan_tmp_len(int64_t n);
 cudaError_t launch_strip_codes(const uint32_t* ent, int32_t* idx, int64_t m, cudaStream_t s);
 cudaError_t launch_site_max(const double* sigma, const double* q, int64_t n, unsigned long long* out_bits,
@@ -379,7 +384,9 @@ cudaError_t launch_emb_exact(bool second, bool fp64, int nl, const DevPot& P, co
 cudaError_t launch_emb_tab(bool second, const DevPot& P, const DevGrid& g, const PassArgs& A, const EmbArgs& E,
                            const RadialTab& tab, cudaStream_t s);
 cudaError_t launch_pack_ab(const double* a, const double* b, int64_t n, int S, float4* ab32, cudaStream_t s);
-cudaError_t launch_energy_reduce(const double* site_E, int64_t n, double* partials, double* F4, cudaStream_t s);
+// ticket: zero between launches
+cudaError_t launch_energy_reduce(const double* site_E, int64_t n, double* partials, unsigned* ticket, double* F4,
+                                 cudaStream_t s);
 // batches: F4 [nsys][4], one block per system in a fixed order
 cudaError_t launch_energy_seg(const double* site_E, int64_t n, const Batch& B, double* F4, cudaStream_t s);
 

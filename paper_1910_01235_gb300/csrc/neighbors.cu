@@ -17,6 +17,8 @@
 // which the FP32 kernels use to rebuild d from cell-relative positions.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "mxe_internal.cuh"
 
 namespace mxe {
@@ -281,7 +283,11 @@ __global__ void k_nbr_fill(const double* __restrict__ q, const float4* __restric
 // takes one home site of the cell at a time and tests it against the staged
 // candidates with the same rule as above.  The warp-per-site kernels above are
 // the fallback when a stencil holds more candidates than shared memory fits.
-constexpr int kCellThreads = 128;
+// 128 threads a cell, eight blocks an SM; grids with fewer cells than two per SM
+// take 512, so that a cell's 20-30 home sites are two rounds of warps and not
+// eight (500 sites, 27 cells: 40 -> 17 us a fill).
+constexpr int kCellThreads = 128, kCellThreadsFew = 512;
+inline bool few_cells(int64_t ncell) { return ncell <= 304; }
 
 struct CellStage {
   int ncand;
@@ -480,7 +486,7 @@ __device__ __forceinline__ void warp_sort_row(const uint32_t* __restrict__ buf, 
   }
 }
 
-__global__ void __launch_bounds__(kCellThreads) k_cell_count(
+__global__ void __launch_bounds__(kCellThreadsFew) k_cell_count(
     const double* __restrict__ q, const float4* __restrict__ qf, const uint8_t* __restrict__ sub, uint32_t mobile_mask,
     int64_t n, DevGrid g0, Batch B, const int* __restrict__ cell_start, const int* __restrict__ cell_sites, double rl2,
     double rb2, float2 bands, int cand_cap, int* __restrict__ nb_cnt, int* __restrict__ bd_cnt,
@@ -534,8 +540,8 @@ __global__ void __launch_bounds__(kCellThreads) k_cell_count(
 // = the stride, from the previous build) with its counts in nb_cnt / bd_cnt
 // and the longest row in *row_max; a row longer than the stride is cut and
 // its true length reported, so the caller can fall back to count + fill.
-template <bool DIRECT>
-__global__ void __launch_bounds__(kCellThreads, 8) k_cell_fill(
+template <bool DIRECT, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == kCellThreads ? 8 : 1) k_cell_fill(
     const double* __restrict__ q, const float4* __restrict__ qf, const uint8_t* __restrict__ sub, uint32_t mobile_mask,
     int64_t n, DevGrid g0, Batch B, const int* __restrict__ cell_start, const int* __restrict__ cell_sites,
     const int* __restrict__ abs_cell, double rl2, double rb2, float2 bands, int cand_cap,
@@ -692,23 +698,25 @@ __global__ void __launch_bounds__(kCellThreads, 8) k_cell_fill(
   }
 }
 
-// Largest number of candidates of any cell's stencil.
+// Largest number of candidates of any cell's stencil (one atomic per warp).
 __global__ void k_cand_max(int64_t ncell, DevGrid g0, Batch B, const int* __restrict__ cell_start,
                            int* __restrict__ out) {
   const int64_t c0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (c0 >= ncell) return;
-  const int sys = B.nsys ? B.cell_sys[c0] : 0;
-  const DevGrid g = B.nsys ? B.grids[sys] : g0;
-  const int base = B.nsys ? B.cell_base[sys] : 0;
-  const Stencil st = make_stencil((int)c0 - base, g);
   int tot = 0;
-  for (int ax = 0; ax < st.cnt[0]; ++ax)
-    for (int ay = 0; ay < st.cnt[1]; ++ay)
-      for (int az = 0; az < st.cnt[2]; ++az) {
-        const int c = base + (st.off[0][ax] * g.nc[1] + st.off[1][ay]) * g.nc[2] + st.off[2][az];
-        tot += cell_start[c + 1] - cell_start[c];
-      }
-  atomicMax(out, tot);
+  if (c0 < ncell) {
+    const int sys = B.nsys ? B.cell_sys[c0] : 0;
+    const DevGrid g = B.nsys ? B.grids[sys] : g0;
+    const int base = B.nsys ? B.cell_base[sys] : 0;
+    const Stencil st = make_stencil((int)c0 - base, g);
+    for (int ax = 0; ax < st.cnt[0]; ++ax)
+      for (int ay = 0; ay < st.cnt[1]; ++ay)
+        for (int az = 0; az < st.cnt[2]; ++az) {
+          const int c = base + (st.off[0][ax] * g.nc[1] + st.off[1][ay]) * g.nc[2] + st.off[2][az];
+          tot += cell_start[c + 1] - cell_start[c];
+        }
+  }
+  tot = __reduce_max_sync(0xffffffffu, tot);
+  if ((threadIdx.x & 31) == 0 && tot) atomicMax(out, tot);
 }
 
 // ---------------------------------------------------------------- scan
@@ -716,8 +724,11 @@ constexpr int kScanThreads = 256;
 constexpr int kScanPer = 8;
 constexpr int kScanBlock = kScanThreads * kScanPer;
 
-__global__ void k_scan_blocks(const int* __restrict__ in, int* __restrict__ out, int64_t n,
-                              long long* __restrict__ block_tot) {
+// Up to three scans of the same length in one launch (blockIdx.y: which).
+__global__ void k_scan_blocks(ScanJobs J, int64_t n, long long* __restrict__ tops, int64_t tops_len) {
+  const int* __restrict__ in = J.in[blockIdx.y];
+  int* __restrict__ out = J.out[blockIdx.y];
+  long long* __restrict__ block_tot = tops + blockIdx.y * tops_len;
   __shared__ long long warp_tot[kScanThreads / 32];
   int64_t base = blockIdx.x * (int64_t)kScanBlock + threadIdx.x * kScanPer;
   long long v[kScanPer];
@@ -750,8 +761,9 @@ __global__ void k_scan_blocks(const int* __restrict__ in, int* __restrict__ out,
 // Exclusive scan of the block totals by one block of kScanThreads threads:
 // chunks of kScanThreads totals, each scanned with warp shuffles and the
 // warps' sums, carried from chunk to chunk (nblk is n / 2048: a few chunks).
-__global__ void __launch_bounds__(kScanThreads) k_scan_tops(long long* __restrict__ block_tot, int64_t nblk,
-                                                             long long* __restrict__ total64) {
+__global__ void __launch_bounds__(kScanThreads) k_scan_tops(ScanJobs J, long long* __restrict__ tops, int64_t tops_len,
+                                                             int64_t nblk) {
+  long long* __restrict__ block_tot = tops + blockIdx.x * tops_len;
   __shared__ long long warp_sum[kScanThreads / 32];
   __shared__ long long carry;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -775,14 +787,60 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tops(long long* __restric
     if (threadIdx.x == kScanThreads - 1) carry = before + incl;
     __syncthreads();
   }
-  if (threadIdx.x == 0) *total64 = carry;
+  if (threadIdx.x == 0) *J.total[blockIdx.x] = carry;
 }
 
-__global__ void k_scan_add(int* __restrict__ out, int64_t n, const long long* __restrict__ block_tot,
-                           const long long* __restrict__ total64) {
+__global__ void k_scan_add(ScanJobs J, int64_t n, const long long* __restrict__ tops, int64_t tops_len) {
+  int* __restrict__ out = J.out[blockIdx.y];
+  const long long* __restrict__ block_tot = tops + blockIdx.y * tops_len;
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < n) out[i] = (int)((long long)out[i] + block_tot[i / kScanBlock]);
-  if (i == n) out[n] = (int)(*total64);
+  if (i == n) out[n] = (int)(*J.total[blockIdx.y]);
+}
+
+// Short arrays: one block per scan, chunk after chunk of kScanSmall counts, one
+// launch instead of three.
+constexpr int kScanSmall = 1024;
+__global__ void __launch_bounds__(kScanSmall) k_scan_short(ScanJobs J, int64_t n) {
+  const int* __restrict__ in = J.in[blockIdx.x];
+  int* __restrict__ out = J.out[blockIdx.x];
+  __shared__ long long warp_sum[kScanSmall / 32];
+  __shared__ long long carry;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) carry = 0;
+  __syncthreads();
+  for (int64_t c0 = 0; c0 < n; c0 += kScanSmall) {
+    const int64_t i = c0 + threadIdx.x;
+    const long long v = i < n ? in[i] : 0;
+    long long incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) warp_sum[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+      const long long w = warp_sum[lane];
+      long long s = w;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const long long y = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += y;
+      }
+      warp_sum[lane] = s - w;
+    }
+    __syncthreads();
+    const long long excl = carry + warp_sum[warp] + incl - v;
+    if (i < n) out[i] = (int)excl;
+    __syncthreads();
+    if (threadIdx.x == kScanSmall - 1) carry = excl + v;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    *J.total[blockIdx.x] = carry;
+    out[n] = (int)carry;
+  }
 }
 
 __global__ void k_strip(const uint32_t* __restrict__ ent, int32_t* __restrict__ idx, int64_t m) {
@@ -791,28 +849,36 @@ __global__ void k_strip(const uint32_t* __restrict__ ent, int32_t* __restrict__ 
 }
 
 // out[0] = max sigma, out[1] = max |q| component (maxima of non-negative doubles =
-// maxima of their bit patterns; warp maximum, then one atomic per warp)
-__device__ __forceinline__ void warp_max_bits(unsigned long long* addr, double v) {
-  unsigned long long b = __double_as_longlong(v);
+// maxima of their bit patterns): one atomic per block and value (one per warp
+// serialised 27,000 updates of a word at 864,000 sites)
+__device__ __forceinline__ void block_max_bits(unsigned long long* out, double v0, double v1) {
+  __shared__ unsigned long long s_max[2];
+  if (threadIdx.x < 2) s_max[threadIdx.x] = 0ull;
+  __syncthreads();
+  unsigned long long b[2] = {(unsigned long long)__double_as_longlong(v0), (unsigned long long)__double_as_longlong(v1)};
 #pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    unsigned long long y = __shfl_xor_sync(0xffffffffu, b, o);
-    b = y > b ? y : b;
+  for (int k = 0; k < 2; ++k) {
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      const unsigned long long y = __shfl_xor_sync(0xffffffffu, b[k], o);
+      b[k] = y > b[k] ? y : b[k];
+    }
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_max[k], b[k]);
   }
-  if ((threadIdx.x & 31) == 0) atomicMax(addr, b);
+  __syncthreads();
+  if (threadIdx.x < 2) atomicMax(&out[threadIdx.x], s_max[threadIdx.x]);
 }
 
 __global__ void k_site_max(const double* __restrict__ sigma, const double* __restrict__ q, int64_t n,
                            unsigned long long* __restrict__ out) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   double vs = 0.0, vq = 0.0;
-  if (i < n) {
-    vs = fmax(sigma[i], 0.0);
-    vq = fmax(fabs(q[i]), fmax(fabs(q[n + i]), fabs(q[2 * n + i])));
-    if (!(vq <= 1e300)) vq = 1e300;  // NaN / Inf positions
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    vs = fmax(vs, sigma[i]);
+    double v = fmax(fabs(q[i]), fmax(fabs(q[n + i]), fabs(q[2 * n + i])));
+    if (!(v <= 1e300)) v = 1e300;  // NaN / Inf positions
+    vq = fmax(vq, v);
   }
-  warp_max_bits(&out[0], vs);
-  warp_max_bits(&out[1], vq);
+  block_max_bits(out, vs, vq);
 }
 
 inline unsigned grid_for(int64_t work, int threads) { return (unsigned)((work + threads - 1) / threads); }
@@ -961,12 +1027,15 @@ cudaError_t launch_cand_max(int64_t ncell, const DevGrid& g, const Batch& B, con
   return cudaGetLastError();
 }
 
-size_t cell_stage_bytes(int cand_cap, int max_row, bool fill) {
+static size_t stage_bytes(int threads, int cand_cap, int max_row, bool fill) {
   size_t b = (size_t)cand_cap * (sizeof(float4) + sizeof(int));
   if (fill)
-    b += 16 + (size_t)(kCellThreads / 32) * 2 * (size_t)((max_row + 3) & ~3) * sizeof(uint32_t) +
+    b += 16 + (size_t)(threads / 32) * 2 * (size_t)((max_row + 3) & ~3) * sizeof(uint32_t) +
          (size_t)8 * cand_cap * sizeof(uint16_t);  // rows and sort keys per warp, octant lists
   return b + 16;
+}
+size_t cell_stage_bytes(int cand_cap, int max_row, bool fill) {
+  return stage_bytes(kCellThreads, cand_cap, max_row, fill);
 }
 
 cudaError_t launch_cell_count(const double* q, const float4* qf, const uint8_t* sub, uint32_t mobile_mask, int64_t n,
@@ -977,7 +1046,7 @@ cudaError_t launch_cell_count(const double* q, const float4* qf, const uint8_t* 
   const size_t shm = cell_stage_bytes(cand_cap, 0, false);
   cudaError_t e = cudaFuncSetAttribute(k_cell_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
   if (e != cudaSuccess) return e;
-  k_cell_count<<<(unsigned)ncell, kCellThreads, shm, s>>>(q, qf, sub, mobile_mask, n, g, B, cell_start, cell_sites, rl2,
+  k_cell_count<<<(unsigned)ncell, few_cells(ncell) ? kCellThreadsFew : kCellThreads, shm, s>>>(q, qf, sub, mobile_mask, n, g, B, cell_start, cell_sites, rl2,
                                                           rb2, band, cand_cap, nb_cnt, bd_cnt, max_row, flags);
   return cudaGetLastError();
 }
@@ -989,14 +1058,19 @@ cudaError_t launch_cell_fill(const double* q, const float4* qf, const uint8_t* s
                              int* flags, cudaStream_t s) {
   if (n == 0 || ncell == 0) return cudaSuccess;
   if (max_row < 1) max_row = 1;
-  const size_t shm = cell_stage_bytes(cand_cap, max_row, true);
-  cudaError_t e = cudaFuncSetAttribute(k_cell_fill<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-  if (e != cudaSuccess) return e;
-  k_cell_fill<false><<<(unsigned)ncell, kCellThreads, shm, s>>>(q, qf, sub, mobile_mask, n, g, B, cell_start,
+  auto run = [&](auto kernel, int threads) {
+    const size_t shm = stage_bytes(threads, cand_cap, max_row, true);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+    if (e != cudaSuccess) return e;
+    kernel<<<(unsigned)ncell, threads, shm, s>>>(q, qf, sub, mobile_mask, n, g, B, cell_start,
                                                                 cell_sites, abs_cell, rl2, rb2, band, cand_cap, nb_off,
                                                                 nb_ent, bd_off, bd_idx, max_row, nullptr, nullptr,
                                                                 nullptr, nullptr, nullptr, flags);
-  return cudaGetLastError();
+    return cudaGetLastError();
+  };
+  // the caller bounds the staged bytes at 128 threads; 512 fit whenever those do
+  if (few_cells(ncell)) return run(k_cell_fill<false, kCellThreadsFew>, kCellThreadsFew);
+  return run(k_cell_fill<false, kCellThreads>, kCellThreads);
 }
 
 cudaError_t launch_cell_fill_direct(const double* q, const float4* qf, const uint8_t* sub, uint32_t mobile_mask,
@@ -1005,14 +1079,19 @@ cudaError_t launch_cell_fill_direct(const double* q, const float4* qf, const uin
                                     int cand_cap, int stride, uint32_t* rows, int* brows, int* nb_cnt, int* bd_cnt,
                                     int* n_below, int* pair_cnt, int* row_max, int* flags, cudaStream_t s) {
   if (n == 0 || ncell == 0) return cudaSuccess;
-  const size_t shm = cell_stage_bytes(cand_cap, stride, true);
-  cudaError_t e = cudaFuncSetAttribute(k_cell_fill<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-  if (e != cudaSuccess) return e;
-  k_cell_fill<true><<<(unsigned)ncell, kCellThreads, shm, s>>>(q, qf, sub, mobile_mask, n, g, B, cell_start,
+  auto run = [&](auto kernel, int threads) {
+    const size_t shm = stage_bytes(threads, cand_cap, stride, true);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+    if (e != cudaSuccess) return e;
+    kernel<<<(unsigned)ncell, threads, shm, s>>>(q, qf, sub, mobile_mask, n, g, B, cell_start,
                                                                cell_sites, abs_cell, rl2, rb2, band, cand_cap, nullptr,
                                                                rows, nullptr, brows, stride, nb_cnt, bd_cnt, n_below,
                                                                pair_cnt, row_max, flags);
-  return cudaGetLastError();
+    return cudaGetLastError();
+  };
+  // the caller bounds the staged bytes at 128 threads; 512 fit whenever those do
+  if (few_cells(ncell)) return run(k_cell_fill<true, kCellThreadsFew>, kCellThreadsFew);
+  return run(k_cell_fill<true, kCellThreads>, kCellThreads);
 }
 
 cudaError_t launch_row_compact(const uint32_t* rows, const int* brows, int stride, int64_t n, const int* nb_off,
@@ -1023,17 +1102,21 @@ cudaError_t launch_row_compact(const uint32_t* rows, const int* brows, int strid
   return cudaGetLastError();
 }
 
-int64_t scan_tmp_len(int64_t n) { return (n + kScanBlock) / kScanBlock + 2; }
+int64_t scan_tmp_len(int64_t n) { return 3 * ((n + kScanBlock) / kScanBlock + 2); }
 
-cudaError_t launch_scan(const int* in, int* out, int64_t n, long long* total64, int* tmp, int64_t tmp_len,
-                        cudaStream_t s) {
-  int64_t nblk = (n + kScanBlock - 1) / kScanBlock;
-  if (nblk < 1) nblk = 1;
-  if (nblk + 1 > tmp_len) return cudaErrorInvalidValue;
-  long long* bt = reinterpret_cast<long long*>(tmp);
-  k_scan_blocks<<<(unsigned)nblk, kScanThreads, 0, s>>>(in, out, n, bt);
-  k_scan_tops<<<1, kScanThreads, 0, s>>>(bt, nblk, total64);
-  k_scan_add<<<grid_for(n + 1, 256), 256, 0, s>>>(out, n, bt, total64);
+// Up to 16,384 counts (sixteen chunks of a block, about 1 us each) take the
+// one-launch form: three launches cost about 7 us whatever the length.
+cudaError_t launch_scan(const ScanJobs& J, int count, int64_t n, long long* tmp, int64_t tmp_len, cudaStream_t s) {
+  if (count < 1 || count > 3) return cudaErrorInvalidValue;
+  if (n <= 16 * kScanSmall) {
+    k_scan_short<<<count, kScanSmall, 0, s>>>(J, n);
+    return cudaGetLastError();
+  }
+  const int64_t nblk = (n + kScanBlock - 1) / kScanBlock, tops = nblk + 1;
+  if (count * tops > tmp_len) return cudaErrorInvalidValue;
+  k_scan_blocks<<<dim3((unsigned)nblk, count), kScanThreads, 0, s>>>(J, n, tmp, tops);
+  k_scan_tops<<<count, kScanThreads, 0, s>>>(J, tmp, tops, nblk);
+  k_scan_add<<<dim3(grid_for(n + 1, 256), count), 256, 0, s>>>(J, n, tmp, tops);
   return cudaGetLastError();
 }
 
@@ -1046,7 +1129,7 @@ cudaError_t launch_strip_codes(const uint32_t* ent, int32_t* idx, int64_t m, cud
 cudaError_t launch_site_max(const double* sigma, const double* q, int64_t n, unsigned long long* out_bits,
                             cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  k_site_max<<<grid_for(n, 256), 256, 0, s>>>(sigma, q, n, out_bits);
+  k_site_max<<<std::min(grid_for(n, 256), 1216u), 256, 0, s>>>(sigma, q, n, out_bits);  // 8 blocks per SM
   return cudaGetLastError();
 }
 
