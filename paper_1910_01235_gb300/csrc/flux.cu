@@ -9,16 +9,18 @@
 // of a whole run is 1e-7.
 //
 // k_flux_prep evaluates the per-site factors once: beta_i, D_i = nu0
-// exp(-beta_i Qm), x_iv, and E_ik = exp(beta_i mu_ik) with its reciprocal.
-// Across a bond whose two ends share the temperature, exp(beta (mu_i - mu_j))
-// = E_i / E_j, so a hop costs four multiplications and no exponential; a bond
-// between different temperatures, or an E outside the normal range, takes the
-// exponential of the difference.  Each site gathers over its own bond row (no
-// atomics, deterministic).  A bond's net exchange is always formed by the same
-// function of the bond's canonical orientation (lower index first) with
-// explicitly rounded operations, so site j obtains exactly the negation of
-// what site i obtains: the two updates cancel and mass is conserved up to the
-// rounding of the two row sums.
+// exp(-beta_i Qm), x_iv, and with E_ik = exp(beta_i mu_ik) the pair P_ik = D_i x_ik
+// E_ik, Q_ik = x_iv / E_ik.  Across a bond whose two ends share the temperature,
+// J_{i->j} = P_ik Q_jk: one multiplication a hop (the FP64 pipe bounds the
+// gather; with separate factors a bond took 18 FP64 instructions per species
+// and 12 loads, now 4 and 2); a bond between different temperatures, or an E
+// outside the normal range (its Q holds a marker), takes the exponential of the
+// difference.  Each site gathers over its own bond row (no atomics,
+// deterministic).  A bond's net exchange is always formed by the same function
+// of the bond's canonical orientation (lower index first) with explicitly
+// rounded operations, so site j obtains exactly the negation of what site i
+// obtains: the two updates cancel and mass is conserved up to the rounding of
+// the two row sums.
 #include <cuda_runtime.h>
 
 #include "mxe_internal.cuh"
@@ -27,6 +29,7 @@ namespace mxe {
 namespace {
 
 constexpr double kEMin = 1e-250, kEMax = 1e250;
+constexpr int kNotFactorised = 0x7ff80000;  // high word of a Q that must not be used
 
 // Reservoirs (Sec. 4, fix setchemicalpotential / setatomicfraction): a site
 // of the chemical-potential group enters every rate with its held mu; a site of
@@ -54,30 +57,26 @@ __global__ void __launch_bounds__(256) k_flux_prep(const double* __restrict__ x,
   double xv = 1.0;
 #pragma unroll
   for (int k = 0; k < S; ++k) xv -= x[k * n + i];
-  fl[i] = beta;
-  fl[n + i] = nu0 * exp(-beta * Qm);
-  fl[2 * n + i] = xv;
+  const double D = nu0 * exp(-beta * Qm);
+  double* tail = fl + 2 * S * n;  // beta, D, xv after the (P, Q) pairs [n][S]
+  tail[i] = beta;
+  tail[n + i] = D;
+  tail[2 * n + i] = xv;
 #pragma unroll
   for (int k = 0; k < S; ++k) {
     const double m = held ? res.fix_mu_value[k * n + i] : mu[k * n + i];
     if (res.mu_eff) res.mu_eff[k * n + i] = m;
     const double E = exp(beta * m);
-    fl[(3 + 2 * k) * n + i] = E;
-    fl[(4 + 2 * k) * n + i] = 1.0 / E;
+    const bool normal = E > kEMin && E < kEMax;
+    reinterpret_cast<double2*>(fl)[i * S + k] =
+        make_double2(D * x[k * n + i] * E, normal ? xv / E : __hiloint2double(kNotFactorised, 0));
   }
 }
 
-struct Site {
-  double T, beta, D, xv, x, mu, E, Einv;
-};
-
-// J_{a->b} for one species
-__device__ __forceinline__ double hop(const Site& a, const Site& b, bool factorised) {
-  const double e = factorised ? __dmul_rn(a.E, b.Einv) : exp(__dmul_rn(a.beta, __dsub_rn(a.mu, b.mu)));
-  return __dmul_rn(__dmul_rn(__dmul_rn(a.D, a.x), b.xv), e);
+// J_{a->b} of one species by the exponential of the difference
+__device__ __forceinline__ double hop_exp(double Da, double xa, double xvb, double beta_a, double mua, double mub) {
+  return __dmul_rn(__dmul_rn(__dmul_rn(Da, xa), xvb), exp(__dmul_rn(beta_a, __dsub_rn(mua, mub))));
 }
-
-__device__ __forceinline__ bool normal_E(const Site& s) { return s.E > kEMin && s.E < kEMax; }
 
 template <int S>
 __global__ void __launch_bounds__(256) k_flux(const double* __restrict__ x, const double* __restrict__ T,
@@ -88,36 +87,35 @@ __global__ void __launch_bounds__(256) k_flux(const double* __restrict__ x, cons
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n || (res.gate && res.gate->halted)) return;
   const double* __restrict__ mu = res.mu_eff ? res.mu_eff : mu_in;
-  Site si[S];
-#pragma unroll
-  for (int k = 0; k < S; ++k) {
-    si[k].T = T[i];
-    si[k].beta = fl[i];
-    si[k].D = fl[n + i];
-    si[k].xv = fl[2 * n + i];
-    si[k].x = x[k * n + i];
-    si[k].mu = mu[k * n + i];
-    si[k].E = fl[(3 + 2 * k) * n + i];
-    si[k].Einv = fl[(4 + 2 * k) * n + i];
-  }
+  const double2* __restrict__ pq = reinterpret_cast<const double2*>(fl);
+  const double* __restrict__ tail = fl + 2 * S * n;
+  const long long Ti = __double_as_longlong(T[i]);
+  double2 si[S];
   double rate[S];
 #pragma unroll
-  for (int k = 0; k < S; ++k) rate[k] = 0.0;
+  for (int k = 0; k < S; ++k) {
+    si[k] = pq[i * S + k];
+    rate[k] = 0.0;
+  }
   const int beg = bd_off[i], end = bd_off[i + 1];
+#pragma unroll 2
   for (int t = beg; t < end; ++t) {
     const int64_t j = bd_idx[t];
-    const double Tj = T[j], bj = fl[j], Dj = fl[n + j], xvj = fl[2 * n + j];
+    const bool sameT = __double_as_longlong(__ldg(&T[j])) == Ti;
 #pragma unroll
     for (int k = 0; k < S; ++k) {
-      Site sj{Tj, bj, Dj, xvj, x[k * n + j], mu[k * n + j], fl[(3 + 2 * k) * n + j], fl[(4 + 2 * k) * n + j]};
-      const bool fac = si[k].T == sj.T && normal_E(si[k]) && normal_E(sj);
-      if (i < j) {
-        const double net = __dsub_rn(hop(si[k], sj, fac), hop(sj, si[k], fac));
-        rate[k] = __dsub_rn(rate[k], net);  // outflow from i
+      const double2 sj = __ldg(&pq[j * S + k]);
+      double out, in;  // J_{i->j}, J_{j->i}
+      if (sameT && __double2hiint(si[k].y) != kNotFactorised && __double2hiint(sj.y) != kNotFactorised) {
+        out = __dmul_rn(si[k].x, sj.y);
+        in = __dmul_rn(sj.x, si[k].y);
       } else {
-        const double net = __dsub_rn(hop(sj, si[k], fac), hop(si[k], sj, fac));
-        rate[k] = __dadd_rn(rate[k], net);  // inflow into i
+        const double xi = x[k * n + i], xj = x[k * n + j], mi = mu[k * n + i], mj = mu[k * n + j];
+        out = hop_exp(tail[n + i], xi, tail[2 * n + j], tail[i], mi, mj);
+        in = hop_exp(tail[n + j], xj, tail[2 * n + i], tail[j], mj, mi);
       }
+      if (i < j) rate[k] = __dsub_rn(rate[k], __dsub_rn(out, in));  // outflow from i
+      else rate[k] = __dadd_rn(rate[k], __dsub_rn(in, out));        // inflow into i
     }
   }
   double tot = 0.0;
@@ -126,7 +124,7 @@ __global__ void __launch_bounds__(256) k_flux(const double* __restrict__ x, cons
   const double dti = res.dt_sys ? __dmul_rn(dt, res.dt_sys[res.sys_of[i]]) : dt;
 #pragma unroll
   for (int k = 0; k < S; ++k) {
-    const double v = held_x ? res.fix_x_value[k * n + i] : __dadd_rn(si[k].x, __dmul_rn(dti, rate[k]));
+    const double v = held_x ? res.fix_x_value[k * n + i] : __dadd_rn(x[k * n + i], __dmul_rn(dti, rate[k]));
     x_new[k * n + i] = v;
     tot += v;
     ok = ok && (v >= -kXTol);
