@@ -133,6 +133,8 @@ struct mxe_ctx {
   DevGrid* grids_h = nullptr;   // pinned staging of grids
   int* cell_base_h = nullptr;   // pinned staging of cell_base
   SysFire* sf = nullptr;        // [nsys] FIRE state of each system
+  double* sf_part = nullptr;    // partial sums of the per-system reductions
+  int64_t max_sites = 0;        // sites of the largest system
   SysFire* sf_h = nullptr;      // pinned copy after a relaxation
   double* dt_sys = nullptr;     // [nsys] Euler step multipliers
   Batch B{};
@@ -980,7 +982,8 @@ mxe_status enqueue_fire_iter(mxe_ctx* c, mxe_state* s, const PassArgs& A) {
   if (fm != MXE_OK) return fm;
   float4* p32 = c->precision != MXE_FP64 ? c->pos32 : nullptr;
   if (c->nsys) {
-    CK(TIMED("fire_reduce", launch_fire_seg_reduce(c->gq, c->gs, s->sigma, c->vq, c->vs, n, c->B, c->sf, c->ctrl, c->flags, st)));
+    CK(TIMED("fire_reduce", launch_fire_seg_reduce(c->gq, c->gs, s->sigma, c->vq, c->vs, n, c->max_sites, c->B, c->sf, c->sf_part,
+                                                   c->ctrl, c->flags, st)));
     CK(TIMED("fire_logic", launch_fire_seg_logic(c->sf, c->nsys, c->ctrl, c->flags, st)));
     CK(TIMED("fire_update", launch_fire_seg_update(s->q, s->sigma, c->vq, c->vs, c->gq, c->gs, c->q_build, c->abs_cell, n,
                                                    c->grid, c->B, c->sf, p32, c->ctrl, st)));
@@ -1525,6 +1528,8 @@ mxe_status mxe_create_batch(mxe_ctx** out, int32_t n_systems, const mxe_box* box
     A(dalloc(&c->grids, nsys));
     A(dalloc(&c->cell_base, nsys + 1));
     A(dalloc(&c->sf, nsys));
+    A(dalloc(&c->sf_part, fire_seg_partials_len(nsys)));
+    for (int b = 0; b < nsys; ++b) c->max_sites = std::max<int64_t>(c->max_sites, offsets[b + 1] - offsets[b]);
     A(dalloc(&c->dt_sys, nsys));
     A(cudaMallocHost((void**)&c->grids_h, sizeof(DevGrid) * nsys));
     A(cudaMallocHost((void**)&c->cell_base_h, sizeof(int) * (nsys + 1)));
@@ -1637,6 +1642,7 @@ mxe_status mxe_destroy(mxe_ctx* c) {
   dfree(c->cell_base);
   dfree(c->cell_sys);
   dfree(c->sf);
+  dfree(c->sf_part);
   dfree(c->dt_sys);
   if (c->grids_h) cudaFreeHost(c->grids_h);
   if (c->cell_base_h) cudaFreeHost(c->cell_base_h);

@@ -172,6 +172,7 @@ struct SysFire {
   int halted, reason, iter, n_pos;
   double dt, alpha, keep, mix, one_minus_alpha, fmax;
   double P, vv, ff;
+  unsigned int ticket;  // blocks of the current reduction done (0 between launches)
 };
 
 // Programmatic dependent launch.  A kernel launched by launch_pdl may be
@@ -396,10 +397,12 @@ cudaError_t launch_fire_reduce(const double* gq, const double* gs, const double*
 cudaError_t launch_fire_update(double* q, double* sigma, double* vq, double* vs, const double* gq,
                                const double* gs, const double* q_build, const int* abs_cell, int64_t n,
                                const DevGrid& g, const Batch& B, float4* pos32, Ctrl* ctrl, cudaStream_t s);
-// batches: one block per system reduces, one block runs every system's FIRE logic
+// batches: up to fire_seg_partials_len / nsys / 4 blocks a system reduce, one
+// block runs every system's FIRE logic.  max_sites: sites of the largest system.
+int64_t fire_seg_partials_len(int nsys);
 cudaError_t launch_fire_seg_reduce(const double* gq, const double* gs, const double* sigma, const double* vq,
-                                   const double* vs, int64_t n, const Batch& B, SysFire* sf, Ctrl* ctrl, int* flags,
-                                   cudaStream_t s);
+                                   const double* vs, int64_t n, int64_t max_sites, const Batch& B, SysFire* sf,
+                                   double* part, Ctrl* ctrl, int* flags, cudaStream_t s);
 cudaError_t launch_fire_seg_logic(SysFire* sf, int nsys, Ctrl* ctrl, const int* flags, cudaStream_t s);
 cudaError_t launch_fire_seg_update(double* q, double* sigma, double* vq, double* vs, const double* gq,
                                    const double* gs, const double* q_build, const int* abs_cell, int64_t n,
