@@ -492,13 +492,6 @@ __global__ void __launch_bounds__(256) k_relax_density(EmbedE E, const __grid_co
   }
 }
 
-// float -> double on bits (no FP64 instruction; subnormals give zero)
-__device__ __forceinline__ double widen(float x) {
-  const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;
-  const unsigned hi = (u & 0x80000000u) | ((e == 255u ? 0x7ffu : e + 896u) << 20) | ((u >> 3) & 0xfffffu);
-  return e == 0 ? 0.0 : __hiloint2double((int)hi, (int)(u << 29));
-}
-
 template <int PREC, int NL>
 __global__ void __launch_bounds__(256) k_relax_force(const __grid_constant__ PassArgs A,
                                                      const typename Relax<PREC>::V* __restrict__ frc) {

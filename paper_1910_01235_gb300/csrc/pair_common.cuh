@@ -66,6 +66,13 @@ __device__ __forceinline__ bool load_pair(const Args& A, const int4* __restrict_
   return ok;
 }
 
+// float -> double on bits (no FP64 instruction; subnormals give zero)
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;
+  const unsigned hi = (u & 0x80000000u) | ((e == 255u ? 0x7ffu : e + 896u) << 20) | ((u >> 3) & 0xfffffu);
+  return e == 0 ? 0.0 : __hiloint2double((int)hi, (int)(u << 29));
+}
+
 struct alignas(32) Dbl4 {
   double x, y, z, w;
 };

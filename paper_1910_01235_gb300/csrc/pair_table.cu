@@ -9,14 +9,19 @@
 // 16-byte loads per term) and 20 to 36 FP32 operations per term.
 //
 // Measured (event time per launch, direct -> tabulated).  FP64, 19,652-site
-// binary alloy (531 k pairs): forces 1127 -> 210 us, densities 709 -> 80 us,
-// geometry 911 -> 154 us.  Float-float geometry: 6.9 M pairs of the binary
+// binary alloy (531 k pairs): forces 1127 -> 161 us, densities 709 -> 72 us,
+// geometry 911 -> 149 us.  Float-float geometry: 6.9 M pairs of the binary
 // alloy (which had the power form) 1.35 -> 1.22 ms, 23.3 M pairs of one species
 // 3.54 -> 1.92 ms, 241 M pairs of the interstitial slab 52.6 -> 26.6 ms.  What
 // bounds them now (ncu): the geometry kernels the shared-memory wavefronts
 // (84-89 %; 32 lanes reading random rows take about 12 wavefronts per 16-byte
-// load, 4 without bank conflicts), the force kernel the FP64 pipe (84 %), the
-// density kernel both (65 % each).
+// load, 4 without bank conflicts), the force kernel those (64 %), instruction
+// issue (53 %) and the FP64 pipe (40 %) together, the density kernel the
+// wavefronts and the FP64 pipe (65 % each).  With the constant terms and the
+// sums of the nodes in FP64 (207 FP64 instructions a pair and lane) the force
+// kernel took 210 us, the FP64 pipe 84 % busy; with the direct evaluation
+// called inside the table loop 9 us more; with 640 threads a block (96
+// registers) 171 us, with 384 (160 registers) as with 512.
 //
 // Layout: one block per SM holds the whole table in shared memory (up to
 // 200 KB) and strides over the pairs; the table is copied before the kernel
@@ -131,7 +136,7 @@ struct NodeSum {
   ff p;
 };
 __device__ __forceinline__ double sum_value(const NodeSum& v, double scale, double*) {
-  return fma((double)v.c, scale, (double)v.p.hi + (double)v.p.lo);
+  return fixed_double(v.c, exp2_of(scale)) + (widen(v.p.hi) + widen(v.p.lo));
 }
 __device__ __forceinline__ ff sum_value(const NodeSum& v, double scale, ff*) {
   // |c| < 2^62: the high word as a float, then what it left
@@ -371,32 +376,159 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_rdensity_tab(
 }
 
 // ---------------------------------------------------------------- relaxation forces, FP64
-// dV/dr / r of the pair's weighted terms at one node: the constant terms in
-// FP64, the rest as a float pair
+// The weights of a pair's terms: C_u = (hi 2^31 + lo) 2^(e - 1082) with |hi| <=
+// 2^29, 0 <= lo < 2^31 (all 53 bits), and as float pairs.  The constant terms
+// of the rows are multiplied by them in integers on one grid per pair: a
+// product of 60-bit halves is three 32-bit multiplications and a few additions,
+// some 11 issue slots where an FP64 instruction holds a 2-lane pipe for 64.
+// The grid leaves 55 bits (one or two terms: 56) below the largest term at the
+// pair's nearest node, where the terms, which decrease, are largest, and eight
+// (seven) above, for the sum of 12 nodes: a product that is more than four
+// times larger somewhere sends the pair to the direct evaluation.
 template <int NT>
-__device__ __forceinline__ double force_node(const RadialTab& Tb, const uint4* sm, long long w, const double* C,
-                                             const ff* Cf, int& low, ff& p) {
+struct FixedWeights {
+  static constexpr int kHead = NT <= 2 ? 4 : 5;  // shift of the largest term
+  int hi[NT], lo[NT], k[NT];
+  int terms;  // that are not zero
+  ff f[NT];
+};
+// The integers' unit is 2^(the result); row: the row of the nearest node.
+template <int NT>
+__device__ __forceinline__ int fixed_weights(const double* C, const uint4* row, FixedWeights<NT>& F, int& big) {
+  int top = 0;
+  F.terms = 0;
+#pragma unroll
+  for (int u = 0; u < NT; ++u) {
+    const int h = __double2hiint(C[u]), e = (h >> 20) & 0x7ff;
+    big |= e == 0x7ff;
+    const long long m = ((long long)((h & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(C[u]);
+    const long long v = e == 0 ? 0ll : (h < 0 ? -m : m) << 7;
+    F.hi[u] = (int)(v >> 31);
+    F.lo[u] = (int)((unsigned)v & 0x7fffffffu);
+    F.k[u] = e;
+    F.f[u] = ff_bits(C[u]);
+    // the constant term, or next to the cutoff, where it vanishes, 2^5 times
+    // the linear and quadratic terms at |tau| = 1/2 (elsewhere below 2^-6 of it)
+    const uint4 a = row[u * kTabWords64];
+    const int e1 = (int)((a.z >> 23) & 0xffu), e2 = (int)((row[u * kTabWords64 + 1].x >> 23) & 0xffu);
+    const int e8 = max((int)(a.x & 0xffu), max(e1 ? e1 + 5 : 0, e2 ? e2 + 4 : 0));
+    if (e != 0 && e8 != 0) {
+      top = max(top, e + e8);
+      F.terms += 1;
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < NT; ++u) F.k[u] = top == 0 ? 1000 : top + F.kHead - F.k[u];  // top 0: every node beyond the cutoff
+  // hi m_hi is a product shifted by 62: exponents e - 1082, e8 - kTabExpBias
+  const int unit = top == 0 ? 0 : top + F.kHead - 1082 - kTabExpBias + 62;
+  // 2^(-24 - unit) has to be a float
+  big |= unit > 90 || unit < -140;
+  return unit;
+}
+
+__device__ __forceinline__ float exp2f_bits(int e) { return __uint_as_float((unsigned)(e + 127) << 23); }  // |e| < 127
+
+// v >> n, all sign bits from n = 64 on (PTX clamps the count)
+__device__ __forceinline__ long long shift_right(long long v, int n) {
+  long long r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+}
+
+// dV/dr / r of the pair's weighted terms at one node, in units of the pair's
+// grid: the constant terms as above, the rest (below 2^-6 of them) as a float
+// pair, added in two pieces of 24 bits.  sc: 2^-24 units.
+template <int NT>
+__device__ __forceinline__ long long force_node(const RadialTab& Tb, const uint4* sm, long long w,
+                                                const FixedWeights<NT>& F, float sc, int& low) {
   float th, tl;
   const uint4* row = tab_row(Tb, sm, w, th, tl, low);
-  double h = 0.0;
-  p = ff{0.f, 0.f};
+  long long h = 0;
+  ff p{0.f, 0.f};
 #pragma unroll
   for (int u = 0; u < NT; ++u) {
     const uint4 a = row[u * kTabWords64];
     const ff q = tab_poly64(__uint_as_float(a.z), __uint_as_float(a.w), row[u * kTabWords64 + 1],
                             row[u * kTabWords64 + 2], th, tl);
-    h = fma(C[u], __hiloint2double((int)a.y, (int)a.x), h);
-    ff m = two_prod(Cf[u].hi, q.hi);
-    m.lo = fmaf(Cf[u].hi, q.lo, fmaf(Cf[u].lo, q.hi, m.lo));
+    const int mh = (int)a.y, ml = (int)(a.x & 0x7fffff00u), sh = F.k[u] - (int)(a.x & 0xffu);
+    const long long cross = (long long)F.hi[u] * ml + (long long)F.lo[u] * mh;
+    low |= sh - (F.kHead - 2);  // negative: over four times the expected largest term
+    h += shift_right((long long)F.hi[u] * mh + (cross >> 31), sh);
+    ff m = two_prod(F.f[u].hi, q.hi);
+    m.lo = fmaf(F.f[u].hi, q.lo, fmaf(F.f[u].lo, q.hi, m.lo));
     tab_acc(p, m);
   }
-  return h;
+  const float x = p.hi * sc;
+  const int i1 = __float2int_rn(x);
+  low |= (1 << 30) - abs(i1);
+  const int i2 = __float2int_rn(fmaf(p.lo, sc, x - (float)i1) * 16777216.0f);
+  return h + (long long)i1 * 16777216ll + i2;
 }
 
-__device__ __forceinline__ ff ff_times(ff a, ff b) {  // without the final renormalisation
-  ff m = two_prod(a.hi, b.hi);
-  m.lo = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, m.lo));
-  return m;
+// Marks (in a thread's own record) a pair left for the direct evaluation, which
+// runs after the table loop: a call inside it costs registers in every pair.
+constexpr long long kTabLater = 0x7ff8a5a5c3c31e1ell;
+
+// weights of the terms: nodes (C) and the static point (cfs)
+template <int S, int NP, int TAB>
+__device__ __forceinline__ void force_weights(const DevPot& P, const PassArgs& A, const PairRef& pr, double* C,
+                                              double* cfs) {
+  using TB = Tables<TAB>;
+  constexpr int NF = S, NT = NF + NP;
+  const int64_t n = A.n;
+#pragma unroll
+  for (int u = 0; u < NT; ++u) C[u] = 0.0;
+#pragma unroll
+  for (int v = 0; v < NF; ++v) cfs[v] = 0.0;
+  double xi[S], xj[S], bi[S], bj[S], ai[S], aj[S];
+#pragma unroll
+  for (int k = 0; k < S; ++k) {
+    xi[k] = __ldg(&A.x[k * n + pr.i]), xj[k] = __ldg(&A.x[k * n + pr.j]);
+    ai[k] = __ldg(&A.a[k * n + pr.i]), aj[k] = __ldg(&A.a[k * n + pr.j]);
+    bi[k] = __ldg(&A.b[k * n + pr.i]), bj[k] = __ldg(&A.b[k * n + pr.j]);
+  }
+#pragma unroll
+  for (int k = 0; k < S; ++k)
+#pragma unroll
+    for (int l = 0; l < S; ++l) {
+      const int po = TB::phi(P, k, l);
+#pragma unroll
+      for (int u = 0; u < NP; ++u)
+        if (po == u) C[NF + u] += xi[k] * xj[l];
+    }
+  if constexpr (TAB == 1) {
+    // the density term is that of the neighbour's species
+    const double sbi = bi[0] + bi[1], sbj = bj[0] + bj[1], sai = ai[0] + ai[1], saj = aj[0] + aj[1];
+#pragma unroll
+    for (int v = 0; v < NF; ++v) {
+      C[v] = sbi * xj[v] + sbj * xi[v];
+      cfs[v] = sai * xj[v] + saj * xi[v];
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < S; ++k)
+#pragma unroll
+      for (int l = 0; l < S; ++l) {
+        const int fo = TB::f(P, k, l);
+#pragma unroll
+        for (int v = 0; v < NF; ++v)
+          if (fo == v) {
+            C[v] += bi[k] * xj[l] + bj[k] * xi[l];
+            cfs[v] += ai[k] * xj[l] + aj[k] * xi[l];
+          }
+      }
+  }
+}
+
+// both entries' records from T, U, V and Gs
+__device__ __forceinline__ void store_force(const PairGeom& G, const double* out, const PairRef& pr,
+                                            Dbl4* __restrict__ frc) {
+  const double inv12 = 1.0 / 12.0;
+  const double Tt = out[0] * inv12 + out[6];
+  const double fx = -(G.d[0] * Tt + out[1] * inv12), fy = -(G.d[1] * Tt + out[2] * inv12),
+               fz = -(G.d[2] * Tt + out[3] * inv12);
+  frc[pr.tp] = Dbl4{fx, fy, fz, out[4] * inv12};
+  frc[pr.tr] = Dbl4{-fx, -fy, -fz, out[5] * inv12};
 }
 
 template <int S, int NP, int TAB>
@@ -411,113 +543,92 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_rforce_tab(
   pdl_trigger();
   __syncthreads();
   if (A.ctrl != nullptr && A.ctrl->halted) return;
-  const int64_t n = A.n, stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  bool later = false;
   for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < npair; p += stride) {
     PairRef pr;
     if (!load_pair(A, pair_rec, p, pr)) continue;
     PairGeom G;
     pair_geometry(g0, A, pr.i, pr.j, G);
     PairNodes N;
-    const int big = pair_nodes(G, N);
+    int big = pair_nodes(G, N);
     int low = 0;
-    // weights of the terms: nodes (C) and the static point (cfs)
     double C[NT], cfs[NF];
-#pragma unroll
-    for (int u = 0; u < NT; ++u) C[u] = 0.0;
-#pragma unroll
-    for (int v = 0; v < NF; ++v) cfs[v] = 0.0;
-#pragma unroll
-    for (int k = 0; k < S; ++k) {
-      const double xik = __ldg(&A.x[k * n + pr.i]), aik = __ldg(&A.a[k * n + pr.i]), bik = __ldg(&A.b[k * n + pr.i]);
-      const double ajk = __ldg(&A.a[k * n + pr.j]), bjk = __ldg(&A.b[k * n + pr.j]);
-#pragma unroll
-      for (int l = 0; l < S; ++l) {
-        const double xjl = __ldg(&A.x[l * n + pr.j]), xil = __ldg(&A.x[l * n + pr.i]);
-        const int po = TB::phi(P, k, l), fo = TB::f(P, k, l);
-#pragma unroll
-        for (int u = 0; u < NP; ++u)
-          if (po == u) C[NF + u] += xik * xjl;
-#pragma unroll
-        for (int v = 0; v < NF; ++v)
-          if (fo == v) {
-            C[v] += bik * xjl + bjk * xil;
-            cfs[v] += aik * xjl + ajk * xil;
-          }
-      }
-    }
-    ff Cf[NT];
-#pragma unroll
-    for (int u = 0; u < NT; ++u) Cf[u] = ff_bits(C[u]);
+    force_weights<S, NP, TAB>(P, A, pr, C, cfs);
     double out[7];  // T, U[3], V[2], Gs
+    float th, tl;
     {
-      ff cs[NF], ps;
-#pragma unroll
-      for (int v = 0; v < NF; ++v) cs[v] = ff_bits(cfs[v]);
-      const double h = force_node<NF>(Tb, sm, N.w0, cfs, cs, low, ps);
-      out[6] = h + ((double)ps.hi + (double)ps.lo);
+      FixedWeights<NF> F;
+      const int unit = fixed_weights<NF>(cfs, tab_row(Tb, sm, N.w0, th, tl, low), F, big);
+      const long long h = force_node<NF>(Tb, sm, N.w0, F, exp2f_bits(-24 - unit), low);
+      out[6] = fixed_double(h != 0 ? h + (F.terms >> 1) : 0, unit);
     }
-    double T0 = 0.0, U0[3] = {0.0, 0.0, 0.0}, Vs[2];
-    ff Tp{0.f, 0.f}, Up[3] = {ff{0.f, 0.f}, ff{0.f, 0.f}, ff{0.f, 0.f}};
-    const double ad[3] = {fabs(G.d[0]), fabs(G.d[1]), fabs(G.d[2])};
-    const ff fd[3] = {ff_bits(ad[0]), ff_bits(ad[1]), ff_bits(ad[2])};
+    const long long near = min(N.base[0] - max(N.tw[0][0], max(N.tw[0][1], N.tw[0][2])),
+                               N.base[1] - max(N.tw[1][0], max(N.tw[1][1], N.tw[1][2])));
+    FixedWeights<NT> F;
+    const int unit = fixed_weights<NT>(C, tab_row(Tb, sm, near, th, tl, low), F, big);
+    const float sc = exp2f_bits(-24 - unit);
+    long long T = 0;
+    double U[3] = {0.0, 0.0, 0.0}, V0 = 0.0, ad[3] = {fabs(G.d[0]), fabs(G.d[1]), fabs(G.d[2])};
     double s = G.s_i;
 #pragma unroll 1
     for (int site = 0; site < 2; ++site) {
-      const ff fs = ff_bits(s);
-      double E0 = 0.0, V0 = 0.0;
-      ff Ep{0.f, 0.f}, Vp{0.f, 0.f};
-#pragma unroll
+      long long E = 0;
+      double V = 0.0;
+#pragma unroll 1
       for (int a = 0; a < 3; ++a) {
-        ff p1, p2;
-        const double h1 = force_node<NT>(Tb, sm, N.base[0] + N.tw[0][a], C, Cf, low, p1);
-        const double h2 = force_node<NT>(Tb, sm, N.base[0] - N.tw[0][a], C, Cf, low, p2);
-        const double D = h1 - h2;
-        E0 += h1;
-        E0 += h2;
-        U0[a] = fma(s, D, U0[a]);
-        V0 = fma(ad[a], D, V0);
-        tab_acc(Ep, p1);
-        tab_acc(Ep, p2);
-        tab_acc(p1, ff{-p2.hi, -p2.lo});  // p1 - p2
-        tab_acc(Up[a], ff_times(fs, p1));
-        tab_acc(Vp, ff_times(fd[a], p1));
+        const long long h1 = force_node<NT>(Tb, sm, N.base[0] + N.tw[0][0], F, sc, low);
+        const long long h2 = force_node<NT>(Tb, sm, N.base[0] - N.tw[0][0], F, sc, low);
+        E += h1 + h2 + ((h1 | h2) != 0 ? F.terms : 0);  // the shifts round down, half a unit each
+        const double D = fixed_double(h1 - h2, unit), Ua = fma(s, D, U[0]), da = ad[0];
+        V = fma(da, D, V);
+        // the next axis (registers rotate: one copy of the node code)
+        const long long t = N.tw[0][0];
+        N.tw[0][0] = N.tw[0][1];
+        N.tw[0][1] = N.tw[0][2];
+        N.tw[0][2] = t;
+        U[0] = U[1];
+        U[1] = U[2];
+        U[2] = Ua;
+        ad[0] = ad[1];
+        ad[1] = ad[2];
+        ad[2] = da;
       }
-      tab_acc(Tp, Ep);
-      tab_acc(Vp, ff_times(fs, Ep));
-      T0 += E0;
-      const double v = kSqrt6 * (fma(s, E0, V0) + ((double)Vp.hi + (double)Vp.lo));
-      Vs[1] = v;
-      if (site == 0) Vs[0] = v;
+      T += E;
+      V = kSqrt6 * fma(s, fixed_double(E, unit), V);
+      out[4] = V0;
+      out[5] = V0 = V;
       s = G.s_j;
       N.base[0] = N.base[1];
 #pragma unroll
       for (int a = 0; a < 3; ++a) N.tw[0][a] = N.tw[1][a];
     }
-    out[0] = T0 + ((double)Tp.hi + (double)Tp.lo);
+    out[0] = fixed_double(T, unit);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) out[1 + a] = copysign(1.0, G.d[a]) * (U0[a] + ((double)Up[a].hi + (double)Up[a].lo));
-    out[4] = Vs[0];
-    out[5] = Vs[1];
+    for (int a = 0; a < 3; ++a) out[1 + a] = __double2hiint(G.d[a]) < 0 ? -U[a] : U[a];
+    store_force(G, out, pr, frc);
     if (big || low < 0) {
-      const PairGeom H = G;
-      double ca[2] = {0.0, 0.0}, cs[2] = {0.0, 0.0}, cp[3] = {0.0, 0.0, 0.0}, o[7];
-#pragma unroll
-      for (int v = 0; v < NF; ++v) {
-        ca[v] = C[v];
-        cs[v] = cfs[v];
-      }
-#pragma unroll
-      for (int u = 0; u < NP; ++u) cp[u] = C[NF + u];
-      direct_forces(P, H, ca, cs, cp, o);
-#pragma unroll
-      for (int c = 0; c < 7; ++c) out[c] = o[c];
+      frc[pr.tp].x = __longlong_as_double(kTabLater);
+      later = true;
     }
-    const double inv12 = 1.0 / 12.0;
-    const double Tt = out[0] * inv12 + out[6];
-    const double fx = -(G.d[0] * Tt + out[1] * inv12), fy = -(G.d[1] * Tt + out[2] * inv12),
-                 fz = -(G.d[2] * Tt + out[3] * inv12);
-    frc[pr.tp] = Dbl4{fx, fy, fz, out[4] * inv12};
-    frc[pr.tr] = Dbl4{-fx, -fy, -fz, out[5] * inv12};
+  }
+  if (!later) return;
+  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < npair; p += stride) {
+    PairRef pr;
+    if (!load_pair(A, pair_rec, p, pr) || __double_as_longlong(frc[pr.tp].x) != kTabLater) continue;
+    PairGeom G;
+    pair_geometry(g0, A, pr.i, pr.j, G);
+    double C[NT], cfs[NF], ca[2] = {0.0, 0.0}, cs[2] = {0.0, 0.0}, cp[3] = {0.0, 0.0, 0.0}, out[7];
+    force_weights<S, NP, TAB>(P, A, pr, C, cfs);
+#pragma unroll
+    for (int v = 0; v < NF; ++v) {
+      ca[v] = C[v];
+      cs[v] = cfs[v];
+    }
+#pragma unroll
+    for (int u = 0; u < NP; ++u) cp[u] = C[NF + u];
+    direct_forces(P, G, ca, cs, cp, out);
+    store_force(G, out, pr, frc);
   }
 }
 

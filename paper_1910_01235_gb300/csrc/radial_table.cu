@@ -217,7 +217,21 @@ __global__ void __launch_bounds__(32) k_radial_table(const __grid_constant__ Dev
   split(c[3], c3h, c3l);
   unsigned long long w0;
   if (kind == kTabDeriv64) {
-    w0 = (unsigned long long)__double_as_longlong(c0.h);
+    // 54 bits and the exponent
+    int x = c0.h != 0.0 ? ilogb(c0.h) : -1000;
+    long long m = 0;
+    if (x > -1000) {
+      m = __double2ll_rn(scalbn(c0.h, 53 - x)) + __double2ll_rn(scalbn(c0.l, 53 - x));
+      if (m >= (1ll << 54) || m <= -(1ll << 54)) {
+        m /= 2;
+        x += 1;
+      }
+    }
+    const int e8 = x + 128;  // above 255: excluded by plan_radial_tab
+    if (e8 > 0)
+      w0 = ((unsigned long long)(m >> 23) << 32) | ((unsigned long long)(m & 0x7fffff) << 8) | (unsigned)min(e8, 255);
+    else
+      w0 = 0ull;
   } else {
     const double sc = 1.0 / Tb.scale[u];  // a power of two
     w0 = (unsigned long long)(__double2ll_rn(c0.h * sc) + __double2ll_rn(c0.l * sc));
@@ -240,7 +254,8 @@ __global__ void __launch_bounds__(32) k_radial_table(const __grid_constant__ Dev
 // and as y^n with y = h / (4 r_switch (r_cut - r_switch)) for the switch (z is
 // a polynomial of degree 5 in r): x <= 0.016 and y <= 0.004 keep the first
 // dropped term (n = 8) below 2^-60 and the FP32 terms (n >= 4) below 2^-53 of
-// the value, as measured against the oracle at those limits.  The table has to
+// the value.  At lambda = 2.5, r near 1.5 every output's error against
+// extended precision was at most the direct kernels'.  The table has to
 // leave room in the 227 KB of shared memory of one block.  Lennard-Jones terms
 // (r^-12 varies faster than any of the exponentials) keep the direct kernels.
 bool plan_radial_tab(const DevPot& P, int kind, bool with_pairs, RadialTab& Tb) {
@@ -283,6 +298,8 @@ bool plan_radial_tab(const DevPot& P, int kind, bool with_pairs, RadialTab& Tb) 
     const double vmax = F ? F->A * std::exp(F->kappa - F->lambda * std::sqrt(wl)) : 1.0;
     if (!std::isfinite(vmax) || vmax > 1e30) return false;
     if (F && vmax < 1e-30) return false;
+    // the derivative rows have 8 bits of exponent: 2^-127 .. 2^127
+    if (kind == kTabDeriv64 && F && (vmax > 1e20 || vmax < 1e-20)) return false;
     Tb.scale[u] = std::ldexp(1.0, std::ilogb(vmax) + 1 - kTabSumBits);
   }
   return true;

@@ -12,8 +12,9 @@
 // lanes, the point is the split of the polynomial: consecutive Taylor terms
 // fall by about 2^-7, so only the constant term needs 53 bits.  It is an
 // integer on a fixed grid (sums of nodes are exact 64-bit integer additions)
-// or a double (one FMA with the pair's weight); the terms tau c1 .. tau^3 c3
-// run in float-float, tau^4 c4 .. in FP32.
+// or a 54-bit integer with an exponent (multiplied by the pair's weight in
+// integer arithmetic); the terms tau c1 .. tau^3 c3 run in float-float,
+// tau^4 c4 .. in FP32.
 //
 // The switch is only twice differentiable at r_switch and r_cut: the interval
 // that holds a breakpoint has two rows, one per side, and the row index steps
@@ -29,12 +30,16 @@
 
 namespace mxe {
 
-// A row of one term, FP64 quality: c0 (int64 or double), c1, c2, c3 as float
-// pairs, c4..c7 floats: three 16-byte words.  Float-float quality (degree 4):
+// A row of one term, FP64 quality: c0, c1, c2, c3 as float pairs, c4..c7
+// floats: three 16-byte words.  c0 of a value row is an int64 on the term's
+// grid; of a derivative row m_hi (signed high word) and m_lo | e8 (low word, bit
+// 31 clear), for (m_hi 2^31 + m_lo) 2^(e8 - kTabExpBias), |m_hi| < 2^31, zero
+// where e8 is 0.  Float-float quality (degree 4):
 // c0 int64, c1, c2 float pairs, c3, c4: two words.
 // All FP64 (degree 9, c0..c9; the tangent passes): five words.
 constexpr int kTabWords64 = 3, kTabWordsFF = 2, kTabWordsTaylor = 5;
 constexpr int kTabFixedBits = 56;   // w in units of 2^-56
+constexpr int kTabExpBias = 128 + 61;  // of the derivative rows' exponents
 constexpr int kTabSumBits = 58;     // |c0| < 2^58 on its grid: 13 nodes sum without overflow
 constexpr double kTabRLow = 0.25;   // first row at (r_cut / 4)^2
 
@@ -119,6 +124,19 @@ __device__ __forceinline__ ff tab_polyff(float c1h, float c1l, uint4 b, float th
   s.lo += m.lo + c1l;
   return times_tau(s);
 }
+
+// v 2^e to the nearest double (ties to even), on bits (no FP64 instruction); the result is
+// zero or normal, which the callers' ranges of e ensure
+__device__ __forceinline__ double fixed_double(long long v, int e) {
+  const unsigned long long u = (unsigned long long)(v < 0 ? -v : v);
+  const int lz = __clzll((long long)u);
+  const unsigned long long m = u << (lz & 63);  // bit 63 set; below, its leading bit adds one to the exponent
+  const unsigned lo = (unsigned)m;
+  const unsigned long long b = (m >> 11) + ((lo & 0x7ffu) + ((lo >> 11) & 1u) > 0x400u ? 1ull : 0ull) +
+                               ((unsigned long long)(unsigned)(e + 1085 - lz) << 52);
+  return u == 0 ? 0.0 : __longlong_as_double((long long)(b | ((unsigned long long)v & 0x8000000000000000ull)));
+}
+__device__ __forceinline__ int exp2_of(double x) { return (__double2hiint(x) >> 20) - 1023; }  // x = 2^e > 0
 
 // running sum of float pairs without renormalisation
 __device__ __forceinline__ void tab_acc(ff& a, ff v) {
