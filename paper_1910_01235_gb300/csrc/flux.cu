@@ -13,9 +13,9 @@
 // E_ik, Q_ik = x_iv / E_ik.  Across a bond whose two ends share the temperature,
 // J_{i->j} = P_ik Q_jk: one multiplication a hop (the FP64 pipe bounds the
 // gather; with separate factors a bond took 18 FP64 instructions per species
-// and 12 loads, now 4 and 2); a bond between different temperatures, or an E
-// outside the normal range (its Q holds a marker), takes the exponential of the
-// difference.  Each site gathers over its own bond row (no atomics,
+// and 12 loads, now 4 and 2); a bond between different temperatures, or a site
+// whose E, P or Q is outside the normal range (its Q holds a marker), takes the
+// exponential of the difference.  Each site gathers over its own bond row (no atomics,
 // deterministic).  A bond's net exchange is always formed by the same function
 // of the bond's canonical orientation (lower index first) with explicitly
 // rounded operations, so site j obtains exactly the negation of what site i
@@ -30,6 +30,9 @@ namespace {
 
 constexpr double kEMin = 1e-250, kEMax = 1e250;
 constexpr int kNotFactorised = 0x7ff80000;  // high word of a Q that must not be used
+__device__ __forceinline__ bool factor_ok(double v, bool zero) {
+  return zero ? v == 0.0 : fabs(v) > 1e-290 && fabs(v) < 1e290;
+}
 
 // Reservoirs (Sec. 4, fix setchemicalpotential / setatomicfraction): a site
 // of the chemical-potential group enters every rate with its held mu; a site of
@@ -67,9 +70,10 @@ __global__ void __launch_bounds__(256) k_flux_prep(const double* __restrict__ x,
     const double m = held ? res.fix_mu_value[k * n + i] : mu[k * n + i];
     if (res.mu_eff) res.mu_eff[k * n + i] = m;
     const double E = exp(beta * m);
-    const bool normal = E > kEMin && E < kEMax;
-    reinterpret_cast<double2*>(fl)[i * S + k] =
-        make_double2(D * x[k * n + i] * E, normal ? xv / E : __hiloint2double(kNotFactorised, 0));
+    const double xk = x[k * n + i], P = D * xk * E, Q = xv / E;
+    // neither product may leave the normal range where the hop itself does not
+    const bool normal = E > kEMin && E < kEMax && factor_ok(P, D == 0.0 || xk == 0.0) && factor_ok(Q, xv == 0.0);
+    reinterpret_cast<double2*>(fl)[i * S + k] = make_double2(P, normal ? Q : __hiloint2double(kNotFactorised, 0));
   }
 }
 
