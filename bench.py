@@ -159,8 +159,9 @@ def ops_per_pair(kernel, n_phi, n_f, S):
         return 13 * (node + term * n_f) + 300
     if kernel.startswith("gradient_ff"):
         return 12 * (node + term * (n_phi + n_f)) + (node + term * n_f) + 500
-    if kernel == "pair_ff":                 # once per unordered pair: 12 nodes x all terms + static f
-        return 12 * (node + term * (n_phi + n_f)) + (node + term * n_f) + 60
+    if kernel == "pair_ff":                 # once per unordered pair, table rows: 12 nodes x all terms + static f
+        row, poly = 4, 34                   # offset from the row's centre; degree-5 row in float-float and its sum
+        return 12 * (row + poly * (n_phi + n_f)) + (row + poly * n_f) + 60
     if kernel == "pair32_density":          # the FP32 density terms of one unordered pair (13 points)
         return 13 * (2 + 7 + 2 * n_f) + 20
     if kernel == "pair32_force":            # the FP32 forces of one unordered pair, both width derivatives

@@ -8,6 +8,13 @@
 // 2 needs the per-site coefficients a = x F''(rho_bar)(<rho> - rho_bar) and
 // b = x F'(rho_bar) of every neighbour.
 //
+// This file holds the passes over full rows (calls without unordered pairs),
+// the direct passes over unordered pairs for potentials without radial tables,
+// the direct exact embedding average, and the energy sums.  Elsewhere:
+// pair_table.cu (tabulated pair passes), pair_fp32.cu (relaxation passes of the
+// FP32 modes), gathers.cu (per-site sums), embed_table.cu (tabulated exact
+// embedding).
+//
 // Work split: a team of NL consecutive lanes owns one site and strides over
 // its neighbour row; each lane evaluates the 13 points of a pair unrolled in
 // registers; the team reduces its per-site sums with warp shuffles.  The
@@ -67,8 +74,7 @@ struct Traits<2> {
   using R = float;
   using Acc = AccFF;
 };
-// 3: float-float node arithmetic (about 48 bits), for the chemical-potential
-// passes of the FP32 modes; pair sums are added into FP64 per-site sums.
+// 3: float-float node arithmetic (about 48 bits; the accurate pass)
 template <>
 struct Traits<3> {
   using R = ff;
@@ -142,10 +148,6 @@ __device__ __forceinline__ void sw(const DevPot& P, ff r, ff& S, ff& dS) {
 // raw exponential part of a radial term
 __device__ __forceinline__ float rad_raw(const RadialFn& F, float r) { return ex2_approx(fmaf(-F.c1, r, F.c0)); }
 __device__ __forceinline__ double rad_raw(const RadialFn& F, double r) { return F.A * exp(F.kappa - F.lambda * r); }
-__device__ __forceinline__ ff rad_raw(const RadialFn& F, ff r) {
-  return ff_exp(F.lnA_kappa_ff - F.lambda_ff * r, c_exp_table);
-}
-__device__ __forceinline__ ff rad_lam(const RadialFn& F, ff) { return F.lambda_ff; }
 __device__ __forceinline__ float rad_lam(const RadialFn& F, float) { return F.lam_f; }
 __device__ __forceinline__ double rad_lam(const RadialFn& F, double) { return F.lambda; }
 
@@ -750,10 +752,10 @@ __global__ void __launch_bounds__(256, MXE_GRADIENT_MIN_BLOCKS) k_gradient(DevPo
 // unordered pair (one thread per pair) into a record of C values, written
 // to both entries of the pair:
 // [f_v static (n_f) | sum over the 12 nodes of f_v (n_f) | of phi_u (n_phi)];
-// k_pair_density / k_pair_mu gather the records over every site's full row
-// in row order and finish exactly as the density and chemical-potential
-// passes do.  Node arithmetic R: float-float (records of
-// float pairs; the FP32 modes) or FP64 (records of doubles).
+// gathers.cu sums the records over every site's full row in row order and
+// finishes with the site's terms.  Node arithmetic R: float-float (records of
+// float pairs; the FP32 modes) or FP64 (records of doubles).  Potentials with
+// radial tables take k_geo_tab (pair_table.cu) instead.
 template <typename R>
 struct GeoRec;
 template <>

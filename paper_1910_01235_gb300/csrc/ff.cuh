@@ -23,7 +23,6 @@ struct ff {
   __host__ __device__ explicit ff(double x) : hi((float)x), lo((float)(x - (double)(float)x)) {}
 };
 
-__device__ __forceinline__ ff ff_make(float h, float l = 0.f) { return ff{h, l}; }
 
 __device__ __forceinline__ ff two_sum(float a, float b) {
   const float s = a + b;

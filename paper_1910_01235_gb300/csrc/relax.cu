@@ -272,8 +272,8 @@ __global__ void __launch_bounds__(256) k_fire_update(double* __restrict__ q, dou
 // seg_blocks-th run; the system's last block to finish (a ticket in its
 // record) adds the partials in a fixed order, so the sums depend on the system
 // alone, not on the rest of the batch.
-// Bound by the FP64 pipe and the 72 bytes read a site: 512 systems of 3.5 to
-// 4 thousand sites, one block a system (every thread FP64 compares, four
+// Bound by the FP64 pipe and the 72 bytes read a site: 512 systems of 256 to
+// 16,384 sites (2.9 M), one block a system (every thread FP64 compares, four
 // systems an SM): 344 us; split, tests on bit patterns: 140 us.
 constexpr int kSegRun = 256, kSegSplitMax = 64;
 __host__ __device__ __forceinline__ int seg_blocks(int64_t sites) {
