@@ -28,11 +28,14 @@
 namespace mxe {
 namespace {
 
-constexpr double kEMin = 1e-250, kEMax = 1e250;
 constexpr int kNotFactorised = 0x7ff80000;  // high word of a Q that must not be used
-__device__ __forceinline__ bool factor_ok(double v, bool zero) {
-  return zero ? v == 0.0 : fabs(v) > 1e-290 && fabs(v) < 1e290;
+// tests on bits (no FP64 instruction): magnitude between 2^lo and 2^hi; zero
+__device__ __forceinline__ bool in_range(double v, int lo, int hi) {
+  const int e = ((__double2hiint(v) >> 20) & 0x7ff) - 1023;
+  return e >= lo && e < hi;
 }
+__device__ __forceinline__ bool is_zero(double v) { return ((unsigned long long)__double_as_longlong(v) << 1) == 0; }
+__device__ __forceinline__ bool factor_ok(double v, bool zero) { return zero ? is_zero(v) : in_range(v, -963, 963); }
 
 // Reservoirs (Sec. 4, fix setchemicalpotential / setatomicfraction): a site
 // of the chemical-potential group enters every rate with its held mu; a site of
@@ -72,7 +75,7 @@ __global__ void __launch_bounds__(256) k_flux_prep(const double* __restrict__ x,
     const double E = exp(beta * m);
     const double xk = x[k * n + i], P = D * xk * E, Q = xv / E;
     // neither product may leave the normal range where the hop itself does not
-    const bool normal = E > kEMin && E < kEMax && factor_ok(P, D == 0.0 || xk == 0.0) && factor_ok(Q, xv == 0.0);
+    const bool normal = in_range(E, -830, 830) && factor_ok(P, is_zero(D) || is_zero(xk)) && factor_ok(Q, is_zero(xv));
     reinterpret_cast<double2*>(fl)[i * S + k] = make_double2(P, normal ? Q : __hiloint2double(kNotFactorised, 0));
   }
 }
