@@ -860,13 +860,18 @@ mxe_status enqueue_passes(mxe_ctx* c, const mxe_state* s, PassArgs& A, bool want
   if (A.gq != nullptr || A.gs != nullptr) {
     PassArgs F = A;
     F.site_E = nullptr;  // energies already come from the accurate pass
-    // the relaxation's force pass: each unordered pair once, then the gather.
-    // Before the first relaxation its records go where the geometry records
-    // were (the gathers above have read them), so the call allocates nothing.
-    // Against the full-list kernel at 108,000 sites FP64: 19.0 -> 1.4 ms.
-    void* frc = half_list_forces(c) ? c->ent_frc : (void*)c->pair_buf;
-    CK(TIMED(relax_pair_name(true, prec), relax_pair_pass(c, true, PP, F, nullptr, frc)));
-    CK(TIMED(relax_gather_name(true, prec), launch_relax_gather(prec, true, c->nl, PP, F, nullptr, frc, st)));
+    if (hl) {
+      // the relaxation's force pass: each unordered pair once, then the gather.
+      // Before the first relaxation its records go where the geometry records
+      // were (the gathers above have read them), so the call allocates nothing.
+      // Against the full-list kernel at 108,000 sites FP64: 19.0 -> 1.2 ms.
+      void* frc = half_list_forces(c) ? c->ent_frc : (void*)c->pair_buf;
+      CK(TIMED(relax_pair_name(true, prec), relax_pair_pass(c, true, PP, F, nullptr, frc)));
+      CK(TIMED(relax_gather_name(true, prec), launch_relax_gather(prec, true, c->nl, PP, F, nullptr, frc, st)));
+    } else {  // no pair index (more density terms than the pair kernels hold)
+      CK(TIMED(cls_name("gradient", prec, kGradForceNoE),
+               launch_gradient(prec, kGradForceNoE, c->nl, PP, c->grid, F, st)));
+    }
   }
   // the accurate pass: the exact average in FP64
   return c->embedding ? enqueue_emb_exact(c, A, true) : MXE_OK;
