@@ -68,13 +68,13 @@ __device__ __forceinline__ long long tab_fixed(double x, int& big) {
 }
 
 // Row of w and the offset from the row's centre; `low` collects w below the
-// first row.  The index is clamped, so every access stays inside the table
-// whatever w is.
+// first row, and below zero (a node that falls on a site to rounding).  The
+// index is clamped, so every access stays inside the table whatever w is.
 __device__ __forceinline__ const uint4* tab_row(const RadialTab& Tb, const uint4* sm, long long w, float& th, float& tl,
                                                 int& low) {
   const unsigned hi = (unsigned)((unsigned long long)w >> 32), lo = (unsigned)w;
   int k = (int)(hi >> Tb.shift) - Tb.k_lo;
-  low |= k;  // negative below the first row
+  low |= k | (int)hi;  // negative below the first row; the high bit of a negative w
   k += hi >= Tb.rs_hi ? 1 : 0;
   if (hi >= Tb.rc_hi) k = Tb.nrow - 1;
   k = min(max(k, 0), Tb.nrow - 1);
