@@ -56,11 +56,12 @@ __device__ __forceinline__ int pair_nodes(const PairGeom& G, PairNodes& N) {
 }
 
 // float pair of x from its bits (no FP64 instruction): 24 bits, then the other
-// 29; magnitudes below 2^-75 give zero
+// 29; magnitudes below 2^-74 (a biased exponent of kNoFloatPair or less) give zero
+constexpr int kNoFloatPair = 948;
 __device__ __forceinline__ ff ff_bits(double x) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const int e = (int)((hi >> 20) & 0x7ff);
-  if (e <= 948) return ff{0.f, 0.f};
+  if (e <= kNoFloatPair) return ff{0.f, 0.f};
   const unsigned sign = hi & 0x80000000u;
   const float h = __uint_as_float(sign | ((unsigned)(e - 896) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
   const float sc = __uint_as_float(sign | ((unsigned)(e - 948) << 23));
@@ -392,10 +393,13 @@ struct FixedWeights {
   int terms;  // that are not zero
   ff f[NT];
 };
-// The integers' unit is 2^(the result); row: the row of the nearest node.
+// The integers' unit is 2^(the result); row: the row of the nearest node.  A
+// weight below 2^-74 has no float pair (ff_bits gives zero): the linear and
+// higher terms of its rows would be lost, at most 2^-6 of the term, so unless
+// the pair's largest term is over 2^50 times it the pair is evaluated directly.
 template <int NT>
 __device__ __forceinline__ int fixed_weights(const double* C, const uint4* row, FixedWeights<NT>& F, int& big) {
-  int top = 0;
+  int top = 0, faint = -1000;  // largest exponents of all terms and of those without a float pair
   F.terms = 0;
 #pragma unroll
   for (int u = 0; u < NT; ++u) {
@@ -415,8 +419,10 @@ __device__ __forceinline__ int fixed_weights(const double* C, const uint4* row, 
     if (e != 0 && e8 != 0) {
       top = max(top, e + e8);
       F.terms += 1;
+      if (e <= kNoFloatPair) faint = max(faint, e + e8);
     }
   }
+  big |= faint > top - 50;
 #pragma unroll
   for (int u = 0; u < NT; ++u) F.k[u] = top == 0 ? 1000 : top + F.kHead - F.k[u];  // top 0: every node beyond the cutoff
   // hi m_hi is a product shifted by 62: exponents e - 1082, e8 - kTabExpBias

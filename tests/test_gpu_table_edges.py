@@ -32,3 +32,23 @@ def test_status_of_a_node_on_a_site(precision):
     with pytest.raises(M.MxeError) as e:
         g.free_energy_grad()
     assert e.value.status == M.ERR_GEOMETRY
+
+
+@pytest.mark.parametrize("x", [2e-11, 6e-12, 1e-12, 4e-13, 1e-14, 1e-20])
+def test_fp64_forces_of_traces_alone(x):
+    """One species of traces without density: every weight of a pair is x^2, small
+    enough in the middle of this range to have no float pair while the integer
+    part still holds it.  The forces scale with x^2, so the bound is that of the
+    other FP64 passes, 1e-11 of the largest component."""
+    pot = W.potential_single()
+    pot.f_xi[:] = 0.0
+    pot.E[:] = 0.0
+    s = W.perturb(W.config_vacancy_lattice(4, pot=pot), 0.05, 0.02, seed=21)
+    s.x[:] = x
+    g = M.MxeSystem(s, "fp64")
+    g.build_neighbors()
+    g.free_energy_grad()
+    st, offs, idx = O.neighbors(s.q, s.L, g.r_list)
+    fe = O.free_energy(s, (offs, idx))
+    assert st == O.OK and fe["status"] == O.OK
+    assert np.abs(g.gq.cpu().numpy() - fe["gq"]).max() <= 1e-11 * np.abs(fe["gq"]).max()
