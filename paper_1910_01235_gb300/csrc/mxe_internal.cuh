@@ -108,7 +108,6 @@ struct RadialTab {
   int shift, k_lo;         // interval of w: (high word of w >> shift) - k_lo
   unsigned rs_hi, rc_hi;   // r_switch^2, r_cut^2 as high words
   double h;
-  double scale[5];         // value of one unit of the integer constant term
 };
 
 // Box / cell grid for positions and image codes.

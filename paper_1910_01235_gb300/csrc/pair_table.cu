@@ -55,6 +55,12 @@ __device__ __forceinline__ int pair_nodes(const PairGeom& G, PairNodes& N) {
   return big;
 }
 
+// the smallest of a pair's twelve squared node distances
+__device__ __forceinline__ long long nearest_node(const PairNodes& N) {
+  return min(N.base[0] - max(N.tw[0][0], max(N.tw[0][1], N.tw[0][2])),
+             N.base[1] - max(N.tw[1][0], max(N.tw[1][1], N.tw[1][2])));
+}
+
 // float pair of x from its bits (no FP64 instruction): 24 bits, then the other
 // 29; magnitudes below 2^-74 (a biased exponent of kNoFloatPair or less) give zero
 constexpr int kNoFloatPair = 948;
@@ -131,22 +137,25 @@ __device__ __noinline__ void direct_forces(const DevPot& P, const PairGeom& G, c
 }
 
 // ---------------------------------------------------------------- geometry records
-// a sum of nodes: integer constant terms and the float pair of the rest
+// a sum of nodes: integer constant terms in units of 2^(k - kTabValueBias) and
+// the float pair of the rest
 struct NodeSum {
   long long c;
   ff p;
+  int k;
 };
-__device__ __forceinline__ double sum_value(const NodeSum& v, double scale, double*) {
-  return fixed_double(v.c, exp2_of(scale)) + (widen(v.p.hi) + widen(v.p.lo));
+constexpr int kSumHead = 5;  // bits above the nearest node's constant term: 12 nodes sum below 2^62
+__device__ __forceinline__ double sum_value(const NodeSum& v, double*) {
+  return fixed_double(v.c, v.k - kTabValueBias) + (widen(v.p.hi) + widen(v.p.lo));
 }
-__device__ __forceinline__ ff sum_value(const NodeSum& v, double scale, ff*) {
+__device__ __forceinline__ ff sum_value(const NodeSum& v, ff*) {
   // |c| < 2^62: the high word as a float, then what it left
   const int h = (int)(v.c >> 32);
   const float fh = (float)h;
   const long long rest = v.c - ((long long)(int)fh << 32);  // below 2^39
-  const float fl = (float)(int)(rest >> 8);
-  const float s = (float)scale;
-  return ff{fh * (s * 4294967296.0f), fl * (s * 256.0f)} + v.p;
+  const float fl = (float)(int)((rest + 128) >> 8);
+  const float s = exp2f_bits(v.k - 128);  // k from 6 on; the units are below the floats' range
+  return ff{fh * 0x1p-30f * s, fl * 0x1p-54f * s} + v.p;
 }
 
 template <typename R>
@@ -173,18 +182,45 @@ struct GeoOut<double> {
   static __device__ __forceinline__ double from(double v) { return v; }
 };
 
-template <int FIRST, int LAST, int W, bool FFQ>
+__device__ __forceinline__ long long row_integer(uint4 a) {
+  return (long long)(((unsigned long long)a.y << 32) | (a.x & 0xffffff00u));
+}
+template <int W, bool FFQ>
+__device__ __forceinline__ ff row_rest(uint4 a, const uint4* t, float th, float tl) {
+  if constexpr (FFQ) return tab_polyff(__uint_as_float(a.z), __uint_as_float(a.w), t[1], th, tl);
+  else return tab_poly64(__uint_as_float(a.z), __uint_as_float(a.w), t[1], t[2], th, tl);
+}
+// the terms at one point, each on its own row's grid
+template <int N, int W, bool FFQ>
+__device__ __forceinline__ void one_node(const RadialTab& Tb, const uint4* sm, long long w, int& low, NodeSum* s) {
+  float th, tl;
+  const uint4* row = tab_row(Tb, sm, w, th, tl, low);
+#pragma unroll
+  for (int u = 0; u < N; ++u) {
+    const uint4 a = row[u * W];
+    s[u] = NodeSum{row_integer(a) >> kSumHead, row_rest<W, FFQ>(a, row + u * W, th, tl), (int)(a.x & 0xffu) + kSumHead};
+  }
+}
+// empty sums on the grid of the pair's nearest node, where the terms are largest
+template <int N, int W>
+__device__ __forceinline__ void start_sums(const RadialTab& Tb, const uint4* sm, const PairNodes& D, int& low,
+                                           NodeSum* s) {
+  float th, tl;
+  const uint4* row = tab_row(Tb, sm, nearest_node(D), th, tl, low);
+#pragma unroll
+  for (int u = 0; u < N; ++u) s[u] = NodeSum{0, ff{0.f, 0.f}, (int)(row[u * W].x & 0xffu) + kSumHead};
+}
+template <int N, int W, bool FFQ>
 __device__ __forceinline__ void add_node(const RadialTab& Tb, const uint4* sm, long long w, int& low, NodeSum* s) {
   float th, tl;
   const uint4* row = tab_row(Tb, sm, w, th, tl, low);
 #pragma unroll
-  for (int u = FIRST; u < LAST; ++u) {
-    const uint4 a = row[u * W], b = row[u * W + 1];
-    ff p;
-    if constexpr (FFQ) p = tab_polyff(__uint_as_float(a.z), __uint_as_float(a.w), b, th, tl);
-    else p = tab_poly64(__uint_as_float(a.z), __uint_as_float(a.w), b, row[u * W + 2], th, tl);
-    s[u].c += (long long)(((unsigned long long)a.y << 32) | a.x);
-    tab_acc(s[u].p, p);
+  for (int u = 0; u < N; ++u) {
+    const uint4 a = row[u * W];
+    const int sh = s[u].k - (int)(a.x & 0xffu);
+    low |= sh;  // negative: over 2^5 times the nearest node's (no table has that)
+    s[u].c += shift_right(row_integer(a), sh);
+    tab_acc(s[u].p, row_rest<W, FFQ>(a, row + u * W, th, tl));
   }
 }
 
@@ -216,23 +252,19 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_geo_tab(
     const int big = pair_nodes(G, N);
     int low = 0;
     NodeSum s[NT];
-#pragma unroll
-    for (int u = 0; u < NT; ++u) s[u] = NodeSum{0, ff{0.f, 0.f}};
-    add_node<0, NF, W, O::kFF>(Tb, sm, N.w0, low, s);
+    one_node<NF, W, O::kFF>(Tb, sm, N.w0, low, s);
     R val[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) val[c] = (R)0;
 #pragma unroll
-    for (int v = 0; v < NF; ++v) {
-      val[v] = sum_value(s[v], Tb.scale[v], (R*)nullptr);
-      s[v] = NodeSum{0, ff{0.f, 0.f}};
-    }
+    for (int v = 0; v < NF; ++v) val[v] = sum_value(s[v], (R*)nullptr);
+    start_sums<NT, W>(Tb, sm, N, low, s);
 #pragma unroll 1
     for (int site = 0; site < 2; ++site) {
 #pragma unroll 1
       for (int a = 0; a < 3; ++a) {
-        add_node<0, NT, W, O::kFF>(Tb, sm, N.base[0] + N.tw[0][0], low, s);
-        add_node<0, NT, W, O::kFF>(Tb, sm, N.base[0] - N.tw[0][0], low, s);
+        add_node<NT, W, O::kFF>(Tb, sm, N.base[0] + N.tw[0][0], low, s);
+        add_node<NT, W, O::kFF>(Tb, sm, N.base[0] - N.tw[0][0], low, s);
         // the next axis (registers rotate: one copy of the node code)
         const long long t = N.tw[0][0];
         N.tw[0][0] = N.tw[0][1];
@@ -244,9 +276,9 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_geo_tab(
       for (int a = 0; a < 3; ++a) N.tw[0][a] = N.tw[1][a];
     }
 #pragma unroll
-    for (int v = 0; v < NF; ++v) val[NF + v] = sum_value(s[v], Tb.scale[v], (R*)nullptr);
+    for (int v = 0; v < NF; ++v) val[NF + v] = sum_value(s[v], (R*)nullptr);
 #pragma unroll
-    for (int u = 0; u < NP; ++u) val[2 * NF + u] = sum_value(s[NF + u], Tb.scale[NF + u], (R*)nullptr);
+    for (int u = 0; u < NP; ++u) val[2 * NF + u] = sum_value(s[NF + u], (R*)nullptr);
     if (big || low < 0) {
       double st[2], av[2], ph[3];
       const PairGeom H = G;
@@ -316,27 +348,23 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_rdensity_tab(
     int low = 0;
     NodeSum s[NF];
     double fst[NF], fav[NF];
+    one_node<NF, W, false>(Tb, sm, N.w0, low, s);
 #pragma unroll
-    for (int v = 0; v < NF; ++v) s[v] = NodeSum{0, ff{0.f, 0.f}};
-    add_node<0, NF, W, false>(Tb, sm, N.w0, low, s);
-#pragma unroll
-    for (int v = 0; v < NF; ++v) {
-      fst[v] = sum_value(s[v], Tb.scale[v], (double*)nullptr);
-      s[v] = NodeSum{0, ff{0.f, 0.f}};
-    }
+    for (int v = 0; v < NF; ++v) fst[v] = sum_value(s[v], (double*)nullptr);
+    start_sums<NF, W>(Tb, sm, N, low, s);
 #pragma unroll 1
     for (int site = 0; site < 2; ++site) {
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        add_node<0, NF, W, false>(Tb, sm, N.base[0] + N.tw[0][a], low, s);
-        add_node<0, NF, W, false>(Tb, sm, N.base[0] - N.tw[0][a], low, s);
+        add_node<NF, W, false>(Tb, sm, N.base[0] + N.tw[0][a], low, s);
+        add_node<NF, W, false>(Tb, sm, N.base[0] - N.tw[0][a], low, s);
       }
       N.base[0] = N.base[1];
 #pragma unroll
       for (int a = 0; a < 3; ++a) N.tw[0][a] = N.tw[1][a];
     }
 #pragma unroll
-    for (int v = 0; v < NF; ++v) fav[v] = sum_value(s[v], Tb.scale[v], (double*)nullptr);
+    for (int v = 0; v < NF; ++v) fav[v] = sum_value(s[v], (double*)nullptr);
     if (big || low < 0) {
       double st[2], av[2], ph[3];
       const PairGeom H = G;
@@ -430,15 +458,6 @@ __device__ __forceinline__ int fixed_weights(const double* C, const uint4* row, 
   // 2^(-24 - unit) has to be a float
   big |= unit > 90 || unit < -140;
   return unit;
-}
-
-__device__ __forceinline__ float exp2f_bits(int e) { return __uint_as_float((unsigned)(e + 127) << 23); }  // |e| < 127
-
-// v >> n, all sign bits from n = 64 on (PTX clamps the count)
-__device__ __forceinline__ long long shift_right(long long v, int n) {
-  long long r;
-  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
-  return r;
 }
 
 // dV/dr / r of the pair's weighted terms at one node, in units of the pair's
@@ -569,8 +588,7 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_rforce_tab(
       const long long h = force_node<NF>(Tb, sm, N.w0, F, exp2f_bits(-24 - unit), low);
       out[6] = fixed_double(h != 0 ? h + (F.terms >> 1) : 0, unit);
     }
-    const long long near = min(N.base[0] - max(N.tw[0][0], max(N.tw[0][1], N.tw[0][2])),
-                               N.base[1] - max(N.tw[1][0], max(N.tw[1][1], N.tw[1][2])));
+    const long long near = nearest_node(N);
     FixedWeights<NT> F;
     const int unit = fixed_weights<NT>(C, tab_row(Tb, sm, near, th, tl, low), F, big);
     const float sc = exp2f_bits(-24 - unit);

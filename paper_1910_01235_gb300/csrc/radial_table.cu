@@ -215,26 +215,22 @@ __global__ void __launch_bounds__(32) k_radial_table(const __grid_constant__ Dev
   c1lf = (float)((c[1] - (double)c1h) + c1l);
   split(c[2], c2h, c2l);
   split(c[3], c3h, c3l);
-  unsigned long long w0;
-  if (kind == kTabDeriv64) {
-    // 54 bits and the exponent
-    int x = c0.h != 0.0 ? ilogb(c0.h) : -1000;
-    long long m = 0;
-    if (x > -1000) {
-      m = __double2ll_rn(scalbn(c0.h, 53 - x)) + __double2ll_rn(scalbn(c0.l, 53 - x));
-      if (m >= (1ll << 54) || m <= -(1ll << 54)) {
-        m /= 2;
-        x += 1;
-      }
+  // the leading bits (derivatives 54, values 55) and the exponent
+  unsigned long long w0 = 0ull;
+  const int top = kind == kTabDeriv64 ? 53 : 54;
+  if (c0.h != 0.0) {
+    int x = ilogb(c0.h);
+    long long m = __double2ll_rn(scalbn(c0.h, top - x)) + __double2ll_rn(scalbn(c0.l, top - x));
+    if (m >= (2ll << top) || m <= -(2ll << top)) {
+      m /= 2;
+      x += 1;
     }
     const int e8 = x + 128;  // above 255: excluded by plan_radial_tab
-    if (e8 > 0)
-      w0 = ((unsigned long long)(m >> 23) << 32) | ((unsigned long long)(m & 0x7fffff) << 8) | (unsigned)min(e8, 255);
-    else
-      w0 = 0ull;
-  } else {
-    const double sc = 1.0 / Tb.scale[u];  // a power of two
-    w0 = (unsigned long long)(__double2ll_rn(c0.h * sc) + __double2ll_rn(c0.l * sc));
+    if (e8 > 0) {
+      if (kind == kTabDeriv64) w0 = ((unsigned long long)(m >> 23) << 32) | ((unsigned long long)(m & 0x7fffff) << 8);
+      else w0 = (unsigned long long)m << 8;
+      w0 |= (unsigned)min(e8, 255);
+    }
   }
   out[0] = make_uint4((unsigned)w0, (unsigned)(w0 >> 32), bits(c1h), bits(c1lf));
   if (kind == kTabValueFF) {
@@ -298,9 +294,10 @@ bool plan_radial_tab(const DevPot& P, int kind, bool with_pairs, RadialTab& Tb) 
     const double vmax = F ? F->A * std::exp(F->kappa - F->lambda * std::sqrt(wl)) : 1.0;
     if (!std::isfinite(vmax) || vmax > 1e30) return false;
     if (F && vmax < 1e-30) return false;
-    // the derivative rows have 8 bits of exponent: 2^-127 .. 2^127
-    if (kind == kTabDeriv64 && F && (vmax > 1e20 || vmax < 1e-20)) return false;
-    Tb.scale[u] = std::ldexp(1.0, std::ilogb(vmax) + 1 - kTabSumBits);
+    // the other rows have 8 bits of exponent, 2^-127 .. 2^127; from the first row
+    // to the last a term falls by less than 2^55 within the limits above
+    if (!taylor && F && vmax < 1e-20) return false;
+    if (kind == kTabDeriv64 && F && vmax > 1e20) return false;
   }
   return true;
 }

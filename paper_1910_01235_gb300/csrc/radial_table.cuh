@@ -11,10 +11,13 @@
 // the node loop.  On GB300, whose FP64 pipe has 2 lanes per SM against 128 FP32
 // lanes, the point is the split of the polynomial: consecutive Taylor terms
 // fall by about 2^-7, so only the constant term needs 53 bits.  It is an
-// integer on a fixed grid (sums of nodes are exact 64-bit integer additions)
-// or a 54-bit integer with an exponent (multiplied by the pair's weight in
-// integer arithmetic); the terms tau c1 .. tau^3 c3 run in float-float,
-// tau^4 c4 .. in FP32.
+// integer with the exponent of its own row: 55 bits for values (shifted to the
+// grid of the pair's nearest node and added in 64-bit integers), 54 bits for
+// derivatives (multiplied by the pair's weight in integer arithmetic first); the
+// terms tau c1 .. tau^3 c3 run in float-float, tau^4 c4 .. in FP32.  One grid for
+// all rows, set by the value at r_cut / 4, left the outer shells short of bits:
+// with every neighbour at 4.95 A (r_cut 5, decay rate 1.96 / A) the energy was off
+// by 5e-14 in FP64 and 2e-12 in float-float, 3e-15 and 9e-14 direct.
 //
 // The switch is only twice differentiable at r_switch and r_cut: the interval
 // that holds a breakpoint has two rows, one per side, and the row index steps
@@ -31,16 +34,17 @@
 namespace mxe {
 
 // A row of one term, FP64 quality: c0, c1, c2, c3 as float pairs, c4..c7
-// floats: three 16-byte words.  c0 of a value row is an int64 on the term's
-// grid; of a derivative row m_hi (signed high word) and m_lo | e8 (low word, bit
-// 31 clear), for (m_hi 2^31 + m_lo) 2^(e8 - kTabExpBias), |m_hi| < 2^31, zero
-// where e8 is 0.  Float-float quality (degree 4):
-// c0 int64, c1, c2 float pairs, c3, c4: two words.
+// floats: three 16-byte words.  c0 of a value row is an int64 m with its low byte
+// e8 in place of its own, for (m & ~255) 2^(e8 - kTabValueBias), 2^62 <= |m| <
+// 2^63; of a derivative row m_hi (signed high word) and m_lo | e8 (low word, bit
+// 31 clear), for (m_hi 2^31 + m_lo) 2^(e8 - kTabExpBias), |m_hi| < 2^31; both
+// zero where e8 is 0.  Float-float quality (degree 5): c0, c1 and c2 pairs, c3,
+// c4, c5 (tab_polyff): two words.
 // All FP64 (degree 9, c0..c9; the tangent passes): five words.
 constexpr int kTabWords64 = 3, kTabWordsFF = 2, kTabWordsTaylor = 5;
 constexpr int kTabFixedBits = 56;   // w in units of 2^-56
-constexpr int kTabExpBias = 128 + 61;  // of the derivative rows' exponents
-constexpr int kTabSumBits = 58;     // |c0| < 2^58 on its grid: 13 nodes sum without overflow
+constexpr int kTabExpBias = 128 + 61;    // of the derivative rows' exponents
+constexpr int kTabValueBias = 128 + 62;  // of the value rows' exponents
 constexpr double kTabRLow = 0.25;   // first row at (r_cut / 4)^2
 
 // 16-byte words between the rows of consecutive intervals: all terms of an
@@ -136,7 +140,14 @@ __device__ __forceinline__ double fixed_double(long long v, int e) {
                                ((unsigned long long)(unsigned)(e + 1085 - lz) << 52);
   return u == 0 ? 0.0 : __longlong_as_double((long long)(b | ((unsigned long long)v & 0x8000000000000000ull)));
 }
-__device__ __forceinline__ int exp2_of(double x) { return (__double2hiint(x) >> 20) - 1023; }  // x = 2^e > 0
+__device__ __forceinline__ float exp2f_bits(int e) { return __uint_as_float((unsigned)(e + 127) << 23); }  // |e| < 127
+
+// v >> n, all sign bits from n = 64 on (PTX clamps the count)
+__device__ __forceinline__ long long shift_right(long long v, int n) {
+  long long r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+}
 
 // running sum of float pairs without renormalisation
 __device__ __forceinline__ void tab_acc(ff& a, ff v) {

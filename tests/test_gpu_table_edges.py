@@ -52,3 +52,21 @@ def test_fp64_forces_of_traces_alone(x):
     fe = O.free_energy(s, (offs, idx))
     assert st == O.OK and fe["status"] == O.OK
     assert np.abs(g.gq.cpu().numpy() - fe["gq"]).max() <= 1e-11 * np.abs(fe["gq"]).max()
+
+
+@pytest.mark.parametrize("scale", [1e-18, 1e-22, 1e-28, 2e-29])
+@pytest.mark.parametrize("precision", ["mixed", "ff"])
+def test_faint_pair_terms(scale, precision):
+    """A pair term too small for the exponents of a table's rows, alone:
+    chemical potentials relative to their own size (float-float terms, 1e-11)."""
+    pot = W.potential_single(A=0.3 * scale)
+    pot.f_xi[:] = 0.0
+    pot.E[:] = 0.0
+    s = W.perturb(W.config_vacancy_lattice(4, pot=pot), 0.05, 0.02, seed=22)
+    g = M.MxeSystem(s, precision)
+    g.build_neighbors()
+    g.free_energy_grad()
+    st, offs, idx = O.neighbors(s.q, s.L, g.r_list)
+    fe = O.free_energy(s, (offs, idx))
+    assert st == O.OK and fe["status"] == O.OK
+    assert np.abs(g.mu_ex.cpu().numpy() - fe["mu_ex"]).max() <= 1e-11 * np.abs(fe["mu_ex"]).max()
