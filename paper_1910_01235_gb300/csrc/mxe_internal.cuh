@@ -106,7 +106,9 @@ struct RadialTab {
   int nrow, stride, words;
   int nf_slots, np_slots;  // terms of a row: density, then pair terms (absent ones are zero)
   int shift, k_lo;         // interval of w: (high word of w >> shift) - k_lo
+  int n_main;              // rows of width h; the rest to the cutoff a quarter as wide (float-float rows)
   unsigned rs_hi, rc_hi;   // r_switch^2, r_cut^2 as high words
+  unsigned near_hi;        // where the narrow rows begin
   double h;
 };
 

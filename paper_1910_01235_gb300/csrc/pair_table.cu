@@ -194,7 +194,7 @@ __device__ __forceinline__ ff row_rest(uint4 a, const uint4* t, float th, float 
 template <int N, int W, bool FFQ>
 __device__ __forceinline__ void one_node(const RadialTab& Tb, const uint4* sm, long long w, int& low, NodeSum* s) {
   float th, tl;
-  const uint4* row = tab_row(Tb, sm, w, th, tl, low);
+  const uint4* row = tab_row<FFQ>(Tb, sm, w, th, tl, low);
 #pragma unroll
   for (int u = 0; u < N; ++u) {
     const uint4 a = row[u * W];
@@ -202,18 +202,18 @@ __device__ __forceinline__ void one_node(const RadialTab& Tb, const uint4* sm, l
   }
 }
 // empty sums on the grid of the pair's nearest node, where the terms are largest
-template <int N, int W>
+template <int N, int W, bool FFQ>
 __device__ __forceinline__ void start_sums(const RadialTab& Tb, const uint4* sm, const PairNodes& D, int& low,
                                            NodeSum* s) {
   float th, tl;
-  const uint4* row = tab_row(Tb, sm, nearest_node(D), th, tl, low);
+  const uint4* row = tab_row<FFQ>(Tb, sm, nearest_node(D), th, tl, low);
 #pragma unroll
   for (int u = 0; u < N; ++u) s[u] = NodeSum{0, ff{0.f, 0.f}, (int)(row[u * W].x & 0xffu) + kSumHead};
 }
 template <int N, int W, bool FFQ>
 __device__ __forceinline__ void add_node(const RadialTab& Tb, const uint4* sm, long long w, int& low, NodeSum* s) {
   float th, tl;
-  const uint4* row = tab_row(Tb, sm, w, th, tl, low);
+  const uint4* row = tab_row<FFQ>(Tb, sm, w, th, tl, low);
 #pragma unroll
   for (int u = 0; u < N; ++u) {
     const uint4 a = row[u * W];
@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_geo_tab(
     for (int c = 0; c < 8; ++c) val[c] = (R)0;
 #pragma unroll
     for (int v = 0; v < NF; ++v) val[v] = sum_value(s[v], (R*)nullptr);
-    start_sums<NT, W>(Tb, sm, N, low, s);
+    start_sums<NT, W, O::kFF>(Tb, sm, N, low, s);
 #pragma unroll 1
     for (int site = 0; site < 2; ++site) {
 #pragma unroll 1
@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_rdensity_tab(
     one_node<NF, W, false>(Tb, sm, N.w0, low, s);
 #pragma unroll
     for (int v = 0; v < NF; ++v) fst[v] = sum_value(s[v], (double*)nullptr);
-    start_sums<NF, W>(Tb, sm, N, low, s);
+    start_sums<NF, W, false>(Tb, sm, N, low, s);
 #pragma unroll 1
     for (int site = 0; site < 2; ++site) {
 #pragma unroll
@@ -467,7 +467,7 @@ template <int NT>
 __device__ __forceinline__ long long force_node(const RadialTab& Tb, const uint4* sm, long long w,
                                                 const FixedWeights<NT>& F, float sc, int& low) {
   float th, tl;
-  const uint4* row = tab_row(Tb, sm, w, th, tl, low);
+  const uint4* row = tab_row<false>(Tb, sm, w, th, tl, low);
   long long h = 0;
   ff p{0.f, 0.f};
 #pragma unroll
@@ -584,13 +584,13 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_rforce_tab(
     float th, tl;
     {
       FixedWeights<NF> F;
-      const int unit = fixed_weights<NF>(cfs, tab_row(Tb, sm, N.w0, th, tl, low), F, big);
+      const int unit = fixed_weights<NF>(cfs, tab_row<false>(Tb, sm, N.w0, th, tl, low), F, big);
       const long long h = force_node<NF>(Tb, sm, N.w0, F, exp2f_bits(-24 - unit), low);
       out[6] = fixed_double(h != 0 ? h + (F.terms >> 1) : 0, unit);
     }
     const long long near = nearest_node(N);
     FixedWeights<NT> F;
-    const int unit = fixed_weights<NT>(C, tab_row(Tb, sm, near, th, tl, low), F, big);
+    const int unit = fixed_weights<NT>(C, tab_row<false>(Tb, sm, near, th, tl, low), F, big);
     const float sc = exp2f_bits(-24 - unit);
     long long T = 0;
     double U[3] = {0.0, 0.0, 0.0}, V0 = 0.0, ad[3] = {fabs(G.d[0]), fabs(G.d[1]), fabs(G.d[2])};

@@ -176,12 +176,12 @@ __global__ void __launch_bounds__(32) k_radial_table(const __grid_constant__ Dev
     for (int t = 0; t < Tb.words; ++t) out[t] = make_uint4(0, 0, 0, 0);
     return;
   }
-  const double h = Tb.h;
   // rows step by one at r_switch^2: its interval has a row for each side
   const int ks = (int)(Tb.rs_hi >> Tb.shift) - Tb.k_lo;
-  const bool beyond = row > ks;
-  const int k = row - (beyond ? 1 : 0);
-  const double wc = ((double)(k + Tb.k_lo) + 0.5) * h;
+  const bool beyond = row > ks, narrow = row >= Tb.n_main;
+  const double h = narrow ? Tb.h / (1 << kTabNarrow) : Tb.h;
+  const int k = narrow ? row - Tb.n_main + (int)(Tb.near_hi >> (Tb.shift - kTabNarrow)) : row - (beyond ? 1 : 0) + Tb.k_lo;
+  const double wc = ((double)k + 0.5) * h;
   dd V0, V1, V2;
   double V[kDeg + 1];
   term_series(*F, wc, h, beyond, P.rs, P.rc, V0, V1, V2, V);
@@ -284,7 +284,19 @@ bool plan_radial_tab(const DevPot& P, int kind, bool with_pairs, RadialTab& Tb) 
   Tb.rs_hi = (unsigned)std::floor(P.rs * P.rs * unit);
   Tb.rc_hi = (unsigned)std::ceil(rc2 * unit);
   if ((int)(Tb.rs_hi >> Tb.shift) < Tb.k_lo) return false;
-  Tb.nrow = (int)((Tb.rc_hi - 1) >> Tb.shift) - Tb.k_lo + 3;  // both sides of r_switch, and the zeros
+  Tb.n_main = (int)((Tb.rc_hi - 1) >> Tb.shift) - Tb.k_lo + 2;  // both sides of r_switch
+  Tb.nrow = Tb.n_main + 1;                                        // and the zeros
+  Tb.near_hi = 0xffffffffu;
+  if (kind == kTabValueFF) {
+    const double rn = P.rc - kTabNearU * (P.rc - P.rs);
+    const unsigned kn = std::max((unsigned)std::floor(rn * rn / h), (Tb.rs_hi >> Tb.shift) + 1u);
+    if (kn <= (Tb.rc_hi - 1) >> Tb.shift) {
+      Tb.near_hi = kn << Tb.shift;
+      Tb.n_main = (int)kn - Tb.k_lo + 1;
+      const int sh = Tb.shift - kTabNarrow;
+      Tb.nrow = Tb.n_main + (int)((Tb.rc_hi - 1) >> sh) - (int)(Tb.near_hi >> sh) + 2;
+    }
+  }
   if ((int64_t)Tb.nrow * Tb.stride * 16 > kTabMaxBytes) return false;
   for (int u = 0; u < Tb.nf_slots + Tb.np_slots; ++u) {
     const int f = u, p = u - Tb.nf_slots;

@@ -46,6 +46,13 @@ constexpr int kTabFixedBits = 56;   // w in units of 2^-56
 constexpr int kTabExpBias = 128 + 61;    // of the derivative rows' exponents
 constexpr int kTabValueBias = 128 + 62;  // of the value rows' exponents
 constexpr double kTabRLow = 0.25;   // first row at (r_cut / 4)^2
+// Float-float rows hold c2 to 32 and c3, c5 to 24 and 8 bits.  Where the switch
+// u = (r_cut - r) / (r_cut - r_switch) falls to the offset's share du of it, the
+// terms are (du / u)^n of the value and those bits show (at u = 0.1, 4.95 A of 5:
+// 1e-12 of the value, the direct kernels 1e-13).  Rows a quarter as wide from
+// u = 0.3 on: du^2 / 16.
+constexpr int kTabNarrow = 2;
+constexpr double kTabNearU = 0.3;
 
 // 16-byte words between the rows of consecutive intervals: all terms of an
 // interval lie side by side; an odd count spreads random intervals over the
@@ -74,16 +81,23 @@ __device__ __forceinline__ long long tab_fixed(double x, int& big) {
 // Row of w and the offset from the row's centre; `low` collects w below the
 // first row, and below zero (a node that falls on a site to rounding).  The
 // index is clamped, so every access stays inside the table whatever w is.
+// NARROW: the table has narrow rows before the cutoff.
+template <bool NARROW>
 __device__ __forceinline__ const uint4* tab_row(const RadialTab& Tb, const uint4* sm, long long w, float& th, float& tl,
                                                 int& low) {
   const unsigned hi = (unsigned)((unsigned long long)w >> 32), lo = (unsigned)w;
-  int k = (int)(hi >> Tb.shift) - Tb.k_lo;
+  int sh = Tb.shift, first = -Tb.k_lo;
+  if (NARROW && hi >= Tb.near_hi) {
+    sh -= kTabNarrow;
+    first = Tb.n_main - 1 - (int)(Tb.near_hi >> sh);
+  }
+  int k = (int)(hi >> sh) + first;
   low |= k | (int)hi;  // negative below the first row; the high bit of a negative w
   k += hi >= Tb.rs_hi ? 1 : 0;
   if (hi >= Tb.rc_hi) k = Tb.nrow - 1;
   k = min(max(k, 0), Tb.nrow - 1);
-  const unsigned f1 = __funnelshift_r(lo, hi, Tb.shift + 9) & 0x7fffffu;
-  const unsigned f2 = (lo >> (Tb.shift - 14)) & 0x7fffffu;
+  const unsigned f1 = __funnelshift_r(lo, hi, sh + 9) & 0x7fffffu;
+  const unsigned f2 = (lo >> (sh - 14)) & 0x7fffffu;
   th = __uint_as_float(0x3f800000u | f1) - 1.5f;
   // the next 23 bits, at the middle of what they truncate
   tl = fmaf(__uint_as_float(0x3f800000u | f2), 0x1p-23f, -0x1p-23f * (1.0f - 0x1p-24f));

@@ -89,3 +89,14 @@ def test_fp64(half, lam, density):
 def test_float_float(half, lam, density, precision):
     off, _, S = error(half, lam, density, precision)
     assert S >= 0.3 and off <= 2.0**-44
+
+
+@pytest.mark.parametrize("precision", ["mixed", "ff"])
+@pytest.mark.parametrize("density", [True, False])
+@pytest.mark.parametrize("lam", [1.2, 1.96, 2.5])
+@pytest.mark.parametrize("half", [3.453125, 3.484375, 3.5, 3.515625])
+def test_float_float_before_the_cutoff(half, lam, density, precision):
+    """Where the switch S is small: within the float-float rounding of 1 - S, 2^-47
+    of the unswitched term."""
+    off, _, S = error(half, lam, density, precision)
+    assert S < 0.1 and off <= 2.0**-47 / S
