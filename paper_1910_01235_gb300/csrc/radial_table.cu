@@ -250,7 +250,9 @@ __global__ void __launch_bounds__(32) k_radial_table(const __grid_constant__ Dev
 // and as y^n with y = h / (4 r_switch (r_cut - r_switch)) for the switch (z is
 // a polynomial of degree 5 in r): x <= 0.016 and y <= 0.004 keep the first
 // dropped term (n = 8) below 2^-60 and the FP32 terms (n >= 4) below 2^-53 of
-// the value.  At lambda = 2.5, r near 1.5 every output's error against
+// the value, provided r = sqrt(w) itself converges: its terms fall as (h / 2w)^n,
+// 1/100 at kTabRMin (at r = 0.7, for a cut-off of 2.8 A, 1/31 left 4e-14 of the
+// value in FP64).  At lambda = 2.5, r near 1.5 every output's error against
 // extended precision was at most the direct kernels'.  The table has to
 // leave room in the 227 KB of shared memory of one block.  Lennard-Jones terms
 // (r^-12 varies faster than any of the exponentials) keep the direct kernels.
@@ -270,7 +272,7 @@ bool plan_radial_tab(const DevPot& P, int kind, bool with_pairs, RadialTab& Tb) 
   // all-FP64 rows of degree 9 afford intervals twice as wide
   const bool taylor = kind == kTabTaylor64;
   const int bits_h = taylor ? 4 : 5;
-  const double h = std::ldexp(1.0, -bits_h), r_lo = kTabRLow * P.rc, wide = taylor ? 2.0 : 1.0;
+  const double h = std::ldexp(1.0, -bits_h), r_lo = std::max(kTabRLow * P.rc, kTabRMin), wide = taylor ? 2.0 : 1.0;
   if (!(lam * h <= 0.016 * wide * 4.0 * r_lo)) return false;
   if (!(h <= 0.004 * wide * 4.0 * P.rs * (P.rc - P.rs))) return false;
   Tb.words = taylor ? kTabWordsTaylor : kind == kTabValueFF ? kTabWordsFF : kTabWords64;

@@ -25,7 +25,7 @@
 //
 // w is a 64-bit integer in units of 2^-56 (w < 128): node distances are integer
 // additions, the interval is a shift, and tau is the remaining bits.  Pairs
-// with a node below the first row (r < r_cut / 4), with |d|^2 >= 64 or with a
+// with a node below the first row (r < r_cut / 4 or 1.25 A), with |d|^2 >= 64 or with a
 // non-finite coordinate take the direct evaluation.
 #pragma once
 
@@ -45,7 +45,7 @@ constexpr int kTabWords64 = 3, kTabWordsFF = 2, kTabWordsTaylor = 5;
 constexpr int kTabFixedBits = 56;   // w in units of 2^-56
 constexpr int kTabExpBias = 128 + 61;    // of the derivative rows' exponents
 constexpr int kTabValueBias = 128 + 62;  // of the value rows' exponents
-constexpr double kTabRLow = 0.25;   // first row at (r_cut / 4)^2
+constexpr double kTabRLow = 0.25, kTabRMin = 1.25;  // first row at r_cut / 4, not below 1.25 A
 // Float-float rows hold c2 to 32 and c3, c5 to 24 and 8 bits.  Where the switch
 // u = (r_cut - r) / (r_cut - r_switch) falls to the offset's share du of it, the
 // terms are (du / u)^n of the value and those bits show (at u = 0.1, 4.95 A of 5:
