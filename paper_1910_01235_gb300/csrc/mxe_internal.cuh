@@ -99,16 +99,19 @@ struct Tables<2> : Tables<1> {};
 // The radial terms as piecewise polynomials in r^2 (radial_table.cuh): rows of
 // `stride` 16-byte words, one row per interval of width h (and per side of a
 // breakpoint), `words` words per term, density terms first.
-constexpr int64_t kTabMaxBytes = 200 * 1024;  // staged in one block's shared memory
+constexpr int64_t kTabMaxBytes = 224 * 1024;  // staged in one block's shared memory
 enum { kTabValue64 = 0, kTabDeriv64 = 1, kTabValueFF = 2, kTabTaylor64 = 3 };
 struct RadialTab {
   const uint4* rows;
   int nrow, stride, words;
   int nf_slots, np_slots;  // terms of a row: density, then pair terms (absent ones are zero)
   int shift, k_lo;         // interval of w: (high word of w >> shift) - k_lo
-  int n_main;              // rows of width h; the rest to the cutoff a quarter as wide (float-float rows)
-  unsigned rs_hi, rc_hi;   // r_switch^2, r_cut^2 as high words
-  unsigned near_hi;        // where the narrow rows begin
+  // float-float rows: n_low rows below the interval k_lo, narrow rows from n_main
+  // on, to the cutoff (elsewhere n_low 0 and no narrow rows)
+  int n_low, n_main;
+  int first, first_near;      // row of interval 0 of either width
+  unsigned rs_hi, rc_hi;      // r_switch^2, r_cut^2 as high words
+  unsigned main_hi, near_hi;  // where the rows of width h and the narrow rows begin
   double h;
 };
 

@@ -29,6 +29,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "pair_common.cuh"
 #include "radial_table.cuh"
@@ -191,10 +192,10 @@ __device__ __forceinline__ ff row_rest(uint4 a, const uint4* t, float th, float 
   else return tab_poly64(__uint_as_float(a.z), __uint_as_float(a.w), t[1], t[2], th, tl);
 }
 // the terms at one point, each on its own row's grid
-template <int N, int W, bool FFQ>
+template <int N, int W, bool FFQ, bool LOWS>
 __device__ __forceinline__ void one_node(const RadialTab& Tb, const uint4* sm, long long w, int& low, NodeSum* s) {
   float th, tl;
-  const uint4* row = tab_row<FFQ>(Tb, sm, w, th, tl, low);
+  const uint4* row = tab_row<FFQ, LOWS>(Tb, sm, w, th, tl, low);
 #pragma unroll
   for (int u = 0; u < N; ++u) {
     const uint4 a = row[u * W];
@@ -202,18 +203,18 @@ __device__ __forceinline__ void one_node(const RadialTab& Tb, const uint4* sm, l
   }
 }
 // empty sums on the grid of the pair's nearest node, where the terms are largest
-template <int N, int W, bool FFQ>
+template <int N, int W, bool FFQ, bool LOWS>
 __device__ __forceinline__ void start_sums(const RadialTab& Tb, const uint4* sm, const PairNodes& D, int& low,
                                            NodeSum* s) {
   float th, tl;
-  const uint4* row = tab_row<FFQ>(Tb, sm, nearest_node(D), th, tl, low);
+  const uint4* row = tab_row<FFQ, LOWS>(Tb, sm, nearest_node(D), th, tl, low);
 #pragma unroll
   for (int u = 0; u < N; ++u) s[u] = NodeSum{0, ff{0.f, 0.f}, (int)(row[u * W].x & 0xffu) + kSumHead};
 }
-template <int N, int W, bool FFQ>
+template <int N, int W, bool FFQ, bool LOWS>
 __device__ __forceinline__ void add_node(const RadialTab& Tb, const uint4* sm, long long w, int& low, NodeSum* s) {
   float th, tl;
-  const uint4* row = tab_row<FFQ>(Tb, sm, w, th, tl, low);
+  const uint4* row = tab_row<FFQ, LOWS>(Tb, sm, w, th, tl, low);
 #pragma unroll
   for (int u = 0; u < N; ++u) {
     const uint4 a = row[u * W];
@@ -251,34 +252,45 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_geo_tab(
     PairNodes N;
     const int big = pair_nodes(G, N);
     int low = 0;
-    NodeSum s[NT];
-    one_node<NF, W, O::kFF>(Tb, sm, N.w0, low, s);
     R val[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) val[c] = (R)0;
+    auto evaluate = [&](auto lows) {
+      constexpr bool kLows = decltype(lows)::value;
+      NodeSum s[NT];
+      one_node<NF, W, O::kFF, kLows>(Tb, sm, N.w0, low, s);
 #pragma unroll
-    for (int v = 0; v < NF; ++v) val[v] = sum_value(s[v], (R*)nullptr);
-    start_sums<NT, W, O::kFF>(Tb, sm, N, low, s);
+      for (int v = 0; v < NF; ++v) val[v] = sum_value(s[v], (R*)nullptr);
+      start_sums<NT, W, O::kFF, kLows>(Tb, sm, N, low, s);
 #pragma unroll 1
-    for (int site = 0; site < 2; ++site) {
+      for (int site = 0; site < 2; ++site) {
 #pragma unroll 1
-      for (int a = 0; a < 3; ++a) {
-        add_node<NT, W, O::kFF>(Tb, sm, N.base[0] + N.tw[0][0], low, s);
-        add_node<NT, W, O::kFF>(Tb, sm, N.base[0] - N.tw[0][0], low, s);
-        // the next axis (registers rotate: one copy of the node code)
-        const long long t = N.tw[0][0];
-        N.tw[0][0] = N.tw[0][1];
-        N.tw[0][1] = N.tw[0][2];
-        N.tw[0][2] = t;
+        for (int a = 0; a < 3; ++a) {
+          add_node<NT, W, O::kFF, kLows>(Tb, sm, N.base[0] + N.tw[0][0], low, s);
+          add_node<NT, W, O::kFF, kLows>(Tb, sm, N.base[0] - N.tw[0][0], low, s);
+          // the next axis (registers rotate: one copy of the node code)
+          const long long t = N.tw[0][0];
+          N.tw[0][0] = N.tw[0][1];
+          N.tw[0][1] = N.tw[0][2];
+          N.tw[0][2] = t;
+        }
+        N.base[0] = N.base[1];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) N.tw[0][a] = N.tw[1][a];
       }
-      N.base[0] = N.base[1];
 #pragma unroll
-      for (int a = 0; a < 3; ++a) N.tw[0][a] = N.tw[1][a];
+      for (int v = 0; v < NF; ++v) val[NF + v] = sum_value(s[v], (R*)nullptr);
+#pragma unroll
+      for (int u = 0; u < NP; ++u) val[2 * NF + u] = sum_value(s[NF + u], (R*)nullptr);
+    };
+    // one branch per warp, not one per node: few warps have a pair this close
+    bool below = false;
+    if constexpr (O::kFF) {
+      const long long w = min(nearest_node(N), N.w0);
+      below = __any_sync(__activemask(), (unsigned)((unsigned long long)w >> 32) < Tb.main_hi);
     }
-#pragma unroll
-    for (int v = 0; v < NF; ++v) val[NF + v] = sum_value(s[v], (R*)nullptr);
-#pragma unroll
-    for (int u = 0; u < NP; ++u) val[2 * NF + u] = sum_value(s[NF + u], (R*)nullptr);
+    if (below) evaluate(std::bool_constant<O::kFF>{});
+    else evaluate(std::false_type{});
     if (big || low < 0) {
       double st[2], av[2], ph[3];
       const PairGeom H = G;
@@ -348,16 +360,16 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_rdensity_tab(
     int low = 0;
     NodeSum s[NF];
     double fst[NF], fav[NF];
-    one_node<NF, W, false>(Tb, sm, N.w0, low, s);
+    one_node<NF, W, false, false>(Tb, sm, N.w0, low, s);
 #pragma unroll
     for (int v = 0; v < NF; ++v) fst[v] = sum_value(s[v], (double*)nullptr);
-    start_sums<NF, W, false>(Tb, sm, N, low, s);
+    start_sums<NF, W, false, false>(Tb, sm, N, low, s);
 #pragma unroll 1
     for (int site = 0; site < 2; ++site) {
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        add_node<NF, W, false>(Tb, sm, N.base[0] + N.tw[0][a], low, s);
-        add_node<NF, W, false>(Tb, sm, N.base[0] - N.tw[0][a], low, s);
+        add_node<NF, W, false, false>(Tb, sm, N.base[0] + N.tw[0][a], low, s);
+        add_node<NF, W, false, false>(Tb, sm, N.base[0] - N.tw[0][a], low, s);
       }
       N.base[0] = N.base[1];
 #pragma unroll
@@ -467,7 +479,7 @@ template <int NT>
 __device__ __forceinline__ long long force_node(const RadialTab& Tb, const uint4* sm, long long w,
                                                 const FixedWeights<NT>& F, float sc, int& low) {
   float th, tl;
-  const uint4* row = tab_row<false>(Tb, sm, w, th, tl, low);
+  const uint4* row = tab_row<false, false>(Tb, sm, w, th, tl, low);
   long long h = 0;
   ff p{0.f, 0.f};
 #pragma unroll
@@ -584,13 +596,13 @@ __global__ void __launch_bounds__(kTabThreads, 1) k_rforce_tab(
     float th, tl;
     {
       FixedWeights<NF> F;
-      const int unit = fixed_weights<NF>(cfs, tab_row<false>(Tb, sm, N.w0, th, tl, low), F, big);
+      const int unit = fixed_weights<NF>(cfs, tab_row<false, false>(Tb, sm, N.w0, th, tl, low), F, big);
       const long long h = force_node<NF>(Tb, sm, N.w0, F, exp2f_bits(-24 - unit), low);
       out[6] = fixed_double(h != 0 ? h + (F.terms >> 1) : 0, unit);
     }
     const long long near = nearest_node(N);
     FixedWeights<NT> F;
-    const int unit = fixed_weights<NT>(C, tab_row<false>(Tb, sm, near, th, tl, low), F, big);
+    const int unit = fixed_weights<NT>(C, tab_row<false, false>(Tb, sm, near, th, tl, low), F, big);
     const float sc = exp2f_bits(-24 - unit);
     long long T = 0;
     double U[3] = {0.0, 0.0, 0.0}, V0 = 0.0, ad[3] = {fabs(G.d[0]), fabs(G.d[1]), fabs(G.d[2])};

@@ -177,10 +177,18 @@ __global__ void __launch_bounds__(32) k_radial_table(const __grid_constant__ Dev
     return;
   }
   // rows step by one at r_switch^2: its interval has a row for each side
-  const int ks = (int)(Tb.rs_hi >> Tb.shift) - Tb.k_lo;
-  const bool beyond = row > ks, narrow = row >= Tb.n_main;
-  const double h = narrow ? Tb.h / (1 << kTabNarrow) : Tb.h;
-  const int k = narrow ? row - Tb.n_main + (int)(Tb.near_hi >> (Tb.shift - kTabNarrow)) : row - (beyond ? 1 : 0) + Tb.k_lo;
+  const int mid = row - Tb.n_low, ks = (int)(Tb.rs_hi >> Tb.shift) - Tb.k_lo;
+  const bool beyond = mid > ks;
+  double h = Tb.h;
+  int k = mid - (beyond ? 1 : 0) + Tb.k_lo;
+  if (mid < 0) {
+    const int oct = min(row >> 6, 2);  // [1/4, 1/2), [1/2, 1), from 1 on
+    h = 1.0 / (256 >> oct);
+    k = row - 64 * (oct - 1);
+  } else if (row >= Tb.n_main) {
+    h *= 1.0 / (1 << kTabNarrow);
+    k = row - Tb.n_main + (int)(Tb.near_hi >> (Tb.shift - kTabNarrow));
+  }
   const double wc = ((double)k + 0.5) * h;
   dd V0, V1, V2;
   double V[kDeg + 1];
@@ -281,36 +289,42 @@ bool plan_radial_tab(const DevPot& P, int kind, bool with_pairs, RadialTab& Tb) 
   Tb.stride = tab_stride(Tb.nf_slots + Tb.np_slots, Tb.words);
   Tb.h = h;
   Tb.shift = kTabFixedBits - 32 - bits_h;
-  Tb.k_lo = (int)std::floor(r_lo * r_lo / h);
+  const bool graded = kind == kTabValueFF;
+  Tb.k_lo = (int)std::floor((graded ? std::max(r_lo * r_lo, kTabMainW) : r_lo * r_lo) / h);
+  Tb.main_hi = (unsigned)Tb.k_lo << Tb.shift;
+  Tb.n_low = graded ? 64 + 2 * Tb.k_lo : 0;  // 64, 64 and 64 per unit of w from 1 on
   const double unit = std::ldexp(1.0, kTabFixedBits - 32);
   Tb.rs_hi = (unsigned)std::floor(P.rs * P.rs * unit);
   Tb.rc_hi = (unsigned)std::ceil(rc2 * unit);
   if ((int)(Tb.rs_hi >> Tb.shift) < Tb.k_lo) return false;
-  Tb.n_main = (int)((Tb.rc_hi - 1) >> Tb.shift) - Tb.k_lo + 2;  // both sides of r_switch
-  Tb.nrow = Tb.n_main + 1;                                        // and the zeros
+  Tb.n_main = Tb.n_low + (int)((Tb.rc_hi - 1) >> Tb.shift) - Tb.k_lo + 2;  // both sides of r_switch
+  Tb.nrow = Tb.n_main + 1;                                                   // and the zeros
   Tb.near_hi = 0xffffffffu;
-  if (kind == kTabValueFF) {
+  if (graded) {
     const double rn = P.rc - kTabNearU * (P.rc - P.rs);
     const unsigned kn = std::max((unsigned)std::floor(rn * rn / h), (Tb.rs_hi >> Tb.shift) + 1u);
     if (kn <= (Tb.rc_hi - 1) >> Tb.shift) {
       Tb.near_hi = kn << Tb.shift;
-      Tb.n_main = (int)kn - Tb.k_lo + 1;
+      Tb.n_main = Tb.n_low + (int)kn - Tb.k_lo + 1;
       const int sh = Tb.shift - kTabNarrow;
       Tb.nrow = Tb.n_main + (int)((Tb.rc_hi - 1) >> sh) - (int)(Tb.near_hi >> sh) + 2;
     }
   }
+  Tb.first = Tb.n_low - Tb.k_lo;
+  Tb.first_near = Tb.n_main - 1 - (int)(Tb.near_hi >> (Tb.shift - kTabNarrow));  // one less: beyond r_switch
   if ((int64_t)Tb.nrow * Tb.stride * 16 > kTabMaxBytes) return false;
   for (int u = 0; u < Tb.nf_slots + Tb.np_slots; ++u) {
     const int f = u, p = u - Tb.nf_slots;
     const RadialFn* F = u < Tb.nf_slots ? (f < P.n_f ? &P.f[f] : nullptr) : (p < P.n_phi ? &P.phi[p] : nullptr);
     // largest value: at the first row's lower end (the terms decrease)
-    const double wl = Tb.k_lo * h;
+    const double wl = graded ? 0.25 : Tb.k_lo * h;
     const double vmax = F ? F->A * std::exp(F->kappa - F->lambda * std::sqrt(wl)) : 1.0;
     if (!std::isfinite(vmax) || vmax > 1e30) return false;
     if (F && vmax < 1e-30) return false;
     // the other rows have 8 bits of exponent, 2^-127 .. 2^127; from the first row
-    // to the last a term falls by less than 2^55 within the limits above
-    if (!taylor && F && vmax < 1e-20) return false;
+    // to the last a term falls by less than 2^55 (float-float 2^70) within the
+    // limits above
+    if (!taylor && F && vmax < (graded ? 1e-15 : 1e-20)) return false;
     if (kind == kTabDeriv64 && F && vmax > 1e20) return false;
   }
   return true;

@@ -25,8 +25,8 @@
 //
 // w is a 64-bit integer in units of 2^-56 (w < 128): node distances are integer
 // additions, the interval is a shift, and tau is the remaining bits.  Pairs
-// with a node below the first row (r < r_cut / 4 or 1.25 A), with |d|^2 >= 64 or with a
-// non-finite coordinate take the direct evaluation.
+// with a node below the first row (float-float: 0.5 A; else r_cut / 4 or 1.25 A),
+// with |d|^2 >= 64 or with a non-finite coordinate take the direct evaluation.
 #pragma once
 
 #include "mxe_internal.cuh"
@@ -53,6 +53,14 @@ constexpr double kTabRLow = 0.25, kTabRMin = 1.25;  // first row at r_cut / 4, n
 // u = 0.3 on: du^2 / 16.
 constexpr int kTabNarrow = 2;
 constexpr double kTabNearU = 0.3;
+// Below w = 2 (or (r_cut / 4)^2) float-float rows are 1/64 wide, from w = 1 down
+// 64 to an octave, to w = 1/4: down to the smallest admissible node distance.
+// For speed: a pair with a node below the first row took the direct evaluation in
+// FP64, and its warp with it (host-solute slab of 16,384 sites, solute widths of
+// 0.25 A: free-energy call 1495 us, 484 with the direct kernels, 285 now).  For
+// precision: the terms dropped after degree 5 fall as w^-6 and left 8e-14 of the
+// value at 1.25 A (decay rate 2.5 / A), the direct kernels 2e-14.
+constexpr double kTabMainW = 2.0;
 
 // 16-byte words between the rows of consecutive intervals: all terms of an
 // interval lie side by side; an odd count spreads random intervals over the
@@ -81,21 +89,29 @@ __device__ __forceinline__ long long tab_fixed(double x, int& big) {
 // Row of w and the offset from the row's centre; `low` collects w below the
 // first row, and below zero (a node that falls on a site to rounding).  The
 // index is clamped, so every access stays inside the table whatever w is.
-// NARROW: the table has narrow rows before the cutoff.
-template <bool NARROW>
+// GRADED: the row width changes with w (float-float tables); LOWS: w may lie below
+// the rows of the common width (a few instructions that every node would pay).
+template <bool GRADED, bool LOWS>
 __device__ __forceinline__ const uint4* tab_row(const RadialTab& Tb, const uint4* sm, long long w, float& th, float& tl,
                                                 int& low) {
   const unsigned hi = (unsigned)((unsigned long long)w >> 32), lo = (unsigned)w;
-  int sh = Tb.shift, first = -Tb.k_lo;
-  if (NARROW && hi >= Tb.near_hi) {
-    sh -= kTabNarrow;
-    first = Tb.n_main - 1 - (int)(Tb.near_hi >> sh);
+  int sh = Tb.shift, first = Tb.first;
+  if constexpr (GRADED) {
+    if (hi >= Tb.near_hi) {
+      sh -= kTabNarrow;
+      first = Tb.first_near;
+    }
+    if (LOWS && hi < Tb.main_hi) {
+      const int o = min(max(31 - __clz((int)hi), 21), 24);  // 22: w in [1/4, 1/2)
+      sh = o - 6;
+      first = 64 * (o - 23);
+    }
   }
   int k = (int)(hi >> sh) + first;
   low |= k | (int)hi;  // negative below the first row; the high bit of a negative w
   k += hi >= Tb.rs_hi ? 1 : 0;
   if (hi >= Tb.rc_hi) k = Tb.nrow - 1;
-  k = min(max(k, 0), Tb.nrow - 1);
+  k = (int)min((unsigned)k, (unsigned)(Tb.nrow - 1));
   const unsigned f1 = __funnelshift_r(lo, hi, sh + 9) & 0x7fffffu;
   const unsigned f2 = (lo >> (sh - 14)) & 0x7fffffu;
   th = __uint_as_float(0x3f800000u | f1) - 1.5f;

@@ -76,3 +76,20 @@ def test_near_a_quarter_of_the_cutoff(k, lam, rs, rc, density, precision):
     d = np.ceil(rc * 256.0) / 1024.0 + (k + 8) / 1024.0
     off, slope = error(d, lam, rs, rc, density, precision)
     assert off <= bound(precision, d, slope)
+
+
+@pytest.mark.parametrize("precision", ["mixed", "ff"])
+@pytest.mark.parametrize("density", [True, False])
+@pytest.mark.parametrize("lam,rs,rc", [(1.96, 4.5, 5.0), (2.5, 4.5, 5.0), (3.0, 5.2, 6.0)])
+@pytest.mark.parametrize("d", [0.50390625, 0.5078125, 0.6005859375, 0.70703125, 0.7080078125, 0.8125, 0.9990234375, 1.0009765625,
+                               1.119140625, 1.248046875, 1.2734375, 1.4140625, 1.4150390625, 1.498046875])
+def test_float_float_below_the_main_rows(d, lam, rs, rc, density, precision):
+    """Every octave of the graded rows and the distances at which their width changes;
+    with a node below 0.5 A, the smallest admissible distance, an error."""
+    if d - 2.4495 * SIGMA < 0.5:
+        with pytest.raises(M.MxeError) as e:
+            error(d, lam, rs, rc, density, precision)
+        assert e.value.status == M.ERR_GEOMETRY
+        return
+    off, _ = error(d, lam, rs, rc, density, precision)
+    assert off <= 2.0**-44
