@@ -457,25 +457,30 @@ void fill_pass(mxe_ctx* c, const mxe_state* s, PassArgs& A) {
   A.pair_tpb = c->pair_tpb;
 }
 
+// Here and in build_lists a capacity is zero from the release of its arrays
+// until all of them are allocated again: after a failed allocation the next
+// build, whatever its size, comes here again and finds no missing array.
 mxe_status ensure_cells(mxe_ctx* c, int64_t ncell) {
   if (ncell <= c->ncell_cap) return MXE_OK;
   dfree(c->cell_count);
   dfree(c->cell_start);
+  c->ncell_cap = 0;
   int64_t cap = ncell + ncell / 4 + 16;
   CK(dalloc(&c->cell_count, cap));
   CK(dalloc(&c->cell_start, cap + 1));
-  c->ncell_cap = cap;
   if (c->nsys) {
     dfree(c->cell_sys);
     CK(dalloc(&c->cell_sys, cap));
     c->B.cell_sys = c->cell_sys;
   }
-  int64_t need = std::max<int64_t>(c->n, cap) + 1;
-  if (c->scan_len < scan_tmp_len(need)) {
+  const int64_t len = scan_tmp_len(std::max<int64_t>(c->n, cap) + 1);
+  if (c->scan_len < len) {
     dfree(c->scan_tmp);
-    c->scan_len = scan_tmp_len(need);
-    CK(dalloc(&c->scan_tmp, c->scan_len));
+    c->scan_len = 0;
+    CK(dalloc(&c->scan_tmp, len));
+    c->scan_len = len;
   }
+  c->ncell_cap = cap;
   return MXE_OK;
 }
 
@@ -620,6 +625,7 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
     if ((int64_t)n * stride > c->rows_cap) {
       dfree(c->rows_tmp);
       dfree(c->brows_tmp);
+      c->rows_cap = 0;
       CK(dalloc(&c->rows_tmp, (int64_t)n * stride));
       CK(dalloc(&c->brows_tmp, (int64_t)n * stride));
       c->rows_cap = (int64_t)n * stride;
@@ -675,6 +681,7 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
   if (npairs > 2147483647LL || nbonds > 2147483647LL) return MXE_ERR_NBR_OVERFLOW;
   if (npairs > c->nb_cap) {
     dfree(c->nb_ent);
+    c->nb_cap = 0;
     int64_t cap = npairs + npairs / 8 + 64;
     CK(dalloc(&c->nb_ent, cap));
     c->nb_cap = cap;
@@ -683,6 +690,7 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
   if (pairs && (npairs > c->pair_cap || !c->pair_rec)) {
     dfree(c->pair_rec);
     dfree(c->pair_buf);
+    c->pair_cap = 0;
     const int64_t cap = std::max<int64_t>(c->nb_cap, npairs);
     CK(dalloc(&c->pair_rec, cap / 2 + 64));
     // one record per entry, wide enough for the force records a free-energy call puts there
@@ -698,6 +706,7 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
   }
   if (nbonds > c->bd_cap) {
     dfree(c->bd_idx);
+    c->bd_cap = 0;
     int64_t cap = nbonds + nbonds / 8 + 64;
     CK(dalloc(&c->bd_idx, cap));
     c->bd_cap = cap;

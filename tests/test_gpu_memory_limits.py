@@ -1,0 +1,56 @@
+"""List builds when the device's memory runs out (csrc/api.cu): the status, and
+the context afterwards.  Another allocation takes all but a given rest of the
+free memory meanwhile.
+"""
+import numpy as np
+import pytest
+
+from paper_1910_01235_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_1910_01235_gb300 import mxe as M  # noqa: E402
+
+
+class AllBut:
+    def __init__(self, rest):
+        self.rest = rest
+
+    def __enter__(self):
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        free = torch.cuda.mem_get_info()[0]
+        self.held = torch.empty(max(free - self.rest, 0), dtype=torch.uint8, device="cuda")
+
+    def __exit__(self, *exc):
+        self.held = None
+        torch.cuda.empty_cache()
+
+
+def evaluate(g):
+    g.build_neighbors()
+    g.free_energy_grad()
+    return [t.clone() for t in (g.F4, g.gq, g.gs, g.mu_ex)]
+
+
+@pytest.mark.parametrize("rest_mb", [20, 100, 250, 600])
+@pytest.mark.parametrize("precision", ["fp64", "ff"])
+def test_a_list_that_does_not_fit(precision, rest_mb):
+    """A wider list fails in one allocation or another of its growth; the narrow
+    one is then built again, with the same results."""
+    s = W.perturb(W.config_vacancy_lattice(30), 0.05, 0.02, seed=5)
+    g = M.MxeSystem(s, precision)
+    narrow = g.skin
+    before = evaluate(g)
+    with AllBut(rest_mb << 20):
+        g.skin = narrow + 3.0
+        with pytest.raises(M.MxeError) as e:
+            g.build_neighbors()
+        assert e.value.status == M.ERR_OOM
+        g.skin = narrow
+    for a, b in zip(evaluate(g), before):
+        assert np.abs((a - b).cpu().numpy()).max() <= 1e-12 * np.abs(b.cpu().numpy()).max()
