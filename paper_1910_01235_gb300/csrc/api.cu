@@ -618,6 +618,7 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
                            {c->totals + 1, c->totals + 2, c->totals + 3}};
   bool direct = false;
   int stride = 0;
+  bool rows_fit = true;  // else count + fill, which needs no rows at a stride
   if (staged && try_direct) {
     // a growing r_list takes in whole shells of a lattice (24 of 54 neighbours
     // at once in FCC): half a row more, at least 32
@@ -626,10 +627,17 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
       dfree(c->rows_tmp);
       dfree(c->brows_tmp);
       c->rows_cap = 0;
-      CK(dalloc(&c->rows_tmp, (int64_t)n * stride));
-      CK(dalloc(&c->brows_tmp, (int64_t)n * stride));
-      c->rows_cap = (int64_t)n * stride;
+      rows_fit = dalloc(&c->rows_tmp, (int64_t)n * stride) == cudaSuccess &&
+                 dalloc(&c->brows_tmp, (int64_t)n * stride) == cudaSuccess;
+      if (rows_fit) {
+        c->rows_cap = (int64_t)n * stride;
+      } else {
+        cudaGetLastError();
+        dfree(c->rows_tmp);
+      }
     }
+  }
+  if (staged && try_direct && rows_fit) {
     const bool pi = has_pair_index(c);
     // a stencil above cand_cap is cut and reported in max_row[2] (not in the
     // context's flags): the check below then discards this fill
@@ -651,7 +659,7 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
     }
     c->cand_cap_prev = cand_true;  // the next guess starts from the true size, not from this guess
     if (!direct) CK(cudaMemsetAsync(c->max_row, 0, sizeof(int), st));
-  } else if (try_direct) {  // the guessed size did not fit shared memory: take the true one
+  } else if (try_direct) {  // the guessed size did not fit shared memory, or the rows the device: take the true one
     CK(cudaMemcpyAsync(c->ints_h + 2, c->max_row + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     cand_cap = std::max(c->ints_h[2], 1);

@@ -54,3 +54,17 @@ def test_a_list_that_does_not_fit(precision, rest_mb):
         g.skin = narrow
     for a, b in zip(evaluate(g), before):
         assert np.abs((a - b).cpu().numpy()).max() <= 1e-12 * np.abs(b.cpu().numpy()).max()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "ff"])
+def test_a_rebuild_without_room_for_its_rows(precision):
+    """The second build of a context fills rows of a fixed stride (29 MB or more
+    here); without room for them it counts and fills, as the first."""
+    s = W.perturb(W.config_vacancy_lattice(30), 0.05, 0.02, seed=6)
+    g = M.MxeSystem(s, precision)
+    before = evaluate(g)
+    with AllBut(16 << 20):
+        g.build_neighbors()
+    g.free_energy_grad()
+    for a, b in zip((g.F4, g.gq, g.gs, g.mu_ex), before):
+        assert np.abs((a - b).cpu().numpy()).max() <= 1e-12 * np.abs(b.cpu().numpy()).max()
