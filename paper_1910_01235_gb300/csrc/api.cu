@@ -93,7 +93,7 @@ struct mxe_ctx {
   double* pair_buf = nullptr;  // pair_cap x pair_record_len 8-byte values (float pairs or doubles; see geo_layout)
   void *ent_dens = nullptr, *ent_frc = nullptr;  // [entries] relaxation records (relax_record_bytes each)
   bool relax_records = false;  // allocate them (first relaxation of the context, then with every list growth)
-  int64_t pair_cap = 0, n_upairs = 0;
+  int64_t pair_cap = 0, n_upairs = 0, pair_bytes = 0;  // pair_bytes: of pair_buf, per entry
   // rows of a fill without a count pass, at a fixed stride
   uint32_t* rows_tmp = nullptr;
   int* brows_tmp = nullptr;
@@ -158,8 +158,8 @@ struct mxe_ctx {
   // pair form of the passes (tangent_table.cu): rows, records of every entry
   uint4* tan_rows = nullptr;
   RadialTab tan_dens{}, tan_tab{};
-  double* tan_rec = nullptr;
-  int64_t tan_rec_cap = 0;     // entries
+  double* tan_rec = nullptr;   // what of the records pair_buf does not hold
+  int64_t tan_rec_len = 0;     // doubles
   double* tan_part = nullptr;  // partial sums of the term sensitivities
   int64_t tan_part_len = 0;
   double* dot_part = nullptr;  // partial sums of dot products
@@ -699,11 +699,13 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
     dfree(c->pair_rec);
     dfree(c->pair_buf);
     c->pair_cap = 0;
+    dfree(c->tan_rec);  // of the shorter list; allocated again where it is wanted
+    c->tan_rec_len = 0;
     const int64_t cap = std::max<int64_t>(c->nb_cap, npairs);
     CK(dalloc(&c->pair_rec, cap / 2 + 64));
     // one record per entry, wide enough for the force records a free-energy call puts there
-    const int64_t rec = std::max<int64_t>(pair_record_len(c->dp) * (int64_t)sizeof(double), relax_record_bytes(c->precision));
-    CK(dalloc_bytes((void**)&c->pair_buf, cap * rec));
+    c->pair_bytes = std::max<int64_t>(pair_record_len(c->dp) * (int64_t)sizeof(double), relax_record_bytes(c->precision));
+    CK(dalloc_bytes((void**)&c->pair_buf, cap * c->pair_bytes));
     dfree(c->ent_dens);
     dfree(c->ent_frc);
     if (c->relax_records) {
@@ -1272,19 +1274,23 @@ bool ensure_taylor_rows(mxe_ctx* c) {
 }
 
 // The tangent passes run over unordered pairs when the potential has Taylor
-// rows and the records of every entry (12 doubles for two species) fit the
-// device; else over the full list (one thread per site).
-bool ensure_tangent_pairs(mxe_ctx* c) {
+// rows and the records of every entry (12 doubles for two species, 8 of them in
+// pair_buf) fit the device; else over the full list (one thread per site).
+bool ensure_tangent_pairs(mxe_ctx* c, int record_len, TanRec& R) {
   if (!has_pair_index(c) || !c->pair_rec || !ensure_taylor_rows(c)) return false;
-  if (c->tan_rec_cap < c->pair_cap) {
+  R.a = c->pair_buf;
+  R.ca = 2 * (int)(c->pair_bytes / 16);
+  const int64_t rest = c->pair_cap * std::max(0, record_len - R.ca);
+  if (c->tan_rec_len < rest) {
     dfree(c->tan_rec);
-    c->tan_rec_cap = 0;
-    if (dalloc(&c->tan_rec, c->pair_cap * tangent_record_len(c->dp)) != cudaSuccess) {
+    c->tan_rec_len = 0;
+    if (dalloc(&c->tan_rec, rest) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
-    c->tan_rec_cap = c->pair_cap;
+    c->tan_rec_len = rest;
   }
+  R.b = c->tan_rec;
   const int64_t part = 4LL * (c->tan_tab.nf_slots + c->tan_tab.np_slots) * tangent_blocks(c->n_upairs);
   if (c->tan_part_len < part) {
     dfree(c->tan_part);
@@ -1348,9 +1354,10 @@ mxe_status enqueue_tangent(mxe_ctx* c, const mxe_state* s, const double* dq, con
   A.flags = c->flags;
   A.batch = c->B;
   A.n_ent = c->n_pairs;
-  if (ensure_tangent_pairs(c)) {
+  TanRec rec;
+  if (ensure_tangent_pairs(c, tangent_record_len(c->dp, A, T > 0 && th_out), rec)) {
     CK(TIMED("tangent_pairs", launch_tangent_pairs(c->dp, c->grid, A, c->tan_dens, c->tan_tab, c->pair_rec,
-                                                   c->n_upairs, c->tan_rec, c->tan_part, T > 0 ? th_out : nullptr,
+                                                   c->n_upairs, rec, c->tan_part, T > 0 ? th_out : nullptr,
                                                    c->stream)));
     return MXE_OK;
   }

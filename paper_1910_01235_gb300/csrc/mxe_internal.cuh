@@ -438,12 +438,17 @@ struct TanArgs {
 };
 // tangent_table.cu: the same passes over unordered pairs with tabulated terms.
 // dens_tab holds the density terms, tab every term (kind kTabTaylor64); rec:
-// [entries] records of tangent_record_len doubles; th_part: tangent_blocks x
+// records of tangent_record_len doubles per entry; th_part: tangent_blocks x
 // 4 T partial sums, th_out [4 T] (null: no term sensitivities)
-int tangent_record_len(const DevPot& P);
+struct TanRec {
+  double* a;  // the first ca doubles of every record [entries][ca]
+  double* b;  // the others
+  int ca;     // even
+};
+int tangent_record_len(const DevPot& P, const TanArgs& A, bool theta);
 int tangent_blocks(int64_t npair);
 cudaError_t launch_tangent_pairs(const DevPot& P, const DevGrid& g, const TanArgs& A, const RadialTab& dens_tab,
-                                 const RadialTab& tab, const int4* pair_rec, int64_t npair, double* rec,
+                                 const RadialTab& tab, const int4* pair_rec, int64_t npair, const TanRec& rec,
                                  double* th_part, double* th_out, cudaStream_t s);
 cudaError_t launch_tangent(const DevPot& P, const DevGrid& g, const TanArgs& A, cudaStream_t s);
 cudaError_t launch_col_sum(const double* col, int ncol, int64_t n, double* out, cudaStream_t s);

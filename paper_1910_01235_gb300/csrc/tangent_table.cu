@@ -41,13 +41,22 @@ __device__ __forceinline__ void pair_rate(const TanArgs& A, int64_t i, int64_t j
 }
 __device__ __forceinline__ double rate_of(const double* __restrict__ t, int64_t k) { return t ? __ldg(&t[k]) : 0.0; }
 
+// Two doubles of a record of C (TanRec: the geometry records' buffer, idle during
+// these passes, holds as many of a record's doubles as fit; with a buffer of its
+// own the 12 doubles of two species took 46 GB for the lists of 4 million sites)
+template <int C>
+__device__ __forceinline__ double2* rec_at(const TanRec& R, int64_t t, int c) {
+  const int ca = min(R.ca, C);
+  return reinterpret_cast<double2*>(2 * c < ca ? R.a + t * ca + 2 * c : R.b + t * (C - ca) + (2 * c - ca));
+}
+
 // ---------------------------------------------------------------- densities
 // Record of an entry: rho_bar, 12 <rho> of its site from the other one, per
 // species, then their tangents: 4 S doubles.
 template <int S>
 __global__ void __launch_bounds__(kTanThreads) k_tan_pair_density(
     const __grid_constant__ DevPot P, const __grid_constant__ DevGrid g0, const __grid_constant__ TanArgs A,
-    const __grid_constant__ TaylorTab Tb, const int4* __restrict__ pair_rec, int64_t npair, double* __restrict__ rec) {
+    const __grid_constant__ TaylorTab Tb, const int4* __restrict__ pair_rec, int64_t npair, const TanRec rec) {
   constexpr int NF = S;
   extern __shared__ uint4 sm[];
   tab_stage(Tb.t, sm);
@@ -121,12 +130,10 @@ __global__ void __launch_bounds__(kTanThreads) k_tan_pair_density(
           }
       }
     }
-    double2* o = reinterpret_cast<double2*>(rec + (int64_t)pr.tp * (4 * S));
-    double2* o2 = reinterpret_cast<double2*>(rec + (int64_t)pr.tr * (4 * S));
 #pragma unroll
     for (int c = 0; c < 2 * S; ++c) {
-      o[c] = make_double2(ri[2 * c], ri[2 * c + 1]);
-      o2[c] = make_double2(rj[2 * c], rj[2 * c + 1]);
+      *rec_at<4 * S>(rec, pr.tp, c) = make_double2(ri[2 * c], ri[2 * c + 1]);
+      *rec_at<4 * S>(rec, pr.tr, c) = make_double2(rj[2 * c], rj[2 * c + 1]);
     }
     if (bad) atomicOr(A.flags, kFlagGeometry);
   }
@@ -136,14 +143,13 @@ constexpr int kTanLanes = 8;  // lanes per site of the gathers
 
 // sum of C doubles per entry over a site's row, complete on every lane of the team
 template <int C>
-__device__ __forceinline__ void team_sum(const double* __restrict__ rec, int beg, int end, int lane, double* s) {
+__device__ __forceinline__ void team_sum(const TanRec& rec, int beg, int end, int lane, double* s) {
 #pragma unroll
   for (int c = 0; c < C; ++c) s[c] = 0.0;
   for (int t = beg + lane; t < end; t += kTanLanes) {
-    const double2* r = reinterpret_cast<const double2*>(rec + (int64_t)t * C);
 #pragma unroll
     for (int c = 0; c < C / 2; ++c) {
-      const double2 v = __ldg(&r[c]);
+      const double2 v = __ldg(rec_at<C>(rec, t, c));
       s[2 * c] += v.x;
       s[2 * c + 1] += v.y;
     }
@@ -157,8 +163,7 @@ __device__ __forceinline__ void team_sum(const double* __restrict__ rec, int beg
 // a = x F'' (<rho> - rho_bar), b = x F' with F = -E sqrt(rho) (one lane per species)
 template <int S>
 __global__ void __launch_bounds__(256) k_tan_density_gather(const __grid_constant__ DevPot P,
-                                                            const __grid_constant__ TanArgs A,
-                                                            const double* __restrict__ rec) {
+                                                            const __grid_constant__ TanArgs A, const TanRec rec) {
   const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, n = A.n;
   const int64_t i = tid / kTanLanes;
   const int lane = (int)(tid % kTanLanes);
@@ -206,7 +211,7 @@ constexpr int grad_len() {
 template <int S, int NP, bool FULL>
 __global__ void __launch_bounds__(kTanThreads) k_tan_pair_grad(
     const __grid_constant__ DevPot P, const __grid_constant__ DevGrid g0, const __grid_constant__ TanArgs A,
-    const __grid_constant__ TaylorTab Tb, const int4* __restrict__ pair_rec, int64_t npair, double* __restrict__ rec,
+    const __grid_constant__ TaylorTab Tb, const int4* __restrict__ pair_rec, int64_t npair, const TanRec rec,
     double* __restrict__ th_part) {
   constexpr int NF = S, NT = NF + NP, RL = grad_len<S, FULL>();
   extern __shared__ uint4 sm[];
@@ -379,12 +384,10 @@ __global__ void __launch_bounds__(kTanThreads) k_tan_pair_grad(
     gsj = ks * W[1];
     gsjt = ks * Wd[1];
     if constexpr (!FULL) {
-      double2* o = reinterpret_cast<double2*>(rec + (int64_t)pr.tp * RL);
-      double2* o2 = reinterpret_cast<double2*>(rec + (int64_t)pr.tr * RL);
-      o[0] = make_double2(-gt[0], -gt[1]);
-      o[1] = make_double2(-gt[2], gt[3]);
-      o2[0] = make_double2(gt[0], gt[1]);
-      o2[1] = make_double2(gt[2], gsjt);
+      *rec_at<RL>(rec, pr.tp, 0) = make_double2(-gt[0], -gt[1]);
+      *rec_at<RL>(rec, pr.tp, 1) = make_double2(-gt[2], gt[3]);
+      *rec_at<RL>(rec, pr.tr, 0) = make_double2(gt[0], gt[1]);
+      *rec_at<RL>(rec, pr.tr, 1) = make_double2(gt[2], gsjt);
     } else {
       double ri[RL], rj[RL];
 #pragma unroll
@@ -433,12 +436,10 @@ __global__ void __launch_bounds__(kTanThreads) k_tan_pair_grad(
         ri[2 * (4 + S) - S + k] = mit;
         rj[2 * (4 + S) - S + k] = mjt;
       }
-      double2* o = reinterpret_cast<double2*>(rec + (int64_t)pr.tp * RL);
-      double2* o2 = reinterpret_cast<double2*>(rec + (int64_t)pr.tr * RL);
 #pragma unroll
       for (int c = 0; c < RL / 2; ++c) {
-        o[c] = make_double2(ri[2 * c], ri[2 * c + 1]);
-        o2[c] = make_double2(rj[2 * c], rj[2 * c + 1]);
+        *rec_at<RL>(rec, pr.tp, c) = make_double2(ri[2 * c], ri[2 * c + 1]);
+        *rec_at<RL>(rec, pr.tr, c) = make_double2(rj[2 * c], rj[2 * c + 1]);
       }
       if (theta) {
 #pragma unroll
@@ -489,8 +490,7 @@ __global__ void __launch_bounds__(32) k_tan_theta(const __grid_constant__ DevPot
 }
 
 template <int S, bool FULL>
-__global__ void __launch_bounds__(256) k_tan_grad_gather(const __grid_constant__ TanArgs A,
-                                                         const double* __restrict__ rec) {
+__global__ void __launch_bounds__(256) k_tan_grad_gather(const __grid_constant__ TanArgs A, const TanRec rec) {
   constexpr int RL = grad_len<S, FULL>();
   const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, n = A.n;
   const int64_t i = tid / kTanLanes;
@@ -520,6 +520,8 @@ __global__ void __launch_bounds__(256) k_tan_grad_gather(const __grid_constant__
   }
 }
 
+bool wants_values(const TanArgs& A, bool theta) { return theta || A.gq_v || A.gs_v || A.mu_v || A.mu_t; }
+
 template <typename... KArgs, typename... Args>
 cudaError_t launch_staged(void (*kernel)(KArgs...), const RadialTab& Tb, int blocks, cudaStream_t s, Args... args) {
   const size_t shm = (size_t)Tb.nrow * Tb.stride * 16;
@@ -532,16 +534,15 @@ cudaError_t launch_staged(void (*kernel)(KArgs...), const RadialTab& Tb, int blo
 
 template <int S, int NP>
 cudaError_t tangent_pairs(const DevPot& P, const DevGrid& g, const TanArgs& A, const RadialTab& dens_tab,
-                          const RadialTab& tab, const int4* pair_rec, int64_t npair, double* rec, double* th_part,
-                          double* th_out, cudaStream_t s) {
+                          const RadialTab& tab, const int4* pair_rec, int64_t npair, const TanRec& rec,
+                          double* th_part, double* th_out, cudaStream_t s) {
   const int blocks = tangent_blocks(npair);
   const unsigned gblocks = (unsigned)((A.n * kTanLanes + 255) / 256);
   cudaError_t e = launch_staged(k_tan_pair_density<S>, dens_tab, blocks, s, P, g, A, taylor_tab(P, dens_tab), pair_rec,
                                 npair, rec);
   if (e != cudaSuccess) return e;
   k_tan_density_gather<S><<<gblocks, 256, 0, s>>>(P, A, rec);
-  const bool full = th_out || A.gq_v || A.gs_v || A.mu_v || A.mu_t;
-  if (full) {
+  if (wants_values(A, th_out != nullptr)) {
     e = launch_staged(k_tan_pair_grad<S, NP, true>, tab, blocks, s, P, g, A, taylor_tab(P, tab), pair_rec, npair, rec,
                       th_out ? th_part : nullptr);
     if (e != cudaSuccess) return e;
@@ -560,7 +561,9 @@ cudaError_t tangent_pairs(const DevPot& P, const DevGrid& g, const TanArgs& A, c
 
 }  // namespace
 
-int tangent_record_len(const DevPot& P) { return 2 * (4 + P.S); }  // the longest record
+int tangent_record_len(const DevPot& P, const TanArgs& A, bool theta) {
+  return wants_values(A, theta) ? 2 * (4 + P.S) : 4 * P.S;  // the longer of both passes' records
+}
 
 int tangent_blocks(int64_t npair) {
   int dev = 0, sms = 0;
@@ -571,7 +574,7 @@ int tangent_blocks(int64_t npair) {
 }
 
 cudaError_t launch_tangent_pairs(const DevPot& P, const DevGrid& g, const TanArgs& A, const RadialTab& dens_tab,
-                                 const RadialTab& tab, const int4* pair_rec, int64_t npair, double* rec,
+                                 const RadialTab& tab, const int4* pair_rec, int64_t npair, const TanRec& rec,
                                  double* th_part, double* th_out, cudaStream_t s) {
   if (A.n == 0) return cudaSuccess;
   if (P.S == 1) return tangent_pairs<1, 1>(P, g, A, dens_tab, tab, pair_rec, npair, rec, th_part, th_out, s);

@@ -68,3 +68,31 @@ def test_a_rebuild_without_room_for_its_rows(precision):
     g.free_energy_grad()
     for a, b in zip((g.F4, g.gq, g.gs, g.mu_ex), before):
         assert np.abs((a - b).cpu().numpy()).max() <= 1e-12 * np.abs(b.cpu().numpy()).max()
+
+
+def used():
+    torch.cuda.synchronize()
+    free, total = torch.cuda.mem_get_info()
+    return total - free
+
+
+@pytest.mark.parametrize("case,extra", [("alloy", 4), ("single", 6)])
+def test_memory_of_the_first_tangent(case, extra):
+    """The first forward-mode pass of a context allocates `extra` doubles per list
+    entry (an eighth more for growth), six per site and species, and its rows and
+    sums (8 MB at most, with the allocator's granularity): the rest of its records
+    lies in the geometry records' buffer."""
+    s = W.perturb(W.config_binary_alloy(20) if case == "alloy" else W.config_vacancy_lattice(24), 0.05, 0.02, seed=7)
+    g = M.MxeSystem(s, "fp64")
+    g.build_neighbors()
+    g.free_energy_grad()
+    few = W.config_binary_alloy(4) if case == "alloy" else W.config_vacancy_lattice(5)
+    small = M.MxeSystem(W.perturb(few, 0.05, 0.02, seed=8), "fp64")
+    small.build_neighbors()
+    small.tangent()  # the kernels are loaded
+    held = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
+    del held  # the outputs come from torch's pool
+    before = used()
+    t = g.tangent()
+    assert used() - before <= 1.125 * 8 * extra * g.n_pairs + 48 * s.S * s.n + (8 << 20)
+    assert (t["gq"] - g.gq).abs().max().item() <= 1e-11 * g.gq.abs().max().item()
