@@ -1308,7 +1308,6 @@ mxe_status ensure_tangent(mxe_ctx* c) {
   if (c->tan_buf) return MXE_OK;
   const int64_t n = c->n, S = c->S, T = n_terms(c);
   CK(dalloc(&c->tan_buf, 6 * S * n));
-  CK(dalloc(&c->th_buf, 2 * 2 * T * n));
   CK(dalloc(&c->th_sum, 4 * T));
   CK(dalloc(&c->dot_part, dot_partials_len(4 * n + 1)));
   CK(dalloc(&c->dot_out, 2));
@@ -1347,10 +1346,6 @@ mxe_status enqueue_tangent(mxe_ctx* c, const mxe_state* s, const double* dq, con
   A.gq_t = gq_t;
   A.gs_t = gs_t;
   A.mu_t = mu_t;
-  if (th_out) {
-    A.th_v = c->th_buf;
-    A.th_t = c->th_buf + 2 * T * n;
-  }
   A.flags = c->flags;
   A.batch = c->B;
   A.n_ent = c->n_pairs;
@@ -1360,6 +1355,11 @@ mxe_status enqueue_tangent(mxe_ctx* c, const mxe_state* s, const double* dq, con
                                                    c->n_upairs, rec, c->tan_part, T > 0 ? th_out : nullptr,
                                                    c->stream)));
     return MXE_OK;
+  }
+  if (th_out) {
+    if (!c->th_buf) CK(dalloc(&c->th_buf, 2 * 2 * T * n));
+    A.th_v = c->th_buf;
+    A.th_t = c->th_buf + 2 * T * n;
   }
   CK(TIMED("tangent", launch_tangent(c->dp, c->grid, A, c->stream)));
   if (th_out && T > 0) {
@@ -1520,7 +1520,6 @@ mxe_status mxe_create_batch(mxe_ctx** out, int32_t n_systems, const mxe_box* box
     A(dalloc(&c->n_below, n));
     A(dalloc(&c->pair_cnt, n));
     A(dalloc(&c->pair_off, n + 1));
-    if (precision != MXE_FP64) A(dalloc(&c->pos32lo, n));
     A(dalloc(&c->srec, n * site_record_len(c->dp)));
   }
   A(init_ff_exp_table());
@@ -1580,6 +1579,8 @@ mxe_status mxe_create_batch(mxe_ctx** out, int32_t n_systems, const mxe_box* box
   if (e == cudaSuccess) e = cudaMemsetAsync(c->flags, 0, 2 * sizeof(int), c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->ctrl, 0, sizeof(Ctrl), c->stream);
   if (e == cudaSuccess) e = build_radial_tabs(c);
+  // the direct float-float pass alone reads the positions' remainders
+  if (e == cudaSuccess && has_pair_index(c) && precision != MXE_FP64 && !c->tab_rows) e = dalloc(&c->pos32lo, n);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) {
     mxe_destroy(c);

@@ -80,7 +80,7 @@ def used():
 def test_memory_of_the_first_tangent(case, extra):
     """The first forward-mode pass of a context allocates `extra` doubles per list
     entry (an eighth more for growth), six per site and species, and its rows and
-    sums (8 MB at most, with the allocator's granularity): the rest of its records
+    sums (6 MB at most, with the allocator's granularity): the rest of its records
     lies in the geometry records' buffer."""
     s = W.perturb(W.config_binary_alloy(20) if case == "alloy" else W.config_vacancy_lattice(24), 0.05, 0.02, seed=7)
     g = M.MxeSystem(s, "fp64")
@@ -94,5 +94,5 @@ def test_memory_of_the_first_tangent(case, extra):
     del held  # the outputs come from torch's pool
     before = used()
     t = g.tangent()
-    assert used() - before <= 1.125 * 8 * extra * g.n_pairs + 48 * s.S * s.n + (8 << 20)
+    assert used() - before <= 1.125 * 8 * extra * g.n_pairs + 48 * s.S * s.n + (6 << 20)
     assert (t["gq"] - g.gq).abs().max().item() <= 1e-11 * g.gq.abs().max().item()
