@@ -1166,10 +1166,8 @@ mxe_status ensure_step_graph(mxe_ctx* c, mxe_state* s, StepKey key) {
     c->step_exec = nullptr;
   }
   if (!c->cap_stream) CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
-  if (!c->loop_dev) {
-    CK(dalloc(&c->loop_dev, 3));
-    CK(cudaMallocHost((void**)&c->loop_h, 3 * sizeof(int)));
-  }
+  if (!c->loop_dev) CK(dalloc(&c->loop_dev, 3));
+  if (!c->loop_h) CK(cudaMallocHost((void**)&c->loop_h, 3 * sizeof(int)));
   cudaGraph_t g = nullptr;
   CK(cudaGraphCreate(&g, 0));
   cudaGraphConditionalHandle h;
@@ -1305,13 +1303,12 @@ bool ensure_tangent_pairs(mxe_ctx* c, int record_len, TanRec& R) {
 }
 
 mxe_status ensure_tangent(mxe_ctx* c) {
-  if (c->tan_buf) return MXE_OK;
   const int64_t n = c->n, S = c->S, T = n_terms(c);
-  CK(dalloc(&c->tan_buf, 6 * S * n));
-  CK(dalloc(&c->th_sum, 4 * T));
-  CK(dalloc(&c->dot_part, dot_partials_len(4 * n + 1)));
-  CK(dalloc(&c->dot_out, 2));
-  CK(cudaMallocHost((void**)&c->dot_h, 2 * sizeof(double)));
+  if (!c->tan_buf) CK(dalloc(&c->tan_buf, 6 * S * n));
+  if (!c->th_sum) CK(dalloc(&c->th_sum, 4 * T));
+  if (!c->dot_part) CK(dalloc(&c->dot_part, dot_partials_len(4 * n + 1)));
+  if (!c->dot_out) CK(dalloc(&c->dot_out, 2));
+  if (!c->dot_h) CK(cudaMallocHost((void**)&c->dot_h, 2 * sizeof(double)));
   return MXE_OK;
 }
 
@@ -2334,10 +2331,8 @@ mxe_status mxe_autotune(mxe_ctx* c, const mxe_state* s, int32_t* lanes_out, int3
 mxe_status mxe_set_embedding(mxe_ctx* c, int32_t mode) {
   if (!c || (mode != MXE_EMBED_TAYLOR && mode != MXE_EMBED_EXACT)) return MXE_ERR_ARG;
   Guard gd(c->device);
-  if (mode == MXE_EMBED_EXACT && !c->emb_buf) {
-    CK(dalloc(&c->emb_buf, 9 * (int64_t)c->S * c->n));
-    CK(dalloc(&c->emb_nrule, c->n));
-  }
+  if (mode == MXE_EMBED_EXACT && !c->emb_buf) CK(dalloc(&c->emb_buf, 9 * (int64_t)c->S * c->n));
+  if (mode == MXE_EMBED_EXACT && !c->emb_nrule) CK(dalloc(&c->emb_nrule, c->n));
   if (mode == MXE_EMBED_EXACT) ensure_taylor_rows(c);  // without rows: the direct kernels
   c->embedding = mode;
   c->list_gen += 1;  // a captured staggered step is captured again

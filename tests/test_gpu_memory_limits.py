@@ -96,3 +96,23 @@ def test_memory_of_the_first_tangent(case, extra):
     t = g.tangent()
     assert used() - before <= 1.125 * 8 * extra * g.n_pairs + 48 * s.S * s.n + (6 << 20)
     assert (t["gq"] - g.gq).abs().max().item() <= 1e-11 * g.gq.abs().max().item()
+
+
+@pytest.mark.parametrize("rest_mb", [4, 65])
+def test_arrays_of_a_first_use_that_do_not_fit(rest_mb):
+    """864,000 sites: the exact embedding average takes 62 + 3 MB, the tangents 41 + 0.1 MB."""
+    s = W.perturb(W.config_vacancy_lattice(60), 0.05, 0.02, seed=9)
+    g = M.MxeSystem(s, "fp64")
+    before = evaluate(g)
+    out = g.tangent  # bound before the memory is gone
+    with AllBut(rest_mb << 20):
+        with pytest.raises(M.MxeError) as e:
+            g.set_embedding("exact")
+        assert e.value.status == M.ERR_OOM
+        with pytest.raises((M.MxeError, torch.cuda.OutOfMemoryError)):
+            out()
+    t = out()
+    assert (t["gq"] - before[1]).abs().max().item() <= 1e-11 * before[1].abs().max().item()
+    g.set_embedding("exact")
+    g.free_energy_grad()
+    assert torch.isfinite(g.gq).all().item()
