@@ -1104,11 +1104,13 @@ cudaError_t launch_row_compact(const uint32_t* rows, const int* brows, int strid
 
 int64_t scan_tmp_len(int64_t n) { return 3 * ((n + kScanBlock) / kScanBlock + 2); }
 
-// Up to 16,384 counts (sixteen chunks of a block, about 1 us each) take the
-// one-launch form: three launches cost about 7 us whatever the length.
+// Up to 11 chunks of a block take the one-launch form: 4.2 us for one chunk, 6.2
+// for four, 10.3 for ten, 12.3 for twelve (12,288 counts), 14.4 for sixteen; three
+// launches take 12.3 us at all these lengths, for one scan as for three.
+constexpr int kScanShortChunks = 11;
 cudaError_t launch_scan(const ScanJobs& J, int count, int64_t n, long long* tmp, int64_t tmp_len, cudaStream_t s) {
   if (count < 1 || count > 3) return cudaErrorInvalidValue;
-  if (n <= 16 * kScanSmall) {
+  if (n <= kScanShortChunks * kScanSmall) {
     k_scan_short<<<count, kScanSmall, 0, s>>>(J, n);
     return cudaGetLastError();
   }
