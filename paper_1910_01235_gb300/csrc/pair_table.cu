@@ -37,7 +37,7 @@
 namespace mxe {
 namespace {
 
-// squared node distances in units of 2^-56: the static point, the common part
+// squared node distances in units of 2^-55: the static point, the common part
 // of each site's nodes and the shifts 2 s |d_a|
 struct PairNodes {
   long long w0, base[2], tw[2][3];

@@ -23,10 +23,13 @@
 // that holds a breakpoint has two rows, one per side, and the row index steps
 // by one at each breakpoint; from r_cut on every w takes one row of zeros.
 //
-// w is a 64-bit integer in units of 2^-56 (w < 128): node distances are integer
+// w is a 64-bit integer in units of 2^-55 (w < 256): node distances are integer
 // additions, the interval is a shift, and tau is the remaining bits.  Pairs
 // with a node below the first row (float-float: 0.5 A; else r_cut / 4 or 1.25 A),
-// with |d|^2 >= 64 or with a non-finite coordinate take the direct evaluation.
+// with |d|^2 >= 128 or with a non-finite coordinate take the direct evaluation.
+// (Units of 2^-56 sent pairs from 8 A on there, in lists of the longest cut-offs a
+// quarter of all: 32,000 sites, r_cut 7.6 A, float-float free-energy call 1.8 ms
+// with the direct kernels, 5.0 ms, now 1.5; FP64 15.8, 11.3, now 2.1.)
 #pragma once
 
 #include "mxe_internal.cuh"
@@ -42,7 +45,7 @@ namespace mxe {
 // c4, c5 (tab_polyff): two words.
 // All FP64 (degree 9, c0..c9; the tangent passes): five words.
 constexpr int kTabWords64 = 3, kTabWordsFF = 2, kTabWordsTaylor = 5;
-constexpr int kTabFixedBits = 56;   // w in units of 2^-56
+constexpr int kTabFixedBits = 55;   // w in units of 2^-55
 constexpr int kTabExpBias = 128 + 61;    // of the derivative rows' exponents
 constexpr int kTabValueBias = 128 + 62;  // of the value rows' exponents
 constexpr double kTabRLow = 0.25, kTabRMin = 1.25;  // first row at r_cut / 4, not below 1.25 A
@@ -76,13 +79,13 @@ __device__ __forceinline__ void tab_stage(const RadialTab& Tb, uint4* __restrict
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
-// x >= 0 in units of 2^-56, truncated; `big` collects x >= 64, infinities and NaN
+// x >= 0 in units of 2^-55, truncated; `big` collects x >= 128, infinities and NaN
 __device__ __forceinline__ long long tab_fixed(double x, int& big) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int e = (int)(b >> 52);  // biased exponent (x >= 0)
-  big |= e >= 1023 + 6;
+  big |= e >= 1023 + 7;  // two of them add up to less than 2^63
   const unsigned long long m = (b << 11) | 0x8000000000000000ull;
-  const int sh = 1023 + 7 - e;
+  const int sh = 1023 + 63 - kTabFixedBits - e;
   return (long long)(sh > 63 ? 0ull : m >> (sh < 1 ? 1 : sh));
 }
 
@@ -102,9 +105,10 @@ __device__ __forceinline__ const uint4* tab_row(const RadialTab& Tb, const uint4
       first = Tb.first_near;
     }
     if (LOWS && hi < Tb.main_hi) {
-      const int o = min(max(31 - __clz((int)hi), 21), 24);  // 22: w in [1/4, 1/2)
+      constexpr int kOne = kTabFixedBits - 32;  // the bit of w = 1
+      const int o = min(max(31 - __clz((int)hi), kOne - 3), kOne);  // kOne - 2: w in [1/4, 1/2)
       sh = o - 6;
-      first = 64 * (o - 23);
+      first = 64 * (o - kOne + 1);
     }
   }
   int k = (int)(hi >> sh) + first;
