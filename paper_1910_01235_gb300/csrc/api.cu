@@ -592,7 +592,7 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
   // largest stencil candidate set: the cell-staged kernels hold it in shared
   // memory.  A rebuild that can skip the count pass (the previous build's
   // longest row bounds this one's) sizes it from the previous build's largest
-  // stencil plus a fifth and checks the true size, computed on the device
+  // stencil plus a margin and checks the true size, computed on the device
   // meanwhile, together with the totals: a larger stencil discards that fill
   // (count + fill instead).  Otherwise the host waits for the size here.
   CK(TIMED("build_misc", launch_cand_max(ncell, g, B, c->cell_start, c->max_row + 1, st)));
@@ -601,9 +601,25 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
   const bool per_site = std::getenv("MXE_NEIGHBOR_PER_SITE") != nullptr;
   const bool try_direct = c->max_row_h > 0 && c->max_row_h + 16 <= 256 && c->cand_cap_prev > 0 && !per_site &&
                           !std::getenv("MXE_NEIGHBOR_COUNT");
-  int cand_cap;
+  int cand_cap, stride = 0;
   if (try_direct) {
-    cand_cap = c->cand_cap_prev + c->cand_cap_prev / 5 + 8;
+    // A fifth of the candidates and, since a growing r_list takes in whole shells of
+    // a lattice (24 of 54 neighbours at once in FCC), half a row, at least 32.  Where
+    // that costs a resident block of the fill, or exceeds its shared memory, an
+    // eighth and 16 (builds of 32,000 sites, r_cut 6.8 A: 729 us wide, three blocks an
+    // SM, 599 lean, four; 16,384 sites: 575 us, counted and filled since the wide
+    // margin did not fit, 400 lean).
+    const int prev = c->cand_cap_prev, row = c->max_row_h;
+    const int cand_lean = prev + prev / 8 + 8, stride_lean = (row + 16 + 3) & ~3;
+    auto resident = [](int cand, int rows) {
+      return std::min<size_t>(8, 228 * 1024 / (cell_stage_bytes(cand, rows, true) + 1024));
+    };
+    cand_cap = prev + prev / 5 + 8;
+    stride = std::min((row + std::max(32, row / 2) + 3) & ~3, 256);
+    if (cell_stage_bytes(cand_cap, 256, true) > 64 * 1024 || resident(cand_cap, stride) < resident(cand_lean, stride_lean)) {
+      cand_cap = cand_lean;
+      stride = stride_lean;
+    }
   } else {
     CK(cudaMemcpyAsync(c->ints_h + 2, c->max_row + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -617,12 +633,8 @@ mxe_status build_lists(mxe_ctx* c, const mxe_state* s, double skin, double r_bon
                            {c->nb_off, c->bd_off, c->pair_off},
                            {c->totals + 1, c->totals + 2, c->totals + 3}};
   bool direct = false;
-  int stride = 0;
   bool rows_fit = true;  // else count + fill, which needs no rows at a stride
   if (staged && try_direct) {
-    // a growing r_list takes in whole shells of a lattice (24 of 54 neighbours
-    // at once in FCC): half a row more, at least 32
-    stride = std::min((c->max_row_h + std::max(32, c->max_row_h / 2) + 3) & ~3, 256);
     if ((int64_t)n * stride > c->rows_cap) {
       dfree(c->rows_tmp);
       dfree(c->brows_tmp);
