@@ -881,6 +881,10 @@ __global__ void k_site_max(const double* __restrict__ sigma, const double* __res
   block_max_bits(out, vs, vq);
 }
 
+// The attribute of a kernel holds for the process: set to the size of one launch,
+// it made the larger launch of another thread's context fail in between.
+constexpr int kSmemLimit = 208 * 1024;
+
 inline unsigned grid_for(int64_t work, int threads) { return (unsigned)((work + threads - 1) / threads); }
 
 // segment of each index by binary search over the segment starts (empty
@@ -1011,7 +1015,7 @@ cudaError_t launch_nbr_fill(const double* q, const float4* qf, const uint8_t* su
   if (warps > 8) warps = 8;
   if (warps < 1) return cudaErrorInvalidValue;
   size_t shm = per_warp * warps + 16;
-  cudaError_t e = cudaFuncSetAttribute(k_nbr_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+  cudaError_t e = cudaFuncSetAttribute(k_nbr_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
   if (e != cudaSuccess) return e;
   int threads = warps * 32;
   k_nbr_fill<<<grid_for(n * 32, threads), threads, shm, s>>>(q, qf, sub, mobile_mask, n, g, B, cell_of, cell_start,
@@ -1044,7 +1048,7 @@ cudaError_t launch_cell_count(const double* q, const float4* qf, const uint8_t* 
                               int* max_row, int* flags, cudaStream_t s) {
   if (n == 0 || ncell == 0) return cudaSuccess;
   const size_t shm = cell_stage_bytes(cand_cap, 0, false);
-  cudaError_t e = cudaFuncSetAttribute(k_cell_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+  cudaError_t e = cudaFuncSetAttribute(k_cell_count, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
   if (e != cudaSuccess) return e;
   k_cell_count<<<(unsigned)ncell, few_cells(ncell) ? kCellThreadsFew : kCellThreads, shm, s>>>(q, qf, sub, mobile_mask, n, g, B, cell_start, cell_sites, rl2,
                                                           rb2, band, cand_cap, nb_cnt, bd_cnt, max_row, flags);
@@ -1060,7 +1064,7 @@ cudaError_t launch_cell_fill(const double* q, const float4* qf, const uint8_t* s
   if (max_row < 1) max_row = 1;
   auto run = [&](auto kernel, int threads) {
     const size_t shm = stage_bytes(threads, cand_cap, max_row, true);
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
     kernel<<<(unsigned)ncell, threads, shm, s>>>(q, qf, sub, mobile_mask, n, g, B, cell_start,
                                                                 cell_sites, abs_cell, rl2, rb2, band, cand_cap, nb_off,
@@ -1081,7 +1085,7 @@ cudaError_t launch_cell_fill_direct(const double* q, const float4* qf, const uin
   if (n == 0 || ncell == 0) return cudaSuccess;
   auto run = [&](auto kernel, int threads) {
     const size_t shm = stage_bytes(threads, cand_cap, stride, true);
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
     kernel<<<(unsigned)ncell, threads, shm, s>>>(q, qf, sub, mobile_mask, n, g, B, cell_start,
                                                                cell_sites, abs_cell, rl2, rb2, band, cand_cap, nullptr,
