@@ -51,7 +51,7 @@ from paper_1910_01235_gb300 import workloads as W  # noqa: E402
 METRIC = "site free-energy+gradient evals/s and diffusion steps/s, FP32-mixed vs FP64"
 WORKLOAD = "binary_alloy_fcc40_256k"
 FIRE_ITERS = 10
-DTYPES = {"fp64": "f64", "mixed": "f32 (f64 sums; mu from float-float node arithmetic)",
+DTYPES = {"fp64": "f64", "mixed": "f32 (three-float sums; mu from float-float node arithmetic)",
           "ff": "f32 (float-float sums and mu)"}
 
 

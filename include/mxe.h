@@ -59,7 +59,9 @@ typedef enum {
 } mxe_status;
 
 typedef enum {
-    MXE_FP64 = 0,        /* every step in FP64 */
+    MXE_FP64 = 0,        /* results to FP64 rounding: FP64 state, sums and control; radial
+                            terms of tabulated potentials from integers of 54 or 55 bits
+                            and float-float and FP32 remainders, else in FP64 */
     MXE_FP32_MIXED = 1,  /* node arithmetic (distance, switch, exp, derivatives) in FP32;
                             each pair's 13-node partial sums added into per-site sums of
                             at least FP64 precision (FP64, or three floats rounded to FP64 once);

@@ -9,22 +9,22 @@
 // 16-byte loads per term) and 20 to 36 FP32 operations per term.
 //
 // Measured (event time per launch, direct -> tabulated).  FP64, 19,652-site
-// binary alloy (531 k pairs): forces 1127 -> 161 us, densities 709 -> 72 us,
-// geometry 911 -> 149 us.  Float-float geometry: 6.9 M pairs of the binary
-// alloy (which had the power form) 1.35 -> 1.22 ms, 23.3 M pairs of one species
-// 3.54 -> 1.92 ms, 241 M pairs of the interstitial slab 52.6 -> 26.6 ms.  What
+// binary alloy (531 k pairs): forces 1127 -> 160 us, densities 709 -> 71 us,
+// geometry 911 -> 140 us.  Float-float geometry: 6.9 M pairs of the binary
+// alloy (which had the power form) 1.35 -> 0.92 ms, 23.3 M pairs of one species
+// 3.54 -> 1.77 ms, 241 M pairs of the interstitial slab 52.6 -> 26.5 ms.  What
 // bounds them now (ncu): the geometry kernels the shared-memory wavefronts
-// (84-89 %; 32 lanes reading random rows take about 12 wavefronts per 16-byte
-// load, 4 without bank conflicts), the force kernel those (64 %), instruction
-// issue (53 %) and the FP64 pipe (40 %) together, the density kernel the
-// wavefronts and the FP64 pipe (65 % each).  With the constant terms and the
+// (86 % float-float, 93 % FP64; 32 lanes reading random rows take about 12
+// wavefronts per 16-byte load, 4 without bank conflicts), the force kernel those
+// (82 %), instruction issue (65 %) and the FP64 pipe (48 %) together, the density
+// kernel the wavefronts (86 %) and the FP64 pipe (64 %).  With the constant terms and the
 // sums of the nodes in FP64 (207 FP64 instructions a pair and lane) the force
 // kernel took 210 us, the FP64 pipe 84 % busy; with the direct evaluation
 // called inside the table loop 9 us more; with 640 threads a block (96
 // registers) 171 us, with 384 (160 registers) as with 512.
 //
 // Layout: one block per SM holds the whole table in shared memory (up to
-// 200 KB) and strides over the pairs; the table is copied before the kernel
+// 224 KB) and strides over the pairs; the table is copied before the kernel
 // waits for the previous one.
 #include <cuda_runtime.h>
 
